@@ -154,7 +154,7 @@ int nl_of(int model) { return model == PORTA_MODEL_TWOLEVEL_UNPOL ? 1 : 6; }
 // (and the biquadratic stencils, which only the general sweep has)
 bool use_jk(const porta_ctx *c)
 {
-    return c->d_dich == nullptr && c->d_kexpl == nullptr && c->jk_fits && c->interp != 2 && !c->sc_faces && !c->gsweep;
+    return c->d_dich == nullptr && c->d_kexpl == nullptr && c->jk_form != 0 && c->interp != 2 && !c->sc_faces && !c->gsweep;
 }
 
 // The J^K_Q sweep sums an FP32 formal solution into fixed-point accumulators;
@@ -162,6 +162,7 @@ bool use_jk(const porta_ctx *c)
 // fixed-point scale cannot hold 1e-10 relative precision for quantities that
 // span many decades within one voxel, as Lambda-bar* does with optical depth).
 bool jfixed(const porta_ctx *c) { return use_jk(c) && c->precision == PORTA_FP32; }
+int jparts(const porta_ctx *c, int ngroups) { return jfixed(c) && c->jk_form == 1 ? ngroups : 1; }
 
 // frequencies of the J^K_Q formal solution (its band, porta_set_freq_range)
 int jnu(const porta_ctx *c) { return c->fr1 > c->fr0 ? c->fr1 - c->fr0 : c->n_nu; }
@@ -190,11 +191,13 @@ std::vector<LaunchCfg> candidates(porta_ctx *c, int nitems)
     const int ny_max = max_ny(c);
     for (int C = 1; C <= 16; ++C) {
         if (C > ny_max) continue;
-        int last_f = -1, kept = 0;
+        int last_units = -1, kept = 0;
         for (int G = 1; G <= jnu(c) && kept < 3; ++G) {
-            int F = (jnu(c) + G - 1) / G;
-            if (F == last_f) continue;
-            last_f = F;
+            const int F = (jnu(c) + G - 1) / G;
+            // (a J^K_Q sweep takes frequencies in units of lanes)
+            const int units = use_jk(c) && c->jk_form == 1 ? (F + jsweep_lanes<Real>() - 1) / jsweep_lanes<Real>() : F;
+            if (units == last_units) continue;
+            last_units = units;
             LaunchCfg cfg{};
             if (choose_launch<Real, NS>(c, cfg, C, F, nitems, use_jk(c), jnu(c)) == PORTA_OK && cfg.F == F) {
                 out.push_back(cfg);
@@ -209,6 +212,8 @@ std::vector<LaunchCfg> candidates(porta_ctx *c, int nitems)
 template <typename Real>
 cudaError_t launch_j(porta_ctx *c, const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st)
 {
+    if (use_jk(c) && c->jk_form == 2)
+        return c->ns == 1 ? launch_jwide<Real, 1>(a, cfg, st) : launch_jwide<Real, 4>(a, cfg, st);
     if (use_jk(c))
         return c->ns == 1 ? launch_jsweep<Real, 1>(a, cfg, st) : launch_jsweep<Real, 4>(a, cfg, st);
     return c->ns == 1 ? launch_sweep<Real, 1>(a, MODE_JKQ, cfg, st) : launch_sweep<Real, 4>(a, MODE_JKQ, cfg, st);
@@ -226,12 +231,15 @@ SweepArgs<Real> jkq_args(porta_ctx *c)
         a.nnu = c->fr1 - c->fr0;
     }
     a.geom = (const PlaneGeom<Real> *)c->d_geom;
+    if (use_jk(c) && c->jk_form == 1)      // the second half: in the form of sweep_j.cu
+        for (const BoxDev &b : c->boxes) a.geom += (size_t)c->nray * b.nz;
     a.rays = (const RayDev<Real> *)c->d_rays;
     a.invn = (const Real *)c->d_invn;
     a.part = jfixed(c) ? nullptr : c->d_part;
     a.partv = (Real *)c->d_partv;
     a.jacc = jfixed(c) ? c->d_jacc : nullptr;
     a.jexp = c->d_jexp;
+    a.pack = (const Real *)c->d_jpack;
     a.jerr = c->d_err;
     a.tw = c->d_tw;
     a.items = c->d_items;
@@ -287,13 +295,15 @@ void check_global_sweep(porta_ctx *c)
 cudaError_t ensure_sweep_buffers(porta_ctx *c)
 {
     check_global_sweep(c);
+    cudaError_t e = cudaSuccess;
+    if (use_jk(c) && c->jk_form == 1 && !c->d_jpack)
+        e = pmalloc(&c->d_jpack, (size_t)(c->ns == 1 ? jpack_words<1>() : jpack_words<4>()) * c->nvox * c->rsz);
+    if (e != cudaSuccess) return e;
     if (jfixed(c)) {
-        cudaError_t e = cudaSuccess;
         if (!c->d_jacc) e = pmalloc(&c->d_jacc, (size_t)(c->nj + 1) * c->nvox * sizeof(unsigned long long));
         if (e == cudaSuccess && !c->d_jexp) e = pmalloc(&c->d_jexp, (size_t)c->nvox * sizeof(int));
         return e;
     }
-    cudaError_t e = cudaSuccess;
     if (!c->d_part) e = pmalloc(&c->d_part, (size_t)c->nray * c->nvox * (c->ns == 1 ? 2 : 4) * c->rsz);
     // polarized lines of a multilevel atom: the per-ray integrals of Stokes V (J^1_Q)
     if (e == cudaSuccess && c->d_dich && !c->d_partv) e = pmalloc(&c->d_partv, (size_t)c->nray * c->nvox * c->rsz);
@@ -326,7 +336,7 @@ cudaError_t ensure_sweep_buffers(porta_ctx *c)
 template <typename Real>
 cudaError_t jacc_prepare(porta_ctx *c, const SweepArgs<Real> &a)
 {
-    if (!jfixed(c)) return cudaSuccess;
+    if (!use_jk(c) || (c->jk_form == 2 && !jfixed(c))) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
     return c->ns == 1 ? launch_jacc_prepare<Real, 1>(a, c->stream) : launch_jacc_prepare<Real, 4>(a, c->stream);
@@ -355,11 +365,12 @@ cudaError_t finalize_jkq(porta_ctx *c)
 // the fixed-point sums' overflow flag (reads device memory: synchronizes the stream)
 int check_jacc(porta_ctx *c)
 {
-    if (!jfixed(c) && !c->sc_faces && !c->gsweep && !c->d_kexpl) return PORTA_OK;
+    if ((!use_jk(c) || (c->jk_form == 2 && !jfixed(c))) && !c->sc_faces && !c->gsweep && !c->d_kexpl) return PORTA_OK;
     int flag = 0;
     CK(cudaMemcpyAsync(&flag, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     if (flag & 2) return fail(c, PORTA_ENOTCONV, "formal solution: a plane of face points did not converge");
+    if (flag & 4) return fail(c, PORTA_EKERNEL, "formal solution: a strip's wait for its neighbour ran out");
     if (flag) return fail(c, PORTA_EKERNEL, "formal solution: a J^K_Q term exceeded the fixed-point range (2^16 times "
                                             "max(|S^0_0|, |B|) of its voxel), or was not finite");
     return PORTA_OK;
@@ -399,10 +410,10 @@ cudaError_t sweep_jkq(porta_ctx *c, SweepArgs<Real> a, LaunchCfg cfg, const int 
     b.items = items + nA;
     b.nitems = nB;
     b.next_item = c->fill->d_ctr + 1;
-    fc.clusters = std::min(fc.clusters, nB);
+    fc.clusters = std::min(fc.clusters, nB * jparts(c, b.ngroups));
     a.nitems = nA;
     a.next_item = c->fill->d_ctr;
-    cfg.clusters = std::min(cfg.clusters, nA);
+    cfg.clusters = std::min(cfg.clusters, nA * jparts(c, a.ngroups));
     // the main launch's clusters are placed first; the filler takes what is left
     int least = 0, greatest = 0;
     e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
@@ -475,6 +486,7 @@ int formal_solve_t(porta_ctx *c, int probe_ray, Real *probe, Real *probe_ls)
     a.partv = (Real *)c->d_partv;
     a.jacc = jfixed(c) ? c->d_jacc : nullptr;
     a.jexp = c->d_jexp;
+    a.pack = (const Real *)c->d_jpack;
     e = jacc_prepare<Real>(c, a);
     if (e == cudaSuccess) e = sweep_jkq<Real>(c, a, cfg, a.items, a.nitems, probe_ray < 0);
     if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
@@ -510,7 +522,7 @@ int autotune_t(porta_ctx *c)
         // one box: time one wave (every resident cluster sweeps one ray);
         // batches: time a strided sample of the (box, ray) items
         if (c->nbox == 1) {
-            a.nitems = cfg.clusters;
+            a.nitems = std::min(cfg.clusters, c->nray);
         } else {
             a.items = c->d_tune_items;
             a.nitems = c->n_tune;
@@ -527,8 +539,9 @@ int autotune_t(porta_ctx *c)
             ms = std::min(ms, t);
         }
         if (rc != PORTA_OK) break;
-        double waves = c->nbox == 1 ? std::ceil((double)c->nray / cfg.clusters)
-                                    : (double)c->nbox * c->nray / c->n_tune;
+        const double parts = jparts(c, a.ngroups);        // work items per ray
+        auto rounds = [&](int rays) { return std::ceil(rays * parts / cfg.clusters); };
+        double waves = c->nbox == 1 ? rounds(c->nray) / rounds(a.nitems) : (double)c->nbox * c->nray / c->n_tune;
         double est = ms * waves;
         est_of[ci] = est;
         if (est < best) {
@@ -586,9 +599,12 @@ int autotune_t(porta_ctx *c)
         // of its resident clusters (rays cost the same); batches -> fractions
         std::vector<double> fracs;
         if (c->nbox == 1) {
-            const int rounds = (tn + pick.clusters - 1) / pick.clusters;
-            for (int r = rounds - 1; r >= std::max(1, rounds - 6); --r) {
-                const int nB = tn - r * pick.clusters;
+            SweepArgs<Real> a = jkq_args<Real>(c);
+            shape_args<Real>(c, a, pick, use_jk(c));
+            const int parts = jparts(c, a.ngroups);
+            const int rounds = (tn * parts + pick.clusters - 1) / pick.clusters;
+            for (int r = rounds - 1; r >= std::max(1, rounds - 6 * parts); r -= parts) {
+                const int nB = tn - r * pick.clusters / parts;
                 if (nB > 0 && nB < tn) fracs.push_back((double)nB / tn);
             }
         } else {
@@ -654,7 +670,7 @@ void free_all(porta_ctx *c)
         if (ev) cudaEventDestroy(ev);
     void *ptrs[] = {c->d_atm, c->d_eps, c->d_bpl, c->d_b, c->d_rho, c->d_rhoR, c->d_invn, c->d_geom, c->d_rays,
                     c->d_freq, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->d_resid, c->d_err, c->d_boxes,
-                    c->d_items, c->d_tune_items, c->d_tape, c->d_gpart, c->d_jacc, c->d_jexp, c->d_kexpl, c->d_sexpl,
+                    c->d_items, c->d_tune_items, c->d_tape, c->d_gpart, c->d_jacc, c->d_jexp, c->d_jpack, c->d_kexpl, c->d_sexpl,
                     c->d_partv, c->d_j1, c->d_tw1, c->d_gjR, c->d_vjp_out, c->d_faces, c->d_fdxy};
     for (void *p : ptrs)
         if (p) pfree(p);
@@ -809,7 +825,7 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
     ok(dalloc(&c->d_rho, nvox * c->nl));
     ok(pmalloc(&c->d_rhoR, nvox * c->nl * R));
     ok(pmalloc(&c->d_invn, (size_t)c->nray * nvox * R));
-    ok(pmalloc(&c->d_geom, (size_t)c->nray * nplane * (prec == PORTA_FP32 ? sizeof(PlaneGeom<float>) : sizeof(PlaneGeom<double>))));
+    ok(pmalloc(&c->d_geom, 2 * (size_t)c->nray * nplane * (prec == PORTA_FP32 ? sizeof(PlaneGeom<float>) : sizeof(PlaneGeom<double>))));
     ok(pmalloc(&c->d_boxes, (size_t)nbox * sizeof(BoxDev)));
     ok(dalloc(&c->d_items, (size_t)nbox * c->nray));
     c->n_tune = (int)std::min<long long>((long long)nbox * c->nray, 256);
@@ -847,7 +863,7 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
         for (int i = 0; i < c->n_tune; ++i) tune[i] = items[(size_t)i * items.size() / c->n_tune];
         ok(cudaMemcpy(c->d_tune_items, tune.data(), tune.size() * sizeof(int), cudaMemcpyHostToDevice));
         if (prec == PORTA_FP32) {
-            std::vector<PlaneGeom<float>> geom((size_t)c->nray * nplane);
+            std::vector<PlaneGeom<float>> geom(2 * (size_t)c->nray * nplane);
             std::vector<RayDev<float>> rays(c->nray);
             std::vector<float> fr(2 * c->n_nu);
             for (int b = 0; b < nbox; ++b)
@@ -855,13 +871,14 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
                     plane_geometry<float>(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
                                           c->bz[b].data(), c->mu[m], c->chi[m],
                                           geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz);
+            for (size_t i = 0; i < geom.size() / 2; ++i) geom[geom.size() / 2 + i] = relative_geometry(geom[i]);
             for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<float>(c->mu[m], c->chi[m], c->w[m]);
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = (float)c->xf[j]; fr[c->n_nu + j] = (float)c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));
             ok(cudaMemcpy(c->d_rays, rays.data(), rays.size() * sizeof(rays[0]), cudaMemcpyHostToDevice));
             ok(cudaMemcpy(c->d_freq, fr.data(), fr.size() * sizeof(float), cudaMemcpyHostToDevice));
         } else {
-            std::vector<PlaneGeom<double>> geom((size_t)c->nray * nplane);
+            std::vector<PlaneGeom<double>> geom(2 * (size_t)c->nray * nplane);
             std::vector<RayDev<double>> rays(c->nray);
             std::vector<double> fr(2 * c->n_nu);
             for (int b = 0; b < nbox; ++b)
@@ -869,6 +886,7 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
                     plane_geometry<double>(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
                                            c->bz[b].data(), c->mu[m], c->chi[m],
                                            geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz);
+            for (size_t i = 0; i < geom.size() / 2; ++i) geom[geom.size() / 2 + i] = relative_geometry(geom[i]);
             for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<double>(c->mu[m], c->chi[m], c->w[m]);
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = c->xf[j]; fr[c->n_nu + j] = c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));
@@ -877,15 +895,16 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
         }
         // a launch shape must exist for this grid
         LaunchCfg cfg{};
-        int r2 = PORTA_OK;
-        for (int jk = 1; jk >= 0; --jk) {
-            r2 = prec == PORTA_FP32
-                     ? (c->ns == 1 ? choose_launch<float, 1>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk)
-                                   : choose_launch<float, 4>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk))
-                     : (c->ns == 1 ? choose_launch<double, 1>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk)
-                                   : choose_launch<double, 4>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk));
-            if (jk) c->jk_fits = r2 == PORTA_OK;
-        }
+        auto fits = [&](bool jk) {
+            return prec == PORTA_FP32
+                       ? (c->ns == 1 ? choose_launch<float, 1>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk)
+                                     : choose_launch<float, 4>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk))
+                       : (c->ns == 1 ? choose_launch<double, 1>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk)
+                                     : choose_launch<double, 4>(c, cfg, c->opt_cluster, c->opt_nu_group, c->nray, jk));
+        };
+        for (c->jk_form = 1; c->jk_form <= 2 && fits(true) != PORTA_OK;) ++c->jk_form;
+        if (c->jk_form > 2) c->jk_form = 0;
+        const int r2 = fits(false);
         if (rc == PORTA_OK && r2 != PORTA_OK) {
             if (c->opt_cluster > 0 || c->opt_nu_group > 0) {
                 rc = PORTA_EINVAL;

@@ -109,6 +109,22 @@ void plane_geometry(int nx, int ny, int nz, double lx, double ly, const double *
     }
 }
 
+// the same for the J^K_Q sweep, which uses the bilinear weights relative to the first one:
+// in place of (tx, ty, ds, pad2) it reads u = t / (1 - t) along x and y, the first weight
+// (1 - tx) (1 - ty), and ds / 2. A factor 1 - t that rounds to 0 is held at the rounding unit of 1.
+template <typename Real>
+PlaneGeom<Real> relative_geometry(const PlaneGeom<Real> &p)
+{
+    const double unit = sizeof(Real) == 4 ? 5.9604644775390625e-08 : 1.1102230246251565e-16;
+    const double mx = std::max(1.0 - (double)p.tx, unit), my = std::max(1.0 - (double)p.ty, unit);
+    PlaneGeom<Real> r = p;
+    r.tx = (Real)(p.tx / mx);
+    r.ty = (Real)(p.ty / my);
+    r.ds = (Real)(mx * my);
+    r.pad2 = (Real)(0.5 * p.ds);
+    return r;
+}
+
 template <typename Real>
 RayDev<Real> ray_dev(double mu, double chi, double w = 0.0)
 {
@@ -127,6 +143,7 @@ RayDev<Real> ray_dev(double mu, double chi, double w = 0.0)
 
 const int kThreads = 512;   // maximum threads per CTA of the sweep kernel
 const int kSmemLimit = 220 * 1024;
+const int kJSmemLimit = 226 * 1024;   // J^K_Q sweep (its static shared memory stays below 1 KB)
 
 // Shared-memory capacities of a launch with cluster size C over all boxes:
 // ring plane (16-byte chunks) and Stokes-plane points, each the maximum over boxes.
@@ -141,9 +158,9 @@ void launch_caps(const porta_ctx *c, int C, int &ring_plane, int &ipts_max, bool
         const int rmax = (b.ny + C - 1) / C;
         const int chunk = (rmax + 2) * b.nx;
         if (jk) {
-            // the J^K_Q sweep (sweep_j.cu): ring capacity in nodes
+            // the J^K_Q sweep (sweep_j.cu): ring capacity in nodes, Stokes planes
             ring_plane = std::max(ring_plane, chunk);
-            ipts_max = std::max(ipts_max, rmax * b.nx);
+            ipts_max = std::max(ipts_max, (rmax + (c->jk_form == 1 ? 1 : 0)) * b.nx);   // (sweep_j.cu: with the halo row)
             continue;
         }
         // with dichroism the slots of a second ring follow the node ring (eta_U / eta_I and the
@@ -160,7 +177,8 @@ void launch_caps(const porta_ctx *c, int C, int &ring_plane, int &ipts_max, bool
 // The J^K_Q formal solution runs the kernel of sweep_j.cu (per-frequency
 // node coefficients in shared memory) unless the lines carry dichroism, which
 // only the general sweep (sweep.cu) implements, or a plane is too wide for its
-// shared memory (then the general sweep, which needs less per frequency, runs).
+// shared memory: then that of sweep_jw.cu, which needs less per node, or the general
+// sweep, which needs less per frequency. jk_form says which of the two kernels.
 bool use_jk(const porta_ctx *c);
 
 // The J^K_Q sweep sums an FP32 formal solution into fixed-point accumulators;
@@ -168,6 +186,8 @@ bool use_jk(const porta_ctx *c);
 // fixed-point scale cannot hold 1e-10 relative precision for quantities that
 // span many decades within one voxel, as Lambda-bar* does with optical depth).
 bool jfixed(const porta_ctx *c);
+// work items of a ray: sweep_j.cu deals out the passes of an FP32 ray separately
+int jparts(const porta_ctx *c, int ngroups);
 
 // frequencies of the J^K_Q formal solution (its band, porta_set_freq_range)
 int jnu(const porta_ctx *c);
@@ -176,17 +196,119 @@ int jnu(const porta_ctx *c);
 int max_ny(const porta_ctx *c);
 int min_ny(const porta_ctx *c);
 
-// Launch shape of the sweep: cluster size C (CTAs sharing one ray's plane)
+// threads of a J^K_Q sweep CTA (those of the box that needs most) and the entries of its
+// totals buffer: as many where some box's strips take several groups of threads, else 0
+template <typename Real, int NS>
+int jsweep_tots(const porta_ctx *c, int C, int F, int *threads_out)
+{
+    const int FX = (F + jsweep_lanes<Real>() - 1) / jsweep_lanes<Real>();
+    int threads = 64;
+    for (const BoxDev &b : c->boxes)
+        threads = std::max(threads, jsweep_threads(b.nx, (b.ny + C - 1) / C, FX, jsweep_max_threads<Real, NS>()));
+    if (threads_out) *threads_out = threads;
+    for (const BoxDev &b : c->boxes)
+        // (a strip of the box may have one row less than the largest)
+        if (FX > 1 && threads / ((std::max(1, b.ny / C) * b.nx + 31) / 32 * 32) > 1) return threads;
+    return 0;
+}
+
+// Cycles of one plane of one pass of the J^K_Q sweep in a CTA: a chain of fixed length
+// (barrier, geometry, sources of the corners, sums), the units of the points' rounds one
+// after the other, and a round of the nodes' filling, whose length grows little with the
+// frequencies; in FP64 the operations of all points besides, at 1/64 of the FP32 rate.
+// Fitted to forced shapes of boxes from 8 x 8 x 16 to 64 x 64 x 64 (C 1 to 16, every number of
+// passes): the shape it picks was the fastest of all, or within 12% of it, for each.
+template <typename Real, int NS>
+double jsweep_plane_cost(int nx, int R, int F, int threads)
+{
+    const int W = jsweep_lanes<Real>(), FX = (F + W - 1) / W;
+    const int pts = R * nx, nodes = (R + 2) * nx;
+    const int pw = std::min(threads, (pts + 31) / 32 * 32), Lg = std::min(FX, threads / pw);
+    const double units = (double)((pts + pw - 1) / pw) * ((FX + Lg - 1) / Lg);
+    const double fills = (nodes + threads - 1) / threads;
+    if (sizeof(Real) == 4)
+        return NS == 4 ? 2660.0 + 1106.0 * units + fills * (1190.0 + 151.0 * FX)
+                       : 3180.0 + 778.0 * units + fills * (339.0 + 6.0 * FX);
+    const double warps = (double)((pts + 31) / 32) * FX, nwarps = (double)((nodes + 31) / 32) * FX;
+    return NS == 4 ? 5610.0 + 5520.0 * units + fills * (2790.0 + 1200.0 * FX) + 1630.0 * warps + 611.0 * nwarps
+                   : 3550.0 + 17166.0 * units + fills * 550.0 * FX + 600.0 * nwarps;
+}
+
+// Launch shape of the J^K_Q sweep: every cluster size, every number of passes whose
+// frequencies fit in shared memory; the (box, ray) items, in FP32 the passes of a ray each,
+// spread over the resident clusters.
+template <typename Real, int NS>
+int choose_jsweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, int NU)
+{
+    double best_cost = 1e300;
+    best = LaunchCfg{};
+    const int ny_max = max_ny(c);
+    auto even = [&](int g) { return (NU + g - 1) / g; };
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    for (int C = 1; C <= std::min(16, ny_max); ++C) {
+        if (force_c > 0 && C != force_c) continue;
+        int nodes, ipts;
+        launch_caps<Real, NS>(c, C, nodes, ipts, true);
+        int last_units = 0;
+        for (int g = 1; g <= NU; ++g) {
+            // (a forced number of frequencies per pass is spread evenly over as many passes, or
+            // over the fewest that fit)
+            if (force_f > 0) g = std::max(g, (NU + force_f - 1) / force_f);
+            const int F = even(g);
+            const int units = (F + jsweep_lanes<Real>() - 1) / jsweep_lanes<Real>();
+            if (units == last_units) continue;
+            last_units = units;
+            int threads = 0;
+            const int tots = jsweep_tots<Real, NS>(c, C, F, &threads);
+            const int smem = jsweep_smem_bytes<Real, NS>(nodes, ipts, tots, F);
+            if (smem > kJSmemLimit) continue;
+            const int G = jsweep_groups<Real>(NU, F);
+            const int parts = sizeof(Real) == 4 ? G : 1;
+            const long long n = (long long)nitems * parts;
+            double total = 0.0, item_max = 0.0;
+            for (const BoxDev &b : c->boxes) {
+                const double item =
+                    (double)b.nz * (G / parts) * jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads);
+                total += item * c->nray * parts;
+                item_max = std::max(item_max, item);
+            }
+            // (CTAs on one SM hide one another's chains, but share its FP64 pipe)
+            auto cost = [&](int ncl) {
+                const double share = sizeof(Real) == 8 ? std::max(1, (ncl * C + nsm - 1) / nsm) : 1;
+                return share * (c->nbox == 1 ? (double)((n + ncl - 1) / ncl) * item_max : std::max(total / ncl, item_max) * 1.05);
+            };
+            // no better even with every SM's thread slots taken
+            const int per_sm = std::min(2048 / threads, 227 * 1024 / (smem + 1024));
+            const double bound = cost(std::max(1, nsm * (sizeof(Real) == 8 ? 1 : std::max(1, per_sm)) / C));
+            if (best.cluster > 0 && bound >= best_cost) continue;
+            int act = 0;
+            if (jsweep_max_active_clusters<Real, NS>(C, smem, threads, &act) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if (act < 1) continue;
+            const int ncl = (int)std::min<long long>(act, n);
+            if (cost(ncl) < best_cost) {
+                best_cost = cost(ncl);
+                best = {C, F, threads, smem, ncl, 0};
+            }
+            if (force_f > 0) break;
+        }
+    }
+    return best.cluster > 0 ? PORTA_OK : PORTA_EINVAL;
+}
+
+// Launch shape of the general sweep: cluster size C (CTAs sharing one ray's plane)
 // and frequencies per pass F. Estimated time of a candidate (in units of one
 // point update): the (box, ray) work items spread over the resident clusters,
 // each item costing, per plane and frequency pass, the thread slots of its
 // point updates, the ring fill (halo rows included), the partial-integral
 // writes and a barrier.
 template <typename Real, int NS>
-int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, bool jk = false, int nnu = 0)
+int choose_sweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, int NU, bool wide = false)
 {
-    const int NU = nnu > 0 ? nnu : c->n_nu;     // frequencies swept
-    if (force_f > NU) force_f = NU;
     // accumulated quantities per point (Stokes V too for the polarized lines of a multilevel atom)
     const int NA = NS == 1 ? 2 : (c->d_dich ? 5 : 4);
     double best_cost = 1e300;
@@ -197,15 +319,15 @@ int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int n
         if (force_c <= 0 && C > 1 && (C & (C - 1)) != 0 && C != 6 && C != 12) continue;   // heuristic set
         if (C > ny_max) continue;
         // biquadratic stencils reach two rows into the next strip: every CTA needs two rows
-        if (c->interp == 2 && !c->d_kexpl && !jk && min_ny(c) / C < 2) continue;
+        if (c->interp == 2 && !c->d_kexpl && !wide && min_ny(c) / C < 2) continue;
         int ring_plane, ipts_max;
-        launch_caps<Real, NS>(c, C, ring_plane, ipts_max, jk);
+        launch_caps<Real, NS>(c, C, ring_plane, ipts_max, wide);
         int fmax = 0;
-        if (jk) {
-            // J^K_Q kernel: besides the Stokes planes, each frequency of a pass keeps
-            // the nodes' coefficients of three planes (jsweep_smem_bytes)
+        if (wide) {
+            // besides the Stokes planes, each frequency of a pass keeps the nodes' coefficients
+            // of three planes
             for (int f = NU; f >= 1 && fmax == 0; --f)
-                if (jsweep_smem_bytes<Real, NS>(ring_plane, ipts_max, f, kThreads) <= kSmemLimit) fmax = f;
+                if (jwide_smem_bytes<Real, NS>(ring_plane, ipts_max, f, kThreads) <= kSmemLimit) fmax = f;
             if (fmax == 0) continue;
         } else {
             const long long ring = 3LL * ring_plane * 16;
@@ -222,14 +344,13 @@ int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int n
         const int F = (NU + G - 1) / G;
         // threads: the strip's points times the frequency lanes they can use, whole warps, 64..512
         const int threads = std::min(kThreads, std::max(64, (ipts_max * F + 31) / 32 * 32));
-        const int smem = jk ? jsweep_smem_bytes<Real, NS>(ring_plane, ipts_max, F, threads)
-                            : sweep_smem_bytes<Real, NS>(ring_plane, ipts_max, F, threads, NA);
+        const int smem = wide ? jwide_smem_bytes<Real, NS>(ring_plane, ipts_max, F, threads)
+                              : sweep_smem_bytes<Real, NS>(ring_plane, ipts_max, F, threads, NA);
         if (smem > kSmemLimit + 16) continue;
         int act = 0;
-        if ((jk ? jsweep_max_active_clusters<Real, NS>(C, smem, threads, &act)
-                : max_active_clusters<Real, NS>(C, smem, threads, &act, c->d_dich != nullptr,
-                                                c->interp == 2 && !c->d_kexpl, c->d_kexpl != nullptr)) !=
-            cudaSuccess) {
+        if ((wide ? jwide_max_active_clusters<Real, NS>(C, smem, threads, &act)
+                  : max_active_clusters<Real, NS>(C, smem, threads, &act, c->d_dich != nullptr,
+                                                  c->interp == 2 && !c->d_kexpl, c->d_kexpl != nullptr)) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -256,6 +377,28 @@ int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int n
         }
     }
     return best.cluster > 0 ? PORTA_OK : PORTA_EINVAL;
+}
+
+// The shape of a context's sweep (jk: the J^K_Q sweep's). It follows from sizes and options
+// alone and takes some tens of occupancy queries, so the context keeps what it chose.
+template <typename Real, int NS>
+int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, bool jk = false, int nnu = 0)
+{
+    const int NU = nnu > 0 ? nnu : c->n_nu;     // frequencies swept
+    if (force_f > NU) force_f = NU;
+    const std::array<int, 8> key = {force_c, force_f, nitems, jk ? c->jk_form : 0, NU, c->d_dich != nullptr, c->interp, c->d_kexpl != nullptr};
+    for (const auto &s : c->shapes)
+        if (s.first == key) {
+            best = s.second;
+            return PORTA_OK;
+        }
+    const int rc = jk && c->jk_form == 1 ? choose_jsweep<Real, NS>(c, best, force_c, force_f, nitems, NU)
+                                         : choose_sweep<Real, NS>(c, best, force_c, force_f, nitems, NU, jk);
+    if (rc == PORTA_OK) {
+        if (c->shapes.size() >= 64) c->shapes.clear();
+        c->shapes.emplace_back(key, best);
+    }
+    return rc;
 }
 
 // sweep arguments common to every mode: sizes, atmosphere, unknowns, frequencies
@@ -291,13 +434,19 @@ template <typename Real>
 void shape_args(porta_ctx *c, SweepArgs<Real> &a, const LaunchCfg &cfg, bool jk = false)
 {
     a.F = cfg.F;
-    a.ngroups = (a.nnu + cfg.F - 1) / cfg.F;
+    const bool split = jk && c->jk_form == 1;
+    a.ngroups = split ? jsweep_groups<Real>(a.nnu, cfg.F) : (a.nnu + cfg.F - 1) / cfg.F;
     if (c->ns == 1)
         launch_caps<Real, 1>(c, cfg.cluster, a.ring_plane, a.ipts_max, jk);
     else
         launch_caps<Real, 4>(c, cfg.cluster, a.ring_plane, a.ipts_max, jk);
-    a.cstride = jsweep_stride(a.ring_plane * (c->ns == 1 ? 1 : 2), (int)sizeof(Real));
-    a.istride = jsweep_stride(a.ipts_max * c->ns, (int)sizeof(Real));
+    if (jk && !split) {
+        a.cstride = jwide_stride(a.ring_plane * (c->ns == 1 ? 1 : 2), (int)sizeof(Real));
+        a.istride = jwide_stride(a.ipts_max * c->ns, (int)sizeof(Real));
+    }
+    if (split)
+        a.tots = c->ns == 1 ? jsweep_tots<Real, 1>(c, cfg.cluster, cfg.F, nullptr)
+                            : jsweep_tots<Real, 4>(c, cfg.cluster, cfg.F, nullptr);
 }
 
 // api.cu

@@ -72,24 +72,57 @@ __device__ __forceinline__ Coef<double> coefficients(double t)
     return c;
 }
 
-// Single precision: three regimes, chosen so that every coefficient stays
-// within 6e-7 relative of its exact value for all t > 0 when evaluated in
-// FP32: degree-6 series for t < 0.25 (truncation below 2e-7 there), degree-12
-// series for t < 1.5, closed forms above (where their cancellation costs at
-// most a factor ~5).
+// reciprocal: IEEE in FP64; in FP32 the hardware approximation rcp.approx.ftz
+// (max 1 ulp; the operands here are normal numbers below 2^126), since the FP32
+// form's error budget is 1e-5. The bare instruction saves the scaling steps of a
+// general approximate division (4% of the J^K_Q sweep's time).
+__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+__device__ __forceinline__ float rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Single precision: two regimes. Below t = 1.5, w / t as a polynomial whose relative
+// error on [0, 1.5] is minimax (Remez exchange on the Taylor series, coefficients
+// rounded to FP32: 5e-9 for w_M, 3e-9 for w_O, 1e-9 for w_C before rounding); above,
+// the closed forms, where their cancellation costs at most a factor ~3. Every
+// coefficient stays within 4e-7 relative of its exact value (rms 6e-8 to 8e-8). One
+// polynomial range of degree 6 or 7 takes the place of Taylor series of degree 6
+// below 0.25 and 12 below 1.5 (23 multiply-adds instead of 18 or 36, and lanes of a
+// warp no longer diverge between the two).
+__device__ __forceinline__ void wpoly(float t, float &wm, float &wo, float &wc)
+{
+    float m = fmaf(t, -9.985858924e-06f, 1.324526238e-04f);
+    float c = fmaf(t, -2.395259799e-06f, 3.410954741e-05f);
+    float o = fmaf(t, 3.294269391e-06f, -4.541862290e-05f);
+    m = fmaf(t, m, -1.014578040e-03f);
+    c = fmaf(t, c, -2.921269333e-04f);
+    o = fmaf(t, o, 3.927011858e-04f);
+    m = fmaf(t, m, 5.933146924e-03f);
+    c = fmaf(t, c, 1.980281435e-03f);
+    o = fmaf(t, o, -2.775641857e-03f);
+    m = fmaf(t, m, -2.777018584e-02f);
+    c = fmaf(t, c, -1.110962220e-02f);
+    o = fmaf(t, o, 1.666613296e-02f);
+    m = fmaf(t, m, 9.999849647e-02f);
+    c = fmaf(t, c, 4.999971390e-02f);
+    o = fmaf(t, o, -8.333328366e-02f);
+    m = fmaf(t, m, -2.499998808e-01f);
+    c = fmaf(t, c, -1.666666418e-01f);
+    o = fmaf(t, o, 3.333333433e-01f);
+    wm = t * fmaf(t, m, 3.333333433e-01f);
+    wc = t * fmaf(t, c, 3.333333433e-01f);
+    wo = t * o;
+}
 // w_M, w_O, w_C of one optical path t given e = exp(-t)
 __device__ __forceinline__ void wcoef(float t, float e, float &wm, float &wo, float &wc)
 {
-    if (t < 0.25f) {
-        wm = horner<float, 6, c_wm>(t);
-        wo = horner<float, 6, c_wo>(t);
-        wc = horner<float, 6, c_wc>(t);
-    } else if (t < 1.5f) {
-        wm = horner<float, 12, c_wm>(t);
-        wo = horner<float, 12, c_wo>(t);
-        wc = horner<float, 12, c_wc>(t);
+    if (t < 1.5f) {
+        wpoly(t, wm, wo, wc);
     } else {
-        const float it = 1.0f / t, it2 = it * it;
+        const float it = rcp(t), it2 = it * it;
         wm = (2.0f - e * (t * t + 2.0f * t + 2.0f)) * it2;
         wo = 1.0f - 2.0f * (e + t - 1.0f) * it2;
         wc = 2.0f * (t - 2.0f + e * (t + 2.0f)) * it2;
@@ -104,18 +137,6 @@ __device__ __forceinline__ Coef<float> coefficients(float t)
     c.pm = c.wm + 0.5f * c.wc;
     c.po = c.wo + 0.5f * c.wc;
     return c;
-}
-
-// reciprocal: IEEE in FP64; in FP32 the hardware approximation rcp.approx.ftz
-// (max 1 ulp; the operands here are normal numbers below 2^126), since the FP32
-// form's error budget is 1e-5. The bare instruction saves the scaling steps of a
-// general approximate division (4% of the J^K_Q sweep's time).
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float rcp(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
 }
 
 // Profile shape exp(-(x - s)^2). In FP32 it is evaluated as a power of two by

@@ -3,8 +3,10 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <array>
 #include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "ml_kernels.cuh"
@@ -48,10 +50,11 @@ struct porta_ctx {
     int n_mu = 0, n_chi = 0, n_nu = 0;
     double x_max = 4;
     int precision = PORTA_FP32;
-    bool jk_fits = true;                // a launch shape of the J^K_Q sweep kernel (sweep_j.cu) fits the grid
+    int jk_form = 1;                    // J^K_Q sweep kernel with a launch shape that fits the grid: 1 sweep_j.cu, 2 sweep_jw.cu, 0 none
     int fr0 = 0, fr1 = 0;               // frequency band [fr0, fr1) of the J^K_Q formal solution (fr1 = 0: all)
     bool jkq_loaded = false;            // J^K_Q / Lambda-bar* set by porta_set_partial (not from this context's sweep)
     int opt_cluster = 0, opt_nu_group = 0;
+    std::vector<std::pair<std::array<int, 8>, porta::LaunchCfg>> shapes;   // launch shapes chosen so far (choose_launch)
     int user_cluster = 0, user_nu_group = 0;     // as given in porta_opts (0: automatic)
     bool user_shape = false;            // launch shape given in porta_opts (not autotuned)
     std::map<int, porta::LaunchCfg> emg_tuned;   // emergent sweep: shape timed once per direction count
@@ -72,12 +75,13 @@ struct porta_ctx {
     double *d_rho = nullptr;        // nvox*nl FP64
     void *d_rhoR = nullptr;         // nl*nvox Real
     void *d_invn = nullptr;         // nray*nvox Real
-    void *d_geom = nullptr;         // nray*nz PlaneGeom
+    void *d_geom = nullptr;         // nray*nz PlaneGeom, then the same as relative_geometry gives it (J^K_Q sweep)
     void *d_rays = nullptr;         // nray RayDev
     void *d_freq = nullptr;         // xf, wf (Real)
     void *d_part = nullptr;         // nray*nvox*(ns==1 ? 2 : 4) Real (general sweep only; allocated on first use)
     unsigned long long *d_jacc = nullptr;   // J^K_Q sweep: fixed-point sums [nj + 1][nvox] (allocated on first use)
     int *d_jexp = nullptr;                  // J^K_Q sweep: per-voxel fixed-point exponent
+    void *d_jpack = nullptr;                // J^K_Q sweep: packed inputs, jpack_words Reals per voxel
     double *d_tw = nullptr;         // nray*19 FP64: w_m, T (18)
     double *d_jkq = nullptr, *d_lstar = nullptr;
     unsigned long long *d_resid = nullptr;

@@ -49,9 +49,9 @@ struct SweepArgs {
     const int *items;    // J mode: item -> box * nray + ray, ordered by decreasing cost
     const BoxDev *boxes;
     int ngroups, F;      // frequency groups and frequencies per group
+    int tots;            // J^K_Q sweep: entries of the totals buffer (0: one group of threads everywhere)
     int ring_plane;      // shared-memory ring plane capacity (16-byte chunks), max over boxes
     int ipts_max;        // Stokes-plane capacity (points), max over boxes
-    int cstride, istride;  // J^K_Q sweep: Reals per (slot, frequency) coefficient plane and per (buffer, frequency) Stokes plane
     int interp;            // general sweep: 2 biquadratic interpolation at M and P, else bilinear
     // explicit medium (emergent general sweep, NS = 4): K'/eta_I [6][nvox] and S [4][nvox], FP64
     const double *kexpl, *sexpl;
@@ -92,6 +92,8 @@ struct SweepArgs {
     unsigned long long *jacc;
     const int *jexp;
     int *jerr;
+    int cstride, istride;          // wide planes (sweep_jw.cu): Reals per coefficient and per Stokes plane
+    const Real *pack;              // the voxels' inputs side by side, jpack_words each (launch_jacc_prepare)
 };
 
 struct LaunchCfg {
@@ -118,22 +120,59 @@ cudaError_t max_active_clusters(int cluster, int smem, int threads, int *out, bo
 
 // the J^K_Q formal solution (sweep_j.cu): per-frequency node coefficients in
 // shared memory; ring capacity `nodes` per slot, Stokes planes of `ipts` points.
-// Plane strides are padded to 16 (mod 32) 4-byte words, so that the two
-// frequency lanes of a point (adjacent threads) read distinct banks.
-__host__ __device__ inline int jsweep_stride(int reals, int real_bytes)
+// Frequencies an update thread handles at a time: in FP32 a pair, whose arithmetic is
+// packed (FFMA2, FMUL2, FADD2); in FP64 one.
+template <typename Real> __host__ __device__ constexpr int jsweep_lanes() { return sizeof(Real) == 4 ? 2 : 1; }
+// passes that F frequencies each need for nnu, in whole lane groups
+template <typename Real> __host__ __device__ inline int jsweep_groups(int nnu, int F)
+{
+    constexpr int W = jsweep_lanes<Real>();
+    const int fx = (F + W - 1) / W, n = (nnu + W - 1) / W;
+    return (n + fx - 1) / fx;
+}
+// threads of a CTA whose strip has R rows of nx columns: whole warps of points, in equal
+// rounds where these exceed tmax, else times the frequency groups that fit
+__host__ __device__ inline int jsweep_threads(int nx, int R, int FX, int tmax)
+{
+    const int pts = nx * R;
+    int n;
+    if (pts > tmax) {
+        const int rounds = (pts + tmax - 1) / tmax;
+        n = ((pts + rounds - 1) / rounds + 31) / 32 * 32;
+    } else {
+        const int pw = (pts + 31) / 32 * 32;
+        const int l = FX < tmax / pw ? FX : tmax / pw;
+        n = pw * l;
+    }
+    return n < 64 ? 64 : n;
+}
+template <typename Real, int NS> constexpr int jsweep_max_threads() { return NS == 4 && sizeof(Real) == 8 ? 256 : 512; }
+template <typename Real, int NS>
+int jsweep_smem_bytes(int nodes, int ipts, int tots, int F);
+template <typename Real, int NS>
+cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out);
+template <typename Real, int NS>
+cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st);
+// the same for planes too wide for sweep_j.cu's shared memory (sweep_jw.cu: three ring slots
+// instead of four, one frequency per unit, no staged inputs). Plane strides are padded to 16
+// (mod 32) 4-byte words, so that the two frequency lanes of a point (adjacent threads) read
+// distinct banks.
+__host__ __device__ inline int jwide_stride(int reals, int real_bytes)
 {
     int words = reals * real_bytes / 4;
     words += ((16 - words % 32) + 32) % 32;
     return words * 4 / real_bytes;
 }
 template <typename Real, int NS>
-int jsweep_smem_bytes(int nodes, int ipts, int F, int threads);
+int jwide_smem_bytes(int nodes, int ipts, int F, int threads);
 template <typename Real, int NS>
-cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out);
+cudaError_t jwide_max_active_clusters(int cluster, int smem, int threads, int *out);
 template <typename Real, int NS>
-cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st);
-// before a J^K_Q formal solution: zero the fixed-point accumulators and set each
-// voxel's scale exponent; after it: J^K_Q and Lambda-bar* in FP64 from them
+cudaError_t launch_jwide(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st);
+// words of a voxel's packed inputs
+template <int NS> constexpr int jpack_words() { return NS == 1 ? 4 : 12; }
+// before a J^K_Q formal solution: pack the voxels' inputs, zero the fixed-point
+// accumulators and set each voxel's scale exponent (where jacc is set); after it: J^K_Q and Lambda-bar* in FP64 from them
 template <typename Real, int NS>
 cudaError_t launch_jacc_prepare(const SweepArgs<Real> &a, cudaStream_t st);
 template <int NS>

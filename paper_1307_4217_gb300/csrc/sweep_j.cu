@@ -4,32 +4,48 @@
 // and Lambda* that feeds J^K_Q (Eq. 1, Eq. 14) and the Jacobi update.
 //
 // The decomposition is that of the general sweep (sweep.cu): one thread-block
-// cluster per ray at a time, the plane split into strips of sheared rows, one
-// per CTA, with the first row of the next strip read through DSMEM after a
-// cluster barrier, and the stencils of the bilinear interpolation at the
-// upwind point M and downwind point P fixed nearest-neighbour accesses in the
+// cluster per ray and frequency group at a time, the plane split into strips of
+// sheared rows, one per CTA; the stencils of the bilinear interpolation at the
+// upwind point M and downwind point P are fixed nearest-neighbour accesses in the
 // frame sheared along the characteristics.
 //
-// What this kernel does differently. The transfer coefficients of a node
-// depend on the frequency only through the profile, eta_I = chi phi(x - s) and
-// eta_V = b (x - s) eta_I, while its source vector S(Omega) does not (CRD).
-// When a plane enters the 3-slot ring, its nodes' frequency-independent data
-// (S_I, S_Q, S_U, S^0_0 | chi, s, b, 1/N) are staged once, and then, for every
-// frequency of the pass, the node's (eta_I, eta_V) are computed once and kept
-// in shared memory. A point update then interpolates eps = sum_k w_k eta_k S_k
+// The transfer coefficients of a node depend on the frequency only through the
+// profile, eta_I = chi phi(x - s) and eta_V = b (x - s) eta_I, while its source
+// vector S(Omega) does not (CRD). When a plane enters the 4-slot ring, a thread per
+// node writes the node's source vector once and its (eta_I, eta_V) at every
+// frequency of the pass. A point update then interpolates eps = sum_k w_k eta_k S_k
 // and eta = sum_k w_k eta_k from its 4 upwind and 4 downwind corners without
-// evaluating a profile: the corners' source vectors are read once per point
-// (registers across the frequency loop), their (eta_I, eta_V) once per
-// frequency. Only the point O itself evaluates its profile (for Lambda* and
-// the frequency-integration weight).
+// evaluating a profile.
 //
-// Shared memory per CTA:
-//   ring[3][NCH][nodes]   frequency-independent node data (16-byte chunks)
-//   coef[3][F][nodes]     (eta_I, eta_V) (NS = 4) or eta_I (NS = 1) per frequency
-//   ibuf[2][F][...][pts]  Stokes vectors of planes q-1 and q
-//   lane[threads][NA]     fixed-order frequency-lane reduction
+// An update thread owns a point and takes the frequencies of the pass one unit after
+// the other: two adjacent frequencies in FP32, whose operations are packed (FFMA2,
+// FMUL2, FADD2) wherever no factor is common to both, one frequency in FP64.
+//
+// Strips exchange only their first row: the CTA that computed it writes it into the
+// halo row of the strip before with st.async, which counts the bytes on that CTA's
+// mbarrier, so no CTA waits for another one except for the halo row itself, and
+// nothing waits for a fence of the fixed-point sums in flight. The inputs of the next
+// planes' nodes travel by cp.async during the updates.
+//
+// What bounds it: instruction issue and the length of a plane's chain of operations, not
+// memory (the inputs are re-read from L2). A plane and pass takes about 2660 cycles of fixed
+// chain, 1106 per unit of its points' rounds and 1190 + 151 per unit for the nodes (NS = 4,
+// FP32; jsweep_plane_cost), whatever the strip, so a pass has few units over as many points
+// as the threads hold. Against the kernel of sweep_jw.cu, which this one replaces where it
+// fits (one frequency of one point per thread and step, one cluster barrier per plane), ms
+// per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 18.7, 33 x 27 x 41 x
+// 80 x 21 1.91 -> 1.25, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.8, 64 x 64 x 48 x 160 x 31
+// x 2 lines, unpolarized, 46.4 -> 32.6 (with the rate equations).
+//
+// Shared memory per CTA (X: 8 bytes, a frequency unit):
+//   ring[4][nodes]        source vectors, Real
+//   coef[4][FX][nodes]    (eta_I, eta_V) (NS = 4) or eta_I (NS = 1), X
+//   ibuf[2][FX][points + a halo row]   Stokes vectors of planes q - 1 and q, X
+//   tot, stage, ...       point totals, inputs in flight, geometry
 // with nodes = (rows + 2) nx (one halo row on each side, recomputed locally).
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "device_math.cuh"
 #include "porta_internal.cuh"
@@ -41,17 +57,13 @@ namespace porta {
 
 namespace {
 
-// Shared-memory words per node: the ring holds the frequency-independent source
-// vector (NS = 4: S_I, S_Q, S_U, S^0_0 as 16-byte chunks; NS = 1: S as a scalar
-// plane); the transient staging area holds (chi, s[, b]) of the plane being
-// filled, for the per-frequency coefficients.
 template <typename Real, int NS>
 struct JW {
     static constexpr int per = 16 / (int)sizeof(Real);        // Reals per 16-byte chunk
     static constexpr int s_words = NS == 1 ? 1 : 4;            // source words per node
     static constexpr int s_chunks = NS == 1 ? 0 : 4 / per;     // 16-byte chunks per node (NS = 4)
-    static constexpr int g_words = NS == 1 ? 2 : 3;            // staged geometry words per node
-    static constexpr int cw = NS == 1 ? 1 : 2;                 // coefficient words per node and frequency
+    static constexpr int staged = NS == 1 ? 4 : 12;            // words of a voxel's packed inputs
+    static constexpr int cw = NS == 1 ? 1 : 2;                 // coefficients (X) per node and unit
     static constexpr int na = NS == 1 ? 2 : 4;                 // accumulated quantities per point
     static constexpr int nacc = NS == 1 ? 2 : 7;               // fixed-point accumulators per voxel
 };
@@ -80,34 +92,25 @@ constexpr int kJFrac = 46;   // fixed-point fraction bits below a voxel's refere
 __device__ __forceinline__ float pow2(float, int e) { return __int_as_float((e + 127) << 23); }
 __device__ __forceinline__ double pow2(double, int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// one term of the fixed-point sum: x * 2^e (exact) rounded to an integer. Integer
-// additions are exact and commute, so the sums do not depend on the order in which
-// rays, frequency passes and concurrent launches add their terms. A term beyond
-// 2^62 (or not finite) sets the overflow flag instead.
-__device__ __forceinline__ void jadd(unsigned long long *p, float y, int *err)
+// one term of the fixed-point sum: the integer nearest to y (an FP32 value times a power of
+// two) added to *p. Integer additions are exact and commute, so the sums do not depend on
+// the order in which rays, frequency passes and concurrent launches add their terms.
+// Returns whether the term is beyond 2^62 (or not finite); its sum is then void and the
+// caller reports it.
+// y = h 2^40 + m 2^18 + l by adding 1.5 2^23, whose sum's low bits are the integer nearest
+// to the addend: every step is exact but the last, which rounds y to an integer. (The
+// conversion instruction, float to 64-bit integer, runs in the FP64 pipe at two lanes a
+// cycle and SM: 16 cycles each, 7 per point, 12% of the time of a 64 x 64 plane.)
+__device__ __forceinline__ bool jadd(unsigned long long *p, float y)
 {
-    if (!(fabsf(y) < 4.6116860e18f)) {
-        atomicOr(err, 1);
-        return;
-    }
-    // y = +-m 2^ex with the 24-bit significand m: the integer nearest to y from
-    // integer operations (halves away from zero; |y| < 2^-1 gives 0)
-    const unsigned b = __float_as_uint(y);
-    const int ex = (int)((b >> 23) & 0xffu) - 150;
-    const unsigned m = (b & 0x7fffffu) | 0x800000u;
-    long long n = 0;
-    if (ex >= 0) n = (long long)((unsigned long long)m << ex);
-    else if (ex > -25) n = (long long)((m + (1u << (-ex - 1))) >> (-ex));
-    if (b >> 31) n = -n;
-    atomicAdd(p, (unsigned long long)n);
-}
-__device__ __forceinline__ void jadd(unsigned long long *p, double y, int *err)
-{
-    if (!(fabs(y) < 4.611686018427387904e18)) {
-        atomicOr(err, 1);
-        return;
-    }
-    atomicAdd(p, (unsigned long long)__double2ll_rn(y));
+    constexpr float M = 12582912.0f;
+    constexpr unsigned B = 0x4b400000u;                        // bits of M
+    const float h = fmaf(y, 0x1p-40f, M), r = fmaf(M - h, 0x1p40f, y);
+    const float m = fmaf(r, 0x1p-18f, M), l = fmaf(M - m, 0x1p18f, r) + M;
+    const unsigned long long k = (unsigned long long)__float_as_uint(m) * (1u << 18) +
+                                 (((unsigned long long)(__float_as_uint(h) - B) << 40) - (unsigned long long)B * ((1u << 18) + 1u));
+    atomicAdd(p, k + __float_as_uint(l));
+    return !(fabsf(y) < 4.6116860e18f);
 }
 
 // per-ray partial integrals of a point (the FP64 form: summed over rays in ray
@@ -128,555 +131,940 @@ __device__ __forceinline__ void store_partial(const SweepArgs<Real> &a, int m, l
     }
 }
 
+// byte offsets of the dynamic shared memory (the ring of source vectors comes first) and
+// strides of its coefficient and Stokes planes (one frequency unit each)
+struct JSmem { unsigned coef, ibuf, tot, stage, geo, freq, wgt, vox, stw, ste, stv, end, cplane, iplane; };
+template <typename Real, int NS>
+__host__ __device__ inline JSmem jsmem(int nodes, int pts, int tots, int FX)
+{
+    using W = JW<Real, NS>;
+    const unsigned rb = (unsigned)sizeof(Real);
+    auto up16 = [](unsigned x) { return (x + 15u) / 16u * 16u; };
+    JSmem s;
+    s.cplane = up16(nodes * W::cw * 8);
+    s.iplane = up16(pts * NS * 8);
+    s.coef = up16(4 * nodes * W::s_words * rb);
+    s.ibuf = s.coef + 4 * FX * s.cplane;
+    s.tot = s.ibuf + 2 * FX * s.iplane;
+    s.stage = s.tot + up16(2 * tots * W::na * rb);
+    s.geo = s.stage + W::staged * nodes * rb;
+    s.freq = s.geo + 8 * (unsigned)sizeof(PlaneGeom<Real>);
+    s.wgt = s.freq + 2 * FX * 8;
+    s.stw = s.wgt + 4 * nodes * rb;
+    s.vox = s.stw + nodes * rb;
+    s.ste = s.vox + 4 * nodes * 4;
+    s.stv = s.ste + nodes * 4;
+    s.end = s.stv + nodes * 4;
+    return s;
+}
+
 }  // namespace
 
 template <typename Real, int NS>
-int jsweep_smem_bytes(int nodes, int ipts, int F, int threads)
+int jsweep_smem_bytes(int nodes, int ipts, int tots, int F)
 {
-    using W = JW<Real, NS>;
-    (void)threads;
-    const int ring = (3 * nodes * W::s_words * (int)sizeof(Real) + 15) / 16 * 16;
-    const int coef = (3 * F * jsweep_stride(nodes * W::cw, (int)sizeof(Real)) * (int)sizeof(Real) + 15) / 16 * 16;
-    const int stokes = 2 * F * jsweep_stride(ipts * NS, (int)sizeof(Real)) * (int)sizeof(Real);
-    const int stage = W::g_words * nodes * (int)sizeof(Real);
-    const int freq = 2 * F * (int)sizeof(Real);
-    return ring + coef + stokes + stage + freq;
+    constexpr int W = jsweep_lanes<Real>();
+    return (int)jsmem<Real, NS>(nodes, ipts, tots, (F + W - 1) / W).end;
 }
 
-// Pairs of Reals: the Stokes vector of the polarized atom is handled as the pairs
-// (I, Q) and (U, V), whose arithmetic shares every coefficient. In FP32 a pair
-// op is one packed instruction (FFMA2, FMUL2, FADD2: each lane rounds exactly
-// as the scalar op); in FP64 it is two scalar ops.
-template <typename Real> struct PairT;
-template <> struct PairT<float> { using T = float2; };
-template <> struct PairT<double> { using T = double2; };
+// ---- frequency units: a pair of floats (every operation packed; each lane rounds as the
+// scalar operation) or one double -----------------------------------------------------
+template <typename Real> struct XOf;
+template <> struct XOf<float> { using X = float2; };
+template <> struct XOf<double> { using X = double; };
 
-__device__ __forceinline__ float2 pmk(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ double2 pmk(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ double2 pmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ double2 pfma(double2 a, double2 b, double2 c)
+__device__ __forceinline__ float2 xset(float a) { return make_float2(a, a); }
+__device__ __forceinline__ double xset(double a) { return a; }
+__device__ __forceinline__ float2 xmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 xfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 xadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ double xmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double xfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double xadd(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 xneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ double xneg(double a) { return -a; }
+__device__ __forceinline__ float2 xrcp(float2 a) { return make_float2(rcp(a.x), rcp(a.y)); }
+__device__ __forceinline__ double xrcp(double a) { return rcp(a); }
+// -1 / a
+__device__ __forceinline__ float2 xnrcp(float2 a) { return make_float2(rcp(-a.x), rcp(-a.y)); }
+__device__ __forceinline__ double xnrcp(double a) { return rcp(-a); }
+// the same Real times both lanes (scalar operations: a pair made of one value costs a move)
+__device__ __forceinline__ float2 xms(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
+__device__ __forceinline__ double xms(double s, double a) { return s * a; }
+__device__ __forceinline__ float2 xfs(float s, float2 a, float2 c) { return make_float2(fmaf(s, a.x, c.x), fmaf(s, a.y, c.y)); }
+__device__ __forceinline__ double xfs(double s, double a, double c) { return fma(s, a, c); }
+// s + sum over the lanes of a b
+__device__ __forceinline__ float xdot(float2 a, float2 b, float s) { return fmaf(a.y, b.y, fmaf(a.x, b.x, s)); }
+__device__ __forceinline__ double xdot(double a, double b, double s) { return fma(a, b, s); }
+__device__ __forceinline__ float2 xprofile(float2 xs) { return make_float2(profile_shape(xs.x), profile_shape(xs.y)); }
+__device__ __forceinline__ double xprofile(double xs) { return profile_shape(xs); }
+// 1 - a^2
+__device__ __forceinline__ float2 xdet(float2 a) { return make_float2(1.0f - a.x * a.x, 1.0f - a.y * a.y); }
+__device__ __forceinline__ double xdet(double a) { return 1.0 - a * a; }
+__device__ __forceinline__ float xlane(float2 a, int i) { return i ? a.y : a.x; }
+__device__ __forceinline__ double xlane(double a, int) { return a; }
+
+// Coefficients of the step (Eqs. 9-13) of a unit: e = e^-t and the three w. In FP32 e^-t is
+// one hardware power of two (its argument's rounding, t 2^-24 relative, is multiplied by
+// e^-t <= 1/(e t) in the step); the polynomial and the closed forms are evaluated where
+// some lane needs them.
+template <typename X> struct XCoef { X e, wm, wo, wc; };
+__device__ __forceinline__ XCoef<double> xcoef(double t)
 {
-    return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
+    const Coef<double> c = coefficients(t);
+    return {c.e, c.wm, c.wo, c.wc};
 }
-__device__ __forceinline__ double2 padd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-
-// BESSER control points (Sec. 3.2, steps 1-9) of two Stokes parameters at once;
-// the same steps and selections as control_point (device_math.cuh)
-template <typename P2, typename Real>
-__device__ __forceinline__ P2 control_point2(P2 yM, P2 yO, P2 yP, const BesserGeom<Real> &g)
+__device__ __forceinline__ XCoef<float2> xcoef(float2 t)
 {
-    const P2 dm = psub(yO, yM), dp = psub(yP, yO);                      // step 1
-    const P2 yp = pfma(pmk(g.a, g.a), dp, pmul(pmk(g.b, g.b), dm));     // step 3 (Eq. 6)
-    const P2 w = pmul(pmk(g.hm2, g.hm2), yp);                            // step 4: c_M = y_O - w
-    P2 u = pmul(pmk(g.hp2, g.hp2), yp);                                  //         c_P = y_O + u
-    const P2 tc = pmul(u, psub(u, dp));                                  // step 7: c_P outside [y_O, y_P]
-    u.x = tc.x > Real(0) ? dp.x : u.x;
-    u.y = tc.y > Real(0) ? dp.y : u.y;
-    const P2 c9 = pfma(pmk(-g.r, -g.r), u, yO);                          // steps 8-9
-    const P2 to = pmul(psub(dm, w), w);                                  // steps 5-6: c_M outside [y_M, y_O]
-    const P2 te = pmul(dm, dp);                                          // step 2: extremum at O
-    P2 r;
-    r.x = te.x <= Real(0) ? yO.x : (to.x < Real(0) ? yM.x : c9.x);
-    r.y = te.y <= Real(0) ? yO.y : (to.y < Real(0) ? yM.y : c9.y);
+    XCoef<float2> c;
+    const float2 u = xmul(t, xset(-1.4426950408889634f));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(c.e.x) : "f"(u.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(c.e.y) : "f"(u.y));
+    if (fmaxf(t.x, t.y) >= 1.5f) {
+        const float2 one = xset(1.0f), two = xset(2.0f), it = xrcp(t), it2 = xmul(it, it), ne = xneg(c.e);
+        const float2 tp = xadd(t, two);
+        c.wm = xmul(xfma(ne, xfma(t, tp, two), two), it2);
+        c.wo = xfma(xmul(xadd(xadd(c.e, t), xset(-1.0f)), xset(-2.0f)), it2, one);
+        c.wc = xmul(xmul(xfma(c.e, tp, xadd(t, xset(-2.0f))), two), it2);
+    }
+    if (fminf(t.x, t.y) < 1.5f) {
+        float m, o, k;
+        wpoly(t.x, m, o, k);
+        if (t.x < 1.5f) { c.wm.x = m; c.wo.x = o; c.wc.x = k; }
+        wpoly(t.y, m, o, k);
+        if (t.y < 1.5f) { c.wm.y = m; c.wo.y = o; c.wc.y = k; }
+    }
+    return c;
+}
+
+// y_O - c_M of the BESSER control point (Sec. 3.2, steps 1-9) from d_M = y_O - y_M and
+// -d_P = y_O - y_P. The parabola's c_M = y_O - w has w = a d_P + b d_M, and the step clipped
+// at c_P = y_P has w = r d_P (Eq. 6 times h_M / 2). Past step 2 (d_M d_P <= 0: c_M = y_O)
+// both differences and w have one sign, so the interval tests compare magnitudes: |w| >
+// |d_M| is c_M outside [y_M, y_O] (steps 5-6, c_M = y_M), |w| > |r d_P| is c_P outside
+// [y_O, y_P] (steps 7-9). na = -a, nr = -r.
+template <typename Real> __device__ __forceinline__ Real cp_select(Real dm, Real w, Real rdp, Real te)
+{
+    Real c = fabs(w) > fabs(rdp) ? rdp : w;
+    c = fabs(w) > fabs(dm) ? dm : c;
+    return te < Real(0) ? c : Real(0);
+}
+__device__ __forceinline__ float2 xoffset(float2 dm, float2 ndp, float2 na, float2 b, float2 nr)
+{
+    const float2 w = xfma(na, ndp, xmul(b, dm)), rdp = xmul(nr, ndp), te = xmul(dm, ndp);
+    return make_float2(cp_select(dm.x, w.x, rdp.x, te.x), cp_select(dm.y, w.y, rdp.y, te.y));
+}
+__device__ __forceinline__ double xoffset(double dm, double ndp, double na, double b, double nr)
+{
+    return cp_select(dm, fma(na, ndp, b * dm), nr * ndp, dm * ndp);
+}
+
+// ---- shared memory by 32-bit address -------------------------------------------------
+// (a generic pointer to the dynamic array costs an addition of the CTA's window per
+// access). volatile keeps the accesses' order against barriers; stores clobber memory.
+__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void lds(unsigned a, int &x) { asm volatile("ld.shared.s32 %0, [%1];" : "=r"(x) : "r"(a)); }
+__device__ __forceinline__ void lds(unsigned a, float &x) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(a)); }
+__device__ __forceinline__ void lds(unsigned a, double &x) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(x) : "r"(a)); }
+__device__ __forceinline__ void lds(unsigned a, float2 &x)
+{
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y) : "r"(a));
+}
+// two units (16 bytes)
+__device__ __forceinline__ void lds2(unsigned a, float2 &x, float2 &y)
+{
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(y.x), "=f"(y.y) : "r"(a));
+}
+__device__ __forceinline__ void lds2(unsigned a, double &x, double &y)
+{
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(x), "=d"(y) : "r"(a));
+}
+// four Reals: one 16-byte chunk in FP32, two in FP64, `ch` bytes apart
+__device__ __forceinline__ void lds4(unsigned a, unsigned, float *w)
+{
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3]) : "r"(a));
+}
+__device__ __forceinline__ void lds4(unsigned a, unsigned ch, double *w)
+{
+    lds2(a, w[0], w[1]);
+    lds2(a + ch, w[2], w[3]);
+}
+__device__ __forceinline__ void sts(unsigned a, int x) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(x) : "memory"); }
+__device__ __forceinline__ void sts(unsigned a, float x) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(x) : "memory"); }
+__device__ __forceinline__ void sts(unsigned a, double x) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory"); }
+__device__ __forceinline__ void sts(unsigned a, float2 x)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x.x), "f"(x.y) : "memory");
+}
+__device__ __forceinline__ void sts2(unsigned a, float2 x, float2 y)
+{
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y) : "memory");
+}
+__device__ __forceinline__ void sts2(unsigned a, double x, double y)
+{
+    asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(x), "d"(y) : "memory");
+}
+__device__ __forceinline__ void sts4(unsigned a, unsigned, const float *w)
+{
+    sts2(a, make_float2(w[0], w[1]), make_float2(w[2], w[3]));
+}
+__device__ __forceinline__ void sts4(unsigned a, unsigned ch, const double *w)
+{
+    sts2(a, w[0], w[1]);
+    sts2(a + ch, w[2], w[3]);
+}
+// copies from global to shared memory that pass through no register (completed by
+// copies_wait of the same thread)
+template <typename T> __device__ __forceinline__ void copy_async(unsigned dst, const T *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"((int)sizeof(T)) : "memory");
+}
+__device__ __forceinline__ void copy_async16(unsigned dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// a / b with the approximate reciprocal's error removed by one residual step (the error of a
+// node's weight is common to all rays: unlike a step's rounding it would not average out)
+__device__ __forceinline__ float quotient(float a, float b)
+{
+    const float r = rcp(b), q = a * r;
+    return fmaf(fmaf(-q, b, a), r, q);
+}
+__device__ __forceinline__ double quotient(double a, double b) { return a * rcp(b); }
+
+// keeps the compiler from rebuilding a corner's address from its parts at every use
+__device__ __forceinline__ unsigned opaque(unsigned x)
+{
+    asm("" : "+r"(x));
+    return x;
+}
+
+// ---- the halo exchange -----------------------------------------------------------------
+__device__ __forceinline__ unsigned map_rank(unsigned addr, int rank)
+{
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+// stores to another CTA's shared memory that count their bytes on its mbarrier
+__device__ __forceinline__ void push(unsigned dst, unsigned bar, float2 x)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(dst),
+                 "f"(x.x), "f"(x.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void push(unsigned dst, unsigned bar, double x)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(dst), "d"(x),
+                 "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void push2(unsigned dst, unsigned bar, float2 x, float2 y)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
+                     dst), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void push2(unsigned dst, unsigned bar, double x, double y)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(dst),
+                 "d"(x), "d"(y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void bar_init(unsigned bar)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void bar_expect(unsigned bar, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bar_arrive_remote(unsigned bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ unsigned bar_try(unsigned bar, unsigned parity)
+{
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok;
+}
+// Bounded wait for the phase of the given parity. A wait that runs out (the neighbouring
+// CTA stopped) marks the CTA, which from then on waits for and signals nothing (its
+// neighbours' waits run out in turn), and sets the error flag; the kernel then ends with
+// wrong sums and the host reports the flag.
+__device__ __noinline__ void bar_wait_long(unsigned bar, unsigned parity, volatile int *dead, int *err)
+{
+    for (int i = 0; i < (1 << 21); ++i) {
+        if (bar_try(bar, parity) || *dead) return;
+    }
+    *dead = 1;
+    atomicOr(err, 4);
+}
+__device__ __forceinline__ void bar_wait(unsigned bar, unsigned parity, volatile int *dead, int *err)
+{
+    if (!*dead && !bar_try(bar, parity)) bar_wait_long(bar, parity, dead, err);
+}
+
+// Shared control words of a CTA: full (word b) counts the bytes of the halo row of the
+// planes of parity b that the next strip's CTA writes here; freed (word b) receives the
+// arrival of the CTA before once it has read the halo row that this CTA wrote there.
+// JPhase counts the completed phases of each.
+struct JBars { unsigned full, freed; volatile int *dead; };   // [2] words of 8 bytes each
+struct JPhase { unsigned full0, full1, freed0, freed1; };
 
 template <typename Real, int NS, bool PROBE>
-__device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, cg::cluster_group &cluster, Real *ring,
-                                            Real *coef, Real *ibuf, Real *scratch, Real *sray, Real *sfreq,
-                                            int box, int m, int g, int rank, int C)
+__device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsigned sbase, const JSmem &sm,
+                                            const JBars &bars, JPhase &ph, const unsigned sray, int box, int m, int g,
+                                            int rank, int C)
 {
-    using V = typename V16<Real>::T;
-    using P2 = typename PairT<Real>::T;
+    using X = typename XOf<Real>::X;
     using W = JW<Real, NS>;
+    constexpr int XW = jsweep_lanes<Real>();
     constexpr int NA = W::na;
-    constexpr int CW = W::cw;
+    constexpr unsigned SZ = sizeof(Real);
+    constexpr unsigned CB = W::cw * 8;               // bytes of a node's coefficients and of a Stokes element
+                                                     // (NS = 4: of each of its two chunks)
+    constexpr int SCH = W::staged * (int)SZ / 16;    // 16-byte chunks of a voxel's packed inputs
     const BoxDev B = a.boxes[box];
-    const int nx = B.nx, ny = B.ny, nz = B.nz, F = a.F;
+    const int nx = B.nx, ny = B.ny, nz = B.nz, FX = (a.F + XW - 1) / XW;
     const int row0 = (int)(((long long)rank * ny) / C);
     const int R = (int)(((long long)(rank + 1) * ny) / C) - row0;
-    const int next_row = (row0 + R) % ny;
+    // the CTAs that own the sheared rows before and after this strip
+    const int prev_row = row0 == 0 ? ny - 1 : row0 - 1, next_row = (row0 + R) % ny;
+    const int prev_owner = (int)(((long long)(prev_row + 1) * C + ny - 1) / ny) - 1;
+    const int prev_R = prev_row + 1 - (int)(((long long)prev_owner * ny) / C);
     const int next_owner = (int)(((long long)(next_row + 1) * C + ny - 1) / ny) - 1;
-    const Real *ibuf_next = cluster.map_shared_rank(ibuf, next_owner);
-    const int j0 = g * F;
-    const int nf = min(F, a.nnu - j0);
+    // the pass's frequencies: the units of the grid split evenly over the groups
+    const int nunit = (a.nnu + XW - 1) / XW;
+    const int nper = nunit / a.ngroups, nextra = nunit - nper * a.ngroups;
+    const int j0 = XW * (g * nper + min(g, nextra));
+    const int nf = nper + (g < nextra ? 1 : 0);      // units
     const PlaneGeom<Real> *G = a.geom + B.geom0 + (long long)m * nz;
     const int tid = threadIdx.x, nt = blockDim.x;
     const int nodes = a.ring_plane;                  // node capacity of a ring slot
     const int nn = (R + 2) * nx;                     // nodes of this strip's slot
-    const int iplane = a.istride;                    // Reals per (buf, f) Stokes plane
-    const int cplane = a.cstride;                    // Reals per (slot, f) coefficient plane
     const int ipts = a.ipts_max;
     const int npts = R * nx;
     // voxel indices fit in 32 bits (porta_create limits nvox to 2^31)
     const int nvox = (int)a.nvox, vox0 = (int)B.vox0;
-    const Real *__restrict__ chi = a.chi, *__restrict__ vel = a.vel, *__restrict__ rho = a.rho;
     const Real *__restrict__ invn = a.invn + (long long)m * a.nvox;
+    const unsigned geo = sbase + sm.geo;             // plane q's PlaneGeom at q % 8
+    constexpr unsigned GB = sizeof(PlaneGeom<Real>);
+    // four words of the ray's constants (mu, ox, oy, oz | T[18], w, pad)
+    auto ray4 = [&](int i, Real *w) { lds4(sray + i * 4 * SZ, 16, w); };
+    constexpr int GW = (int)sizeof(PlaneGeom<Real>) / 4;
 
-    // the ray's constants and this pass's frequency nodes and weights, staged in
-    // shared memory (the previous item ended at a cluster barrier: no reader is left)
-    if (tid < 24) {
-        const Real *rp = reinterpret_cast<const Real *>(a.rays + m);
-        sray[tid] = rp[tid];                         // mu, ox, oy, oz, T[18], w, pad
+    // the pass's frequency nodes and weights (a last half-empty unit repeats its frequency
+    // with weight 0) and the first planes' geometry; later planes follow five ahead. (The
+    // previous item ended at a CTA barrier: no reader is left.)
+    for (int f = tid; f < nf * XW; f += nt) {
+        const bool in = j0 + f < a.nnu;
+        sts(sbase + sm.freq + f * SZ, a.xf[in ? j0 + f : a.nnu - 1]);
+        sts(sbase + sm.freq + (FX * XW + f) * SZ, in ? a.wf[j0 + f] : Real(0));
     }
-    for (int f = tid; f < nf; f += nt) {
-        sfreq[f] = a.xf[j0 + f];
-        sfreq[F + f] = a.wf[j0 + f];
-    }
+    for (int i = tid; i < GW * min(6, nz); i += nt) sts(geo + 4 * i, reinterpret_cast<const int *>(G)[i]);
     __syncthreads();
-    const Real mu = sray[0];
-    const bool upward = mu > Real(0);
 
-    // Frequency lanes: when the strip has fewer points than threads, L = 2 or 4
-    // adjacent threads share a point and take frequencies lane, lane + L, ...;
-    // their sums meet by warp shuffles in a fixed order.
-    const int lmax = npts > 0 ? min(nf, nt / npts) : 1;
-    const int L = lmax >= 4 ? 4 : (lmax >= 2 ? 2 : 1);
-    const int lane = tid & (L - 1);
-    const int pfirst = tid / L;
-    const int pstep = nt / L;
+    // Update threads: a point (or several in rounds) and every Lg-th unit of the pass from fg
+    // on; the threads of a group are whole warps. (The warp's index comes from a warp
+    // reduction so that the compiler knows that what follows from it is the same for all
+    // lanes and keeps it in uniform registers.)
+    const int pw = min(nt, (npts + 31) / 32 * 32);
+    const int wid = (int)__reduce_max_sync(0xffffffffu, (unsigned)tid >> 5);
+    const int Lg = npts > 0 ? min(nf, nt / pw) : 1;
+    const int fg = npts > 0 ? wid * 32 / pw : 0, ptid = tid - fg * pw;
+    const int p_own = min(ptid, max(npts - 1, 0)), l_own = p_own / nx, c_own = p_own - l_own * nx;
+    // the work beside the updates goes to the last threads first (where the units do not
+    // divide evenly, the last groups have one less)
+    const int rtid = nt - 1 - tid, rowt = rtid / nx, colt = rtid - rowt * nx;
     const int dl = nt / nx, dc = nt - dl * nx;
-    const int pl_ = pstep / nx, pc_ = pstep - pl_ * nx;
 
-    V *const ringv = reinterpret_cast<V *>(ring);
-    Real *const stage = scratch;
+    // voxel of point (l, c) of the strip in a plane (l = -1: the row before the strip)
+    auto point_voxel = [&](int q, int l, int c) {
+        const unsigned o = geo + (q & 7) * GB;
+        int ax, ay, kz;
+        lds(o, ax);
+        lds(o + 4, ay);
+        lds(o + 8, kz);
+        int pi = c + ax;
+        pi -= pi >= nx ? nx : 0;
+        int pj = row0 + l + ay;
+        pj += pj < 0 ? ny : 0;
+        pj -= pj >= ny ? ny : 0;
+        pj -= pj >= ny ? ny : 0;
+        return vox0 + (kz * ny + pj) * nx + pi;
+    };
 
-    // Stage plane q into ring slot q % 3: source vectors, then per-frequency (eta_I, eta_V).
-    auto fill = [&](int q) {
-        const PlaneGeom<Real> gq = G[q];
-        const int s = q % 3;
-        const int kbase = gq.kz * ny;
-        Real T[18], ox = 0, oy = 0, oz = 0;
-        if constexpr (NS == 4) {
+    // Inputs of plane q's nodes on their way to shared memory; the thread that asked for a
+    // node's values is the one that fills the node a phase later.
+    auto fetch = [&](int q) {
+        int lr = rowt, c = colt;
+        for (int idx = rtid; idx < nn; idx += nt) {
+            const int v = point_voxel(q, lr - 1, c);
+            const Real *src = a.pack + (size_t)(unsigned)v * W::staged;
+            const unsigned d = sbase + sm.stage + idx * 16;
+            sts(sbase + sm.stv + idx * 4, v);
+            copy_async(sbase + sm.stw + idx * SZ, invn + v);
+            if (a.jacc) copy_async(sbase + sm.ste + idx * 4, a.jexp + v);
 #pragma unroll
-            for (int i = 0; i < 18; ++i) T[i] = sray[4 + i];
-            ox = sray[1]; oy = sray[2]; oz = sray[3];
-        }
-        int lr = tid / nx, c = tid - (tid / nx) * nx;
-        for (int idx = tid; idx < nn; idx += nt) {
-            int pi = c + gq.ax;
-            pi -= pi >= nx ? nx : 0;
-            int pj = row0 + lr - 1 + gq.ay;
-            pj += pj < 0 ? ny : 0;
-            pj -= pj >= ny ? ny : 0;
-            pj -= pj >= ny ? ny : 0;
-            const int v = vox0 + (kbase + pj) * nx + pi;
-            stage[idx] = chi[v];
-            stage[nodes + idx] = vel[v] * mu;
-            if constexpr (NS == 1) {
-                ring[s * nodes + idx] = rho[v];
-            } else {
-                const Real s00 = rho[v], s20 = rho[nvox + v], s21r = rho[2 * nvox + v], s21i = rho[3 * nvox + v];
-                const Real s22r = rho[4 * nvox + v], s22i = rho[5 * nvox + v];
-                Real w[4];
-                // S_i(Omega) = sum_KQ (-1)^Q T^K_Q(i, Omega) S^K_-Q (Eq. 1 tensors, two-level emissivity)
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const Real *t = T + 6 * i;
-                    w[i] = t[0] * s00 + t[1] * s20 + Real(2) * (t[2] * s21r + t[3] * s21i) +
-                           Real(2) * (t[4] * s22r + t[5] * s22i);
-                }
-                w[3] = s00;
-#pragma unroll
-                for (int h = 0; h < W::s_chunks; ++h) chunk_put<Real>(ringv + (s * W::s_chunks + h) * nodes + idx, w + h * W::per);
-                stage[2 * nodes + idx] = a.bfac * (a.bx[v] * ox + a.by[v] * oy + a.bz[v] * oz);
-            }
+            for (int h = 0; h < SCH; ++h) copy_async16(d + h * nodes * 16, src + h * W::per);
             c += dc;
             lr += dl;
             if (c >= nx) { c -= nx; ++lr; }
         }
-        __syncthreads();
-        // per node its coefficients at every frequency of the pass (a warp writes
-        // consecutive nodes); when the slot has fewer nodes than threads, the
-        // frequencies are split between nt / nn thread groups
-        const int ngrp = max(1, min(nf, nt / nn));
-        const int grp = tid / nn;
-        for (int idx = tid - grp * nn; grp < ngrp && idx < nn; idx += nt) {
-            const Real chi_n = stage[idx], s_n = stage[nodes + idx];
-            Real b_n = 0;
-            if constexpr (NS == 4) b_n = stage[2 * nodes + idx];
-            Real *cp = coef + (s * F + grp) * cplane + idx * CW;
-            for (int f = grp; f < nf; f += ngrp, cp += ngrp * cplane) {
-                const Real xs = sfreq[f] - s_n;
-                const Real eta = chi_n * profile_shape(xs);
-                if constexpr (NS == 1) {
-                    cp[0] = eta;
-                } else {
-                    R2<Real> e2 = {eta, b_n * xs * eta};
-                    *reinterpret_cast<R2<Real> *>(cp) = e2;
+    };
+
+    // Plane q into ring slot q % 4: a thread takes a node, writes its source vector and its
+    // (eta_I, eta_V) at every unit of the pass.
+    auto fill = [&](int q) {
+        const unsigned s = q & 3;
+        copies_wait();
+        if (rtid >= nn) return;
+        Real o[4];
+        ray4(0, o);
+        for (int idx = rtid; idx < nn; idx += nt) {
+            Real d[W::staged];
+            const unsigned src = sbase + sm.stage + idx * 16;
+#pragma unroll
+            for (int h = 0; h < SCH; ++h) {
+                if constexpr (SZ == 4) lds4(src + h * nodes * 16, 0, d + 4 * h);
+                else lds2(src + h * nodes * 16, d[2 * h], d[2 * h + 1]);
+            }
+            const X chi_n = xset(d[0]), ns_n = xset(-d[1] * o[0]);
+            // weight of the node's frequency sums, 1 / (chi N) and, for the fixed-point sums,
+            // the ray's weight and the voxel's power of two
+            Real t[20];
+#pragma unroll
+            for (int i = 0; i < 5; ++i)
+                if (NS == 4 || i == 4) ray4(1 + i, t + 4 * i);
+            Real wn;
+            lds(sbase + sm.stw + idx * SZ, wn);
+            wn = quotient(wn, d[0]);
+            if (a.jacc) {
+                int ex;
+                lds(sbase + sm.ste + idx * 4, ex);
+                wn *= t[18] * pow2(Real(0), ex);
+            }
+            sts(sbase + sm.wgt + (s * nodes + idx) * SZ, wn);
+            int v;
+            lds(sbase + sm.stv + idx * 4, v);
+            sts(sbase + sm.vox + (s * nodes + idx) * 4, v);
+            unsigned oc = opaque(sbase + sm.coef + s * FX * sm.cplane + idx * CB), of = sbase + sm.freq;
+            if constexpr (NS == 1) {
+                sts(sbase + (s * nodes + idx) * SZ, d[2]);
+                for (int f = 0; f < nf; ++f, oc += sm.cplane, of += 8) {
+                    X x;
+                    lds(of, x);
+                    sts(oc, xmul(chi_n, xprofile(xadd(x, ns_n))));
+                }
+            } else {
+                const X b_n = xset(a.bfac * (d[8] * o[1] + d[9] * o[2] + d[10] * o[3]));
+                Real w[4];
+                // S_i(Omega) = sum_KQ (-1)^Q T^K_Q(i, Omega) S^K_-Q (Eq. 1 tensors, two-level emissivity)
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    w[i] = t[6 * i] * d[2] + t[6 * i + 1] * d[3] + Real(2) * (t[6 * i + 2] * d[4] + t[6 * i + 3] * d[5] +
+                                                                              t[6 * i + 4] * d[6] + t[6 * i + 5] * d[7]);
+                w[3] = d[2];
+                sts4(sbase + (s * W::s_chunks * nodes + idx) * 16, nodes * 16, w);
+                for (int f = 0; f < nf; ++f, oc += sm.cplane, of += 8) {
+                    X x;
+                    lds(of, x);
+                    const X xs = xadd(x, ns_n), eta = xmul(chi_n, xprofile(xs));
+                    sts2(oc, eta, xmul(xmul(b_n, xs), eta));
                 }
             }
         }
     };
 
-    // the fixed-point terms of a point's frequency-integrated Stokes parameters and
-    // Lambda* for this pass: J^K_Q += w_m sum_p T^K_Q(p, m) I_p, Lambda-bar* += w_m L
-    // (the ray's weight and tensors in the sweep's precision; FP32 terms convert
-    // to fixed point without rounding). The L frequency lanes of a point hold the
-    // same totals and share the terms: lane k adds the components c = k mod L.
-    auto add_terms = [&](int v, const Real *tot) {
-        const Real scale = pow2(Real(0), a.jexp[v]);
-        const Real w = sray[22];
-        unsigned long long *acc = a.jacc + v;
-        if constexpr (NS == 1) {
-            if (lane == 0) jadd(acc, w * tot[0] * scale, a.jerr);
-            if (lane == (L > 1 ? 1 : 0)) jadd(acc + nvox, w * tot[1] * scale, a.jerr);
-        } else {
-            const Real pI = w * tot[0] * scale, pQ = w * tot[1] * scale, pU = w * tot[2] * scale;
-            for (int k = lane; k < 6; k += L)
-                jadd(acc + (size_t)k * nvox, sray[4 + k] * pI + sray[10 + k] * pQ + sray[16 + k] * pU, a.jerr);
-            if (lane == 6 % L) jadd(acc + (size_t)6 * nvox, w * tot[3] * scale, a.jerr);
+    // A point's sums over the pass, times its node's weight: the fixed-point terms J^K_Q +=
+    // w_m sum_p T^K_Q(p, m) I_p, Lambda-bar* += w_m L, or the per-ray partials (FP64).
+    auto add_point = [&](unsigned n, const Real *sum) {
+        Real wn, t[4] = {0, 0, 0, 0};
+        int v;
+        lds(sbase + sm.wgt + n * SZ, wn);
+        lds(sbase + sm.vox + n * 4, v);
+#pragma unroll
+        for (int s = 0; s < NA; ++s) t[s] = sum[s] * wn;
+        if (!a.jacc) {
+            store_partial<Real, NS>(a, m, v, g, t);
+            return;
+        }
+        if constexpr (SZ == 4) {
+            bool bad = false;
+            unsigned long long *acc = a.jacc + v;
+            if constexpr (NS == 1) {
+                bad |= jadd(acc, t[0]);
+                bad |= jadd(acc + nvox, t[1]);
+            } else {
+                Real T[20];
+#pragma unroll
+                for (int i = 0; i < 5; ++i) ray4(1 + i, T + 4 * i);
+#pragma unroll
+                for (int k = 0; k < 6; ++k, acc += nvox)
+                    bad |= jadd(acc, T[k] * t[0] + T[6 + k] * t[1] + T[12 + k] * t[2]);
+                bad |= jadd(acc, t[3]);
+            }
+            if (bad) atomicOr(a.jerr, 1);
+        }
+    };
+    // the same from the totals of several groups of threads (written a phase before)
+    auto add_totals = [&](int q) {
+        for (int p = rtid; p < npts; p += nt) {
+            Real t[4] = {0, 0, 0, 0};
+            for (int h = 0; h < Lg; ++h) {
+                Real w[4] = {0, 0, 0, 0};
+                const unsigned o = sbase + sm.tot + ((q & 1) * a.tots + h * pw + p) * NA * SZ;
+                if constexpr (NS == 1) {
+                    lds(o, w[0]);
+                    lds(o + SZ, w[1]);
+                } else {
+                    lds4(o, 16, w);
+                }
+#pragma unroll
+                for (int s = 0; s < NA; ++s) t[s] += w[s];
+            }
+            add_point((q & 3) * nodes + p + nx, t);
         }
     };
 
-    fill(0);
-    __syncthreads();
-    if (nz > 1) fill(1);
-    __syncthreads();
-    for (int q = 0; q < nz; ++q) {
-        const PlaneGeom<Real> gq = G[q];
-        const bool has_p = q + 1 < nz;
-        const PlaneGeom<Real> gp = has_p ? G[q + 1] : gq;
-        const int sM = (q + 2) % 3, sO = q % 3, sP = (q + 1) % 3;
-        Real *iw = ibuf + (q & 1) * F * iplane;
-        const int ro = ((q + 1) & 1) * F * iplane;
-        const Real *ir = ibuf + ro;
-        const Real *irn = ibuf_next + ro;
-        const Real mx1 = gq.tx, mx0 = Real(1) - gq.tx, my1 = gq.ty, my0 = Real(1) - gq.ty;
-        const Real px0 = gp.tx, px1 = Real(1) - gp.tx, py0 = gp.ty, py1 = Real(1) - gp.ty;
-        const Real dsM = Real(0.5) * gq.ds, dsP = has_p ? Real(0.5) * gp.ds : Real(0);
-        const Real wM[4] = {mx0 * my0, mx1 * my0, mx0 * my1, mx1 * my1};
-        const Real wP[4] = {px0 * py0, px1 * py0, px0 * py1, px1 * py1};
-        // the weights as pairs (both lanes equal), for the pair arithmetic
-        P2 wM2[4], wP2[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            wM2[k] = pmk(wM[k], wM[k]);
-            wP2[k] = pmk(wP[k], wP[k]);
+    // A point's frequency integral over the thread's units
+    auto totals = [&](int q, int p, const Real *acc) {
+        if (Lg == 1) {
+            add_point((q & 3) * nodes + p + nx, acc);
+            return;
         }
-        const Real *cMb = coef + sM * F * cplane, *cPb = coef + sP * F * cplane;
-        const V *rMb = ringv + sM * W::s_chunks * nodes, *rOb = ringv + sO * W::s_chunks * nodes;
-        const V *rPb = ringv + sP * W::s_chunks * nodes;
+        const unsigned o = sbase + sm.tot + ((q & 1) * a.tots + fg * pw + p) * NA * SZ;
+        if constexpr (NS == 1) {
+            sts(o, acc[0]);
+            sts(o + SZ, acc[1]);
+        } else {
+            sts4(o, 16, acc);
+        }
+    };
 
-        Real acc[NA], accp[NA];
-        bool pend = false, row0_written = false;
-        int vpend = 0;
-        int l = pfirst / nx, c = pfirst - (pfirst / nx) * nx;
-        // every warp takes the same number of point rounds (the lane shuffles below)
-        for (int pb = 0; pb < npts; pb += pstep) {
-            const int p = pb + pfirst;
-            if (pb > 0) {
-                c += pc_;
-                l += pl_;
-                if (c >= nx) { c -= nx; ++l; }
+    // The work of phase q beside the update of plane q: the nodes of plane q + 2, the sums
+    // of plane q - 1, and the inputs of later planes.
+    auto aside = [&](int q) {
+        if (q + 2 < nz) {
+            fill(q + 2);
+            if (q + 3 < nz) fetch(q + 3);
+            if (q + 5 < nz && tid < GW)
+                copy_async(geo + ((q + 5) & 7) * GB + 4 * tid, reinterpret_cast<const int *>(G + q + 5) + tid);
+        }
+        if (Lg > 1 && q >= 1) add_totals(q - 1);
+    };
+
+    // One plane of updates (q >= 1). The bilinear weights are used relative to the first
+    // one, v_M = w_M (v_00 + u_x v_01 + u_y v_10 + u_x u_y v_11), u = t / (1 - t): w_M cancels
+    // in S = eps / eta; those of P are the next plane's. A corner's address is its node's offset, fixed for the sweep, plus a
+    // base that is the same for all threads (array, slot, unit). The order of the steps and
+    // what is held (the upwind corners' weighted sources; the downwind ones are read again
+    // for every unit) keep an FP32 thread within 128 registers: a spilled value would come
+    // back from L2, the halo waits' acquire invalidating L1.
+    const unsigned ibuf_prev = map_rank(sbase + sm.ibuf, prev_owner);
+    const unsigned full_prev = map_rank(bars.full, prev_owner);
+    const unsigned row = nx * CB;
+    const unsigned chS = nodes * 16, chI = ipts * 16;    // second 16-byte chunks: source (FP64), Stokes
+    auto points = [&](auto HASP, int q) {
+        constexpr bool has_p = decltype(HASP)::value;
+        const unsigned pC = FX * sm.cplane, pS = W::s_words * nodes * SZ, pI = FX * sm.iplane;
+        const unsigned stepC = Lg * sm.cplane, stepI = Lg * sm.iplane;
+        const int bI = (q + 1) & 1, bW = q & 1;
+        const unsigned opc = geo + (q & 7) * GB + 16, opp = geo + ((q + 1) & 7) * GB + 16;   // ux, uy, wM, dsM
+        for (int pb = 0; pb < npts && fg < Lg; pb += pw) {
+            // lanes beyond the last point repeat it without storing
+            const bool active = pb + ptid < npts;
+            const int p = min(pb + ptid, npts - 1);
+            const int l = pb == 0 ? l_own : p / nx, c = pb == 0 ? c_own : p - l * nx;
+            if (C > 1) {
+                // the row after the strip's last one comes from the next CTA; the halo row of
+                // this parity was read by the CTA before in its last phase
+                if (l + 1 == R) bar_wait(bars.full + 8 * bI, ((bI ? ph.full1 : ph.full0) + (unsigned)((q - 1) >> 1)) & 1u, bars.dead, a.jerr);
+                if (l == 0 && has_p && q >= 2)
+                    bar_wait(bars.freed + 8 * bW, ((bW ? ph.freed1 : ph.freed0) + (unsigned)((q >> 1) - 1)) & 1u, bars.dead, a.jerr);
             }
-            const bool active = p < npts;
-            row0_written |= active && l == 0;
+            // node offsets (a node's coefficients, a Stokes element and, for NS = 4, a source
+            // chunk have one size): row before, own row, row after; column before, own, after
+            const unsigned n11 = opaque((p + nx) * CB);
+            const unsigned n12 = opaque(n11 + (c + 1 == nx ? (unsigned)(1 - nx) : 1u) * CB);
+            const unsigned n10 = opaque(n11 + (c == 0 ? (unsigned)(nx - 1) : (unsigned)-1) * CB);
+            const unsigned n21 = opaque(n11 + row), n22 = opaque(n12 + row), n01 = opaque(n11 - row), n00 = opaque(n10 - row);
+            const unsigned uS_M = sbase + ((q + 3) & 3) * pS, uS_O = sbase + (q & 3) * pS, uS_P = sbase + ((q + 1) & 3) * pS;
+            const unsigned c0 = sbase + sm.coef + fg * sm.cplane, i0 = sbase + sm.ibuf + fg * sm.iplane - row;
+            unsigned uM = c0 + ((q + 3) & 3) * pC, uO = c0 + (q & 3) * pC, uP = c0 + ((q + 1) & 3) * pC;
+            unsigned uI = i0 + bI * pI, uW = i0 + bW * pI;
+            unsigned of = sbase + sm.freq + FX * XW * SZ + fg * 8;
+            const bool row0 = l == 0 && has_p && active && !(C > 1 && *bars.dead);
+            // halo row of the strip before: row prev_R of its Stokes planes
+            const unsigned hcol = (prev_R * nx + c) * CB;
+            unsigned uH = bW * pI + fg * sm.iplane;
+            Real acc[NA];
 #pragma unroll
             for (int s = 0; s < NA; ++s) acc[s] = Real(0);
-            int v = 0;
-            if (active) {
-                int pi = c + gq.ax;
-                pi -= pi >= nx ? nx : 0;
-                int pj = row0 + l + gq.ay;
-                pj -= pj >= ny ? ny : 0;
-                pj -= pj >= ny ? ny : 0;
-                v = vox0 + (gq.kz * ny + pj) * nx + pi;
-                // the point's own data: source vector from the ring, the rest from global memory
-                const int io = (l + 1) * nx + c;
-                Real SO[NS];
+            // the corners' source vectors (NS = 4: I, Q, U and the S^0_0 that eta_V multiplies)
+            auto source = [&](unsigned u, unsigned n, Real *r) {
+                if constexpr (NS == 1) lds(u + n / CB * SZ, r[0]);
+                else lds4(u + n, chS, r);
+            };
+            Real m0[NS], m1[NS], m2[NS], m3[NS], SO[NS];
+            source(uS_M, n11, m0); source(uS_M, n12, m1); source(uS_M, n21, m2); source(uS_M, n22, m3);
+            source(uS_O, n11, SO);
+            {
+                Real pm[4];
+                lds4(opc, 16, pm);
+                const Real uxy = pm[0] * pm[1];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) { m1[s] *= pm[0]; m2[s] *= pm[1]; m3[s] *= uxy; }
+            }
+            Real p0 = 0, p1 = 0, p2 = 0, p3 = 0;             // NS = 1: the downwind sources
+            if constexpr (NS == 1 && has_p) {
+                source(uS_P, n11, &p0); source(uS_P, n10, &p1); source(uS_P, n01, &p2); source(uS_P, n00, &p3);
+            }
+#pragma unroll 1
+            for (int f = fg; f < nf; f += Lg) {
+                Real pm[4];                                  // ux, uy, wM, dsM
+                lds4(opc, 16, pm);
+                const Real ux = pm[0], uy = pm[1], uxy = ux * uy, wM = pm[2], dsM = pm[3];
+                // a2-a3: transfer coefficients at M, d_M = S_O - eps_M / eta_M, -K'_V at O and M
+                X eO, nkM, nkO, S3, eM, dm[NS];
+                {
+                    X e[NS], k, kM;
+                    if constexpr (NS == 1) {
+                        lds(n11 + uO, eO);
+                        lds(n11 + uM, k);
+                        eM = k; e[0] = xms(m0[0], k);
+                        lds(n12 + uM, k);
+                        eM = xfs(ux, k, eM); e[0] = xfs(m1[0], k, e[0]);
+                        lds(n21 + uM, k);
+                        eM = xfs(uy, k, eM); e[0] = xfs(m2[0], k, e[0]);
+                        lds(n22 + uM, k);
+                        eM = xfs(uxy, k, eM); e[0] = xfs(m3[0], k, e[0]);
+                    } else {
+                        X vO, h;
+                        lds2(n11 + uO, eO, vO);
+                        nkO = xmul(vO, xnrcp(eO));
+                        S3 = xms(-SO[NS - 1], nkO);
+                        lds2(n11 + uM, k, h);
+                        eM = k; kM = h;
+                        e[0] = xms(m0[0], k); e[1] = xms(m0[1], k); e[2] = xms(m0[2], k); e[3] = xms(m0[3], h);
+                        lds2(n12 + uM, k, h);
+                        eM = xfs(ux, k, eM); kM = xfs(ux, h, kM);
+                        e[0] = xfs(m1[0], k, e[0]); e[1] = xfs(m1[1], k, e[1]); e[2] = xfs(m1[2], k, e[2]); e[3] = xfs(m1[3], h, e[3]);
+                        lds2(n21 + uM, k, h);
+                        eM = xfs(uy, k, eM); kM = xfs(uy, h, kM);
+                        e[0] = xfs(m2[0], k, e[0]); e[1] = xfs(m2[1], k, e[1]); e[2] = xfs(m2[2], k, e[2]); e[3] = xfs(m2[3], h, e[3]);
+                        lds2(n22 + uM, k, h);
+                        eM = xfs(uxy, k, eM); kM = xfs(uxy, h, kM);
+                        e[0] = xfs(m3[0], k, e[0]); e[1] = xfs(m3[1], k, e[1]); e[2] = xfs(m3[2], k, e[2]); e[3] = xfs(m3[3], h, e[3]);
+                    }
+                    const X niM = xnrcp(eM);
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) dm[s] = xfma(e[s], niM, NS == 4 && s == 3 ? S3 : xset(SO[s]));
+                    if constexpr (NS == 4) nkM = xmul(kM, niM);
+                }
+                // a4, a6: optical path and coefficients of the step
+                const X tMO = xms(dsM, xfs(wM, eM, eO));
+                const XCoef<X> co = xcoef(tMO);
+                const X ls = has_p ? xadd(co.wo, co.wc) : xfs(Real(0.5), co.wc, co.wo);
+                // a7: right-hand side of Eq. 7, e I_M + (w_M + w_O + w_C) S_O - w_M d_M - w_C (S_O - c_M),
+                // with the upwind Stokes vector over w_M (a3) and K'_V at M coupling I and V
+                X r[NS];
+                {
+                    const X wsum = xadd(xadd(co.wm, co.wo), co.wc), ew = xms(wM, co.e);
+                    // without a downwind point c_M = (S_M + S_O) / 2
+                    const X nwm = has_p ? xneg(co.wm) : xfs(Real(-0.5), co.wc, xneg(co.wm));
+#pragma unroll
+                    for (int s = 0; s < NS; ++s)
+                        r[s] = xfma(nwm, dm[s], NS == 4 && s == 3 ? xmul(wsum, S3) : xms(SO[s], wsum));
+                    if constexpr (NS == 1) {
+                        X t, u;
+                        lds(n11 + uI, t);
+                        lds(n12 + uI, u);
+                        t = xfs(ux, u, t);
+                        lds(n21 + uI, u);
+                        t = xfs(uy, u, t);
+                        lds(n22 + uI, u);
+                        r[0] = xfma(ew, xfs(uxy, u, t), r[0]);
+                    } else {
+                        X t0, t1, t2, t3, u0, u1;
+                        lds2(n11 + uI, t0, t1);
+                        lds2(n12 + uI, u0, u1);
+                        t0 = xfs(ux, u0, t0); t1 = xfs(ux, u1, t1);
+                        lds2(n21 + uI, u0, u1);
+                        t0 = xfs(uy, u0, t0); t1 = xfs(uy, u1, t1);
+                        lds2(n22 + uI, u0, u1);
+                        t0 = xfs(uxy, u0, t0); t1 = xfs(uxy, u1, t1);
+                        lds2(n11 + uI + chI, t2, t3);
+                        lds2(n12 + uI + chI, u0, u1);
+                        t2 = xfs(ux, u0, t2); t3 = xfs(ux, u1, t3);
+                        lds2(n21 + uI + chI, u0, u1);
+                        t2 = xfs(uy, u0, t2); t3 = xfs(uy, u1, t3);
+                        lds2(n22 + uI + chI, u0, u1);
+                        t2 = xfs(uxy, u0, t2); t3 = xfs(uxy, u1, t3);
+                        const X pk = xmul(xms(wM, xfs(Real(0.5), co.wc, co.wm)), nkM);
+                        r[0] = xfma(pk, t3, xfma(ew, t0, r[0]));
+                        r[1] = xfma(ew, t1, r[1]);
+                        r[2] = xfma(ew, t2, r[2]);
+                        r[3] = xfma(pk, t0, xfma(ew, t3, r[3]));
+                    }
+                }
+                if constexpr (has_p) {
+                    // downwind: -d_P = S_O - eps_P / eta_P
+                    Real pp[4];                              // vx, vy, wP, dsP
+                    lds4(opp, 16, pp);
+                    const Real vx = pp[0], vy = pp[1], vxy = vx * vy, wP = pp[2], dsP = pp[3];
+                    X eP, e[NS];
+                    if constexpr (NS == 1) {
+                        X k;
+                        lds(n11 + uP, k);
+                        eP = k; e[0] = xms(p0, k);
+                        lds(n10 + uP, k);
+                        k = xms(vx, k); eP = xadd(eP, k); e[0] = xfs(p1, k, e[0]);
+                        lds(n01 + uP, k);
+                        k = xms(vy, k); eP = xadd(eP, k); e[0] = xfs(p2, k, e[0]);
+                        lds(n00 + uP, k);
+                        k = xms(vxy, k); eP = xadd(eP, k); e[0] = xfs(p3, k, e[0]);
+                    } else {
+                        X k, h;
+                        Real w[4];
+                        lds2(n11 + uP, k, h);
+                        lds4(uS_P + n11, chS, w);
+                        eP = k;
+                        e[0] = xms(w[0], k); e[1] = xms(w[1], k); e[2] = xms(w[2], k); e[3] = xms(w[3], h);
+                        lds2(n10 + uP, k, h);
+                        lds4(uS_P + n10, chS, w);
+                        k = xms(vx, k); h = xms(vx, h); eP = xadd(eP, k);
+                        e[0] = xfs(w[0], k, e[0]); e[1] = xfs(w[1], k, e[1]); e[2] = xfs(w[2], k, e[2]); e[3] = xfs(w[3], h, e[3]);
+                        lds2(n01 + uP, k, h);
+                        lds4(uS_P + n01, chS, w);
+                        k = xms(vy, k); h = xms(vy, h); eP = xadd(eP, k);
+                        e[0] = xfs(w[0], k, e[0]); e[1] = xfs(w[1], k, e[1]); e[2] = xfs(w[2], k, e[2]); e[3] = xfs(w[3], h, e[3]);
+                        lds2(n00 + uP, k, h);
+                        lds4(uS_P + n00, chS, w);
+                        k = xms(vxy, k); h = xms(vxy, h); eP = xadd(eP, k);
+                        e[0] = xfs(w[0], k, e[0]); e[1] = xfs(w[1], k, e[1]); e[2] = xfs(w[2], k, e[2]); e[3] = xfs(w[3], h, e[3]);
+                    }
+                    const X niP = xnrcp(eP);
+                    const X tOP = xms(dsP, xfs(wP, eP, eO));
+                    // a5: BESSER control points per Stokes parameter
+                    const X hh = xms(Real(0.5), xrcp(xadd(tMO, tOP))), nr = xmul(tMO, xnrcp(tOP));
+                    const X na = xmul(xmul(tMO, hh), nr), gb = xmul(tOP, hh), nwc = xneg(co.wc);
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        const X ndp = xfma(e[s], niP, NS == 4 && s == 3 ? S3 : xset(SO[s]));
+                        r[s] = xfma(nwc, xoffset(dm[s], ndp, na, gb, nr), r[s]);
+                    }
+                }
+                if constexpr (NS == 4) {
+                    // kappa^-1 = 1 + psi'_O K'_O (Eq. 8) couples I and V only; psi' = w + w_C / 2
+                    const X nav = xmul(xfs(Real(0.5), co.wc, co.wo), nkO);
+                    const X idet = xrcp(xdet(nav));
+                    const X i = r[0];
+                    r[0] = xmul(xfma(nav, r[3], i), idet);
+                    r[3] = xmul(xfma(nav, i, r[3]), idet);
+                }
+                if (active) {
+                    if constexpr (NS == 1) {
+                        sts(n11 + uW, r[0]);
+                    } else {
+                        sts2(n11 + uW, r[0], r[1]);
+                        sts2(n11 + uW + chI, r[2], r[3]);
+                    }
+                }
+                if (row0) {
+                    if (C > 1) {
+                        const unsigned d = ibuf_prev + hcol + uH, b = full_prev + 8 * bW;
+                        if constexpr (NS == 1) {
+                            push(d, b, r[0]);
+                        } else {
+                            push2(d, b, r[0], r[1]);
+                            push2(d + chI, b, r[2], r[3]);
+                        }
+                    } else {
+                        const unsigned d = sbase + sm.ibuf + hcol + uH;
+                        if constexpr (NS == 1) {
+                            sts(d, r[0]);
+                        } else {
+                            sts2(d, r[0], r[1]);
+                            sts2(d + chI, r[2], r[3]);
+                        }
+                    }
+                }
+                // a8: Lambda* and frequency integration (w_nu phi / N = w_nu eta_I / (chi N))
+                X wt;
+                lds(of, wt);
+                wt = xmul(wt, eO);
+#pragma unroll
+                for (int s = 0; s < NA - 1; ++s) acc[s] = xdot(wt, r[s], acc[s]);
+                acc[NA - 1] = xdot(wt, ls, acc[NA - 1]);
+                if (PROBE && a.probe_ray == m && active) {
+                    const int v = point_voxel(q, l, c);
+                    for (int w = 0; w < XW && j0 + f * XW + w < a.nnu; ++w) {
+                        const long long pv = (long long)(j0 + f * XW + w) * a.nvox + v;
+#pragma unroll
+                        for (int s = 0; s < NS; ++s) a.probe[pv * NS + s] = xlane(r[s], w);
+                        a.probe_ls[pv] = xlane(ls, w);
+                    }
+                }
+                uM += stepC; uO += stepC; uP += stepC; uI += stepI; uW += stepI; uH += stepI; of += Lg * 8;
+            }
+            if (active) totals(q, p, acc);
+        }
+    };
+
+    // boundary plane: I = (B, 0, 0, 0) entering at the bottom, 0 at the top; Lambda* = 0
+    auto boundary = [&]() {
+        Real mu;
+        lds(sray, mu);
+        const bool upward = mu > Real(0);
+        for (int p = ptid; p < npts && fg < Lg; p += pw) {
+            const int l = p / nx, c = p - l * nx;
+            const int v = point_voxel(0, l, c);
+            const X zero = xset(Real(0)), I0 = xset(upward ? a.bpl[v] : Real(0));
+            Real acc[NA];
+#pragma unroll
+            for (int s = 0; s < NA; ++s) acc[s] = Real(0);
+            for (int f = fg; f < nf; f += Lg) {
+                const unsigned o = sbase + sm.ibuf + f * sm.iplane + p * CB, h = f * sm.iplane + (prev_R * nx + c) * CB;
                 if constexpr (NS == 1) {
-                    SO[0] = ring[sO * nodes + io];
-                } else {
-#pragma unroll
-                    for (int h = 0; h < W::s_chunks; ++h) chunk_get<Real>(rOb + h * nodes + io, SO + h * W::per);
-                }
-                const Real chiO = chi[v], sO_ = vel[v] * mu, invnO = invn[v];
-                Real bO = 0;
-                if constexpr (NS == 4) bO = a.bfac * (a.bx[v] * sray[1] + a.by[v] * sray[2] + a.bz[v] * sray[3]);
-
-                if (q == 0) {
-                    // boundary plane: I = (B, 0, 0, 0) entering at the bottom, 0 at the top; Lambda* = 0
-                    Real I0[NS];
-#pragma unroll
-                    for (int s = 0; s < NS; ++s) I0[s] = Real(0);
-                    if (upward) I0[0] = a.bpl[v];
-                    for (int f = lane; f < nf; f += L) {
-                        StokesIO<Real, NS>::store(iw + f * iplane, ipts, l * nx + c, I0);
-                        const Real wt = sfreq[F + f] * profile_shape(sfreq[f] - sO_) * invnO;
-                        acc[0] += wt * I0[0];
-                        if (PROBE && a.probe_ray == m) {
-                            const int j = j0 + f;
-#pragma unroll
-                            for (int s = 0; s < NS; ++s) a.probe[((long long)j * a.nvox + v) * NS + s] = I0[s];
-                            a.probe_ls[(long long)j * a.nvox + v] = Real(0);
-                        }
+                    sts(o, I0);
+                    if (l == 0) {
+                        if (C > 1) push(ibuf_prev + h, full_prev, I0);
+                        else sts(sbase + sm.ibuf + h, I0);
                     }
                 } else {
-                    const int c1 = (c + 1 == nx) ? 0 : c + 1;
-                    const int cm = (c == 0) ? nx - 1 : c - 1;
-                    const int rM[4] = {(l + 1) * nx + c, (l + 1) * nx + c1, (l + 2) * nx + c, (l + 2) * nx + c1};
-                    const int rP[4] = {l * nx + cm, l * nx + c, (l + 1) * nx + cm, (l + 1) * nx + c};
-                    // upwind corners' source vectors times their bilinear weights, held
-                    // across the frequency loop (the downwind corners' sources are read
-                    // again for each frequency: holding both spills at the register cap)
-                    Real SMk[4][W::s_words];
-                    P2 A01[4], A23[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if constexpr (NS == 1) {
-                            SMk[k][0] = wM[k] * ring[sM * nodes + rM[k]];
+                    sts2(o, I0, zero);
+                    sts2(o + chI, zero, zero);
+                    if (l == 0) {
+                        if (C > 1) {
+                            push2(ibuf_prev + h, full_prev, I0, zero);
+                            push2(ibuf_prev + h + chI, full_prev, zero, zero);
                         } else {
-#pragma unroll
-                            for (int h = 0; h < W::s_chunks; ++h) chunk_get<Real>(rMb + h * nodes + rM[k], SMk[k] + h * W::per);
-                            A01[k] = pmul(wM2[k], pmk(SMk[k][0], SMk[k][1]));
-                            A23[k] = pmul(wM2[k], pmk(SMk[k][2], SMk[k][3]));
-                        }
-                    }
-                    const bool last_row = (l + 1 == R);
-                    const int ilo = l * nx;
-                    const Real *ihi_base = last_row ? irn : ir;
-                    const int ihi = last_row ? 0 : (l + 1) * nx;
-
-                    for (int f = lane; f < nf; f += L) {
-                        const Real x = sfreq[f];
-                        const Real *pl = ir + f * iplane;
-                        const Real *ph = ihi_base + f * iplane;
-                        const Real *cM = cMb + f * cplane;
-                        const Real *cP = cPb + f * cplane;
-                        // the point O: its own profile (optical paths, Lambda*, integration weight)
-                        const Real xsO = x - sO_;
-                        const Real phO = profile_shape(xsO);
-                        const Real etaO = chiO * phO;
-                        if constexpr (NS == 1) {
-                            // a3: upwind intensity and transfer coefficients at M and P (bilinear)
-                            const Real IM = wM[0] * pl[ilo + c] + wM[1] * pl[ilo + c1] + wM[2] * ph[ihi + c] +
-                                            wM[3] * ph[ihi + c1];
-                            Real etaM = 0, epsM = 0, etaP = 0, epsP = 0;
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                const Real ek = cM[rM[k]];
-                                etaM += wM[k] * ek;
-                                epsM += SMk[k][0] * ek;           // (w S)_k eta_k
-                            }
-                            if (has_p) {
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    const Real we = wP[k] * cP[rP[k]];
-                                    etaP += we;
-                                    epsP += we * ring[sP * nodes + rP[k]];
-                                }
-                            }
-                            const Real SM = epsM * rcp(etaM), SOs = SO[0];
-                            const Real tMO = (etaM + etaO) * dsM;
-                            const Coef<Real> co = coefficients(tMO);
-                            Real cMs, SP = 0;
-                            if (has_p) {
-                                SP = epsP * rcp(etaP);
-                                const Real tOP = (etaO + etaP) * dsP;
-                                cMs = control_point(SM, SOs, SP, besser_geom(tMO, tOP));
-                            } else {
-                                cMs = Real(0.5) * (SM + SOs);
-                            }
-                            const Real IO = co.e * IM + co.wm * SM + co.wo * SOs + co.wc * cMs;
-                            iw[f * iplane + l * nx + c] = IO;
-                            const Real ls = co.wo + (has_p ? co.wc : Real(0.5) * co.wc);
-                            const Real wt = sfreq[F + f] * phO * invnO;
-                            acc[0] += wt * IO;
-                            acc[1] += wt * ls;
-                            if (PROBE && a.probe_ray == m) {
-                                const int j = j0 + f;
-                                a.probe[(long long)j * a.nvox + v] = IO;
-                                a.probe_ls[(long long)j * a.nvox + v] = ls;
-                            }
-                        } else {
-                            // a3: upwind Stokes vector (bilinear), as the pairs (I, Q), (U, V)
-                            P2 IM01, IM23;
-                            {
-                                Real t[4][4];
-                                StokesIO<Real, 4>::load(pl, ipts, ilo + c, t[0]);
-                                StokesIO<Real, 4>::load(pl, ipts, ilo + c1, t[1]);
-                                // the row after the strip's last is the next CTA's row 0 (DSMEM, a
-                                // generic load); the others are local (shared-memory loads)
-                                if (last_row) {
-                                    StokesIO<Real, 4>::load(ph, ipts, c, t[2]);
-                                    StokesIO<Real, 4>::load(ph, ipts, c1, t[3]);
-                                } else {
-                                    StokesIO<Real, 4>::load(pl, ipts, ilo + nx + c, t[2]);
-                                    StokesIO<Real, 4>::load(pl, ipts, ilo + nx + c1, t[3]);
-                                }
-                                IM01 = pmul(wM2[0], pmk(t[0][0], t[0][1]));
-                                IM23 = pmul(wM2[0], pmk(t[0][2], t[0][3]));
-#pragma unroll
-                                for (int k = 1; k < 4; ++k) {
-                                    IM01 = pfma(wM2[k], pmk(t[k][0], t[k][1]), IM01);
-                                    IM23 = pfma(wM2[k], pmk(t[k][2], t[k][3]), IM23);
-                                }
-                            }
-                            // a2-a3: transfer coefficients at M and P from the corners' (eta_I, eta_V):
-                            // (eta, eta_V) += w (eta_k, eta_V,k); (eps_I, eps_Q) += eta_k w (S_I, S_Q)_k;
-                            // (eps_U, eps_V) += (eta_k, eta_V,k) w (S_U, S^0_0)_k
-                            P2 eM = pmk(Real(0), Real(0)), eM01 = eM, eM23 = eM;
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                const P2 e2 = reinterpret_cast<const P2 *>(cM)[rM[k]];
-                                eM = pfma(wM2[k], e2, eM);
-                                eM01 = pfma(A01[k], pmk(e2.x, e2.x), eM01);
-                                eM23 = pfma(A23[k], e2, eM23);
-                            }
-                            P2 eP = pmk(Real(0), Real(0)), eP01 = eP, eP23 = eP;
-                            if (has_p) {
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) {
-                                    Real sp[4];
-#pragma unroll
-                                    for (int h = 0; h < W::s_chunks; ++h) chunk_get<Real>(rPb + h * nodes + rP[k], sp + h * W::per);
-                                    const P2 e2 = reinterpret_cast<const P2 *>(cP)[rP[k]];
-                                    const P2 wk = pmul(wP2[k], e2);
-                                    eP = padd(eP, wk);
-                                    eP01 = pfma(pmk(wk.x, wk.x), pmk(sp[0], sp[1]), eP01);
-                                    eP23 = pfma(wk, pmk(sp[2], sp[3]), eP23);
-                                }
-                            }
-                            const Real kvO = bO * xsO;
-                            const P2 SO01 = pmk(SO[0], SO[1]), SO23 = pmk(SO[2], kvO * SO[3]);
-                            const Real iM = rcp(eM.x);
-                            const P2 SM01 = pmul(eM01, pmk(iM, iM)), SM23 = pmul(eM23, pmk(iM, iM));
-                            // a4: optical paths (trapezoid along MO and OP)
-                            const Real tMO = (eM.x + etaO) * dsM;
-                            // a6: exponential-integral coefficients (Eqs. 9-13)
-                            const Coef<Real> co = coefficients(tMO);
-                            // a5: BESSER control points per Stokes parameter
-                            P2 cM01, cM23;
-                            if (has_p) {
-                                const Real iP = rcp(eP.x);
-                                const P2 SP01 = pmul(eP01, pmk(iP, iP)), SP23 = pmul(eP23, pmk(iP, iP));
-                                const Real tOP = (etaO + eP.x) * dsP;
-                                const BesserGeom<Real> bg = besser_geom(tMO, tOP);
-                                cM01 = control_point2(SM01, SO01, SP01, bg);
-                                cM23 = control_point2(SM23, SO23, SP23, bg);
-                            } else {
-                                cM01 = pmul(pmk(Real(0.5), Real(0.5)), padd(SM01, SO01));
-                                cM23 = pmul(pmk(Real(0.5), Real(0.5)), padd(SM23, SO23));
-                            }
-                            // a7: BESSER-DELO step (Eq. 7); kappa^-1 = 1 + psi'_O K'_O (Eq. 8)
-                            // couples I and V only
-                            P2 r01 = pmul(pmk(co.e, co.e), IM01), r23 = pmul(pmk(co.e, co.e), IM23);
-                            r01 = pfma(pmk(co.wm, co.wm), SM01, r01);
-                            r23 = pfma(pmk(co.wm, co.wm), SM23, r23);
-                            r01 = pfma(pmk(co.wo, co.wo), SO01, r01);
-                            r23 = pfma(pmk(co.wo, co.wo), SO23, r23);
-                            r01 = pfma(pmk(co.wc, co.wc), cM01, r01);
-                            r23 = pfma(pmk(co.wc, co.wc), cM23, r23);
-                            const Real kvM = eM.y * iM;
-                            const Real pk = co.pm * kvM;
-                            const Real rI = r01.x - pk * IM23.y, rV = r23.y - pk * IM01.x;
-                            const Real av = co.po * kvO;
-                            const Real idet = rcp(Real(1) - av * av);
-                            Real IO[4];
-                            IO[0] = (rI - av * rV) * idet;
-                            IO[3] = (rV - av * rI) * idet;
-                            IO[1] = r01.y;
-                            IO[2] = r23.x;
-                            StokesIO<Real, 4>::store(iw + f * iplane, ipts, l * nx + c, IO);
-                            // a8: Lambda* (Eq. 14; w_O + w_C/2 on the last plane) and accumulation
-                            const Real ls = co.wo + (has_p ? co.wc : Real(0.5) * co.wc);
-                            const Real wt = sfreq[F + f] * phO * invnO;
-                            const P2 a01 = pfma(pmk(wt, wt), pmk(IO[0], IO[1]), pmk(acc[0], acc[1]));
-                            const P2 a23 = pfma(pmk(wt, wt), pmk(IO[2], ls), pmk(acc[2], acc[3]));
-                            acc[0] = a01.x; acc[1] = a01.y; acc[2] = a23.x; acc[3] = a23.y;
-                            if (PROBE && a.probe_ray == m) {
-                                const int j = j0 + f;
-#pragma unroll
-                                for (int s = 0; s < 4; ++s) a.probe[((long long)j * a.nvox + v) * 4 + s] = IO[s];
-                                a.probe_ls[(long long)j * a.nvox + v] = ls;
-                            }
+                            sts2(sbase + sm.ibuf + h, I0, zero);
+                            sts2(sbase + sm.ibuf + h + chI, zero, zero);
                         }
                     }
                 }
-            }   // active
-            // fixed-order sum over the frequency lanes of each point (adjacent threads;
-            // every lane ends with the same totals, the additions being commutative)
-            for (int o = 1; o < L; o <<= 1) {
+                X eta, wt;
+                lds(sbase + sm.coef + f * sm.cplane + (p + nx) * CB, eta);
+                lds(sbase + sm.freq + FX * XW * SZ + f * 8, wt);
+                acc[0] = xdot(xmul(wt, eta), I0, acc[0]);
+                if (PROBE && a.probe_ray == m) {
+                    for (int w = 0; w < XW && j0 + f * XW + w < a.nnu; ++w) {
+                        const long long pv = (long long)(j0 + f * XW + w) * a.nvox + v;
 #pragma unroll
-                for (int s = 0; s < NA; ++s) acc[s] += __shfl_xor_sync(0xffffffffu, acc[s], o);
-            }
-            if (active && (a.jacc || lane == 0)) {
-                if (pb + pstep < npts) {
-                    if (a.jacc) add_terms(v, acc);
-                    else store_partial<Real, NS>(a, m, v, g, acc);
-                } else {
-                    pend = true;
-                    vpend = v;
-#pragma unroll
-                    for (int s = 0; s < NA; ++s) accp[s] = acc[s];
+                        for (int s = 0; s < NS; ++s) a.probe[pv * NS + s] = s == 0 ? xlane(I0, w) : Real(0);
+                        a.probe_ls[pv] = Real(0);
+                    }
                 }
             }
+            totals(0, p, acc);
         }
-        // plane q done here: arrive (release), stage plane q+2, wait (acquire). The
-        // last point round's sums go to global memory after the arrive, so that its
-        // release does not wait for them (nothing in the sweep reads them).
-        __syncthreads();
-        // release by the warps that wrote row 0 (the only Stokes vectors another CTA
-        // reads, through DSMEM); the others' plane data are read in this CTA only
-        if (__any_sync(0xffffffffu, row0_written)) cluster_arrive_release();
-        else cluster_arrive_relaxed();
-        if (pend) {
-            if (a.jacc) add_terms(vpend, accp);
-            else store_partial<Real, NS>(a, m, vpend, g, accp);
+    };
+
+    // One CTA barrier per plane: in phase q the threads update plane q (reading the nodes
+    // of planes q - 1, q, q + 1), fill plane q + 2 and add up plane q - 1. None of these
+    // reads what another writes in the same phase, so the warps run them in either order
+    // and the waits of one hide behind the arithmetic of another: those of the strip's
+    // first rows update first (the CTA before waits for row 0), those of its last rows
+    // last (they wait for the CTA after).
+    fetch(0);
+    fill(0);
+    fetch(1);
+    fill(1);
+    if (nz > 2) fetch(2);
+    __syncthreads();
+    const bool late = 2 * ((wid * 32 - fg * pw) / nx) >= R;
+    const unsigned halo_bytes = (unsigned)(nf * nx * NS) * 8;
+    const unsigned freed_next = map_rank(bars.freed, next_owner);
+    for (int q = 0; q < nz; ++q) {
+        // the halo row of plane q arrives during this plane's update and the next
+        if (C > 1 && tid == 0 && R > 0 && q + 1 < nz && !*bars.dead) bar_expect(bars.full + 8 * (q & 1), halo_bytes);
+        for (int part = 0; part < 2; ++part) {
+            if ((part != 0) != late) {
+                aside(q);
+                continue;
+            }
+            if (q == 0) boundary();
+            else if (q + 1 < nz) points(std::true_type{}, q);
+            else points(std::false_type{}, q);
         }
-        if (q + 2 < nz) fill(q + 2);
         __syncthreads();
-        cluster_wait_acquire();
+        // the halo row of plane q - 1 has been read: plane q + 1 may overwrite it (where it does)
+        if (C > 1 && tid == 0 && R > 0 && q >= 1 && q + 2 < nz && !*bars.dead) bar_arrive_remote(freed_next + 8 * ((q + 1) & 1));
+    }
+    // the last plane's sums
+    aside(nz);
+    __syncthreads();
+    if (R > 0) {
+        // phases of this item: halo rows of the planes 0 .. nz - 2; those that were overwritten
+        ph.full0 += (unsigned)(nz / 2);
+        ph.full1 += (unsigned)((nz - 1) / 2);
+        ph.freed0 += (unsigned)(nz / 2) - 1u;
+        ph.freed1 += nz >= 4 ? (unsigned)((nz - 1) / 2) - 1u : 0u;
     }
 }
 
 template <typename Real, int NS, bool PROBE>
-__global__ void __launch_bounds__(512, 1) jsweep_kernel(const SweepArgs<Real> a)
+__global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kernel(const SweepArgs<Real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ Real sray[24];
-    using W = JW<Real, NS>;
+    __shared__ __align__(16) Real sray[24];
+    __shared__ __align__(8) unsigned long long s_bar[4];
+    __shared__ int s_dead, s_item[2];
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int cid = blockIdx.x / C;
     const int ncl = gridDim.x / C;
-    Real *ring = reinterpret_cast<Real *>(smem_raw);
-    const int ring_bytes = (3 * a.ring_plane * W::s_words * (int)sizeof(Real) + 15) / 16 * 16;
-    Real *coef = reinterpret_cast<Real *>(smem_raw + ring_bytes);
-    const int coef_bytes = (3 * a.F * a.cstride * (int)sizeof(Real) + 15) / 16 * 16;
-    Real *ibuf = reinterpret_cast<Real *>(smem_raw + ring_bytes + coef_bytes);
-    Real *scratch = ibuf + 2 * a.F * a.istride;
-    Real *sfreq = scratch + W::g_words * a.ring_plane;
+    constexpr int XW = jsweep_lanes<Real>();
+    const JSmem sm = jsmem<Real, NS>(a.ring_plane, a.ipts_max, a.tots, (a.F + XW - 1) / XW);
+    JBars bars;
+    bars.full = smem_u32(s_bar);
+    bars.freed = smem_u32(s_bar + 2);
+    bars.dead = &s_dead;
+    JPhase ph = {0, 0, 0, 0};
+    if (threadIdx.x == 0) {
+        s_dead = 0;
+        for (int b = 0; b < 4; ++b) bar_init(smem_u32(s_bar + b));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     cluster.sync();
-    if (a.next_item) {
-        __shared__ int s_item[2];
-        for (int k = 0;; ++k) {
+    // fixed-point sums do not depend on the order of their terms: the frequency groups of a
+    // ray are items of their own; per-ray partials add their groups in order in one item
+    const int split = a.jacc ? a.ngroups : 1;
+    const int total = a.nitems * split;
+    for (int k = 0, own = cid;; ++k, own += ncl) {
+        int item = own;
+        if (a.next_item) {
             if (rank == 0 && threadIdx.x == 0) {
                 const int it = atomicAdd(a.next_item, 1);
                 for (int r = 0; r < C; ++r) *cluster.map_shared_rank(s_item + (k & 1), r) = it;
             }
             cluster.sync();
-            const int item = s_item[k & 1];
-            if (item >= a.nitems) break;
-            const int code = a.items ? a.items[item] : item;
-            const int box = code / a.nray, m = code - box * a.nray;
-            for (int g = 0; g < a.ngroups; ++g)
-                jsweep_item<Real, NS, PROBE>(a, cluster, ring, coef, ibuf, scratch, sray, sfreq, box, m, g, rank, C);
+            item = s_item[k & 1];
         }
-        return;
-    }
-    for (int item = cid; item < a.nitems; item += ncl) {
-        const int code = a.items ? a.items[item] : item;
+        if (item >= total) break;
+        const int ray = item / split;
+        const int code = a.items ? a.items[ray] : ray;
         const int box = code / a.nray, m = code - box * a.nray;
-        for (int g = 0; g < a.ngroups; ++g)
-            jsweep_item<Real, NS, PROBE>(a, cluster, ring, coef, ibuf, scratch, sray, sfreq, box, m, g, rank, C);
+        const int g0 = item - ray * split;
+        // the ray's constants (mu, ox, oy, oz, T[18], w, pad); the item starts with a barrier
+        if (threadIdx.x < 24) sray[threadIdx.x] = reinterpret_cast<const Real *>(a.rays + m)[threadIdx.x];
+        for (int g = g0; g < (split > 1 ? g0 + 1 : a.ngroups); ++g) {
+            jsweep_item<Real, NS, PROBE>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), box, m, g, rank, C);
+            // every halo row of the item has been written and read before the next one
+            // (whose strips may have other neighbours)
+            if (C > 1) cluster.sync();
+        }
     }
 }
 
@@ -685,17 +1073,40 @@ __global__ void __launch_bounds__(512, 1) jsweep_kernel(const SweepArgs<Real> a)
 // carries 46 fraction bits and the accumulator has 2^16 of headroom above it
 // (an FP32 term then converts without rounding; an FP64 term rounds at 2^-47 of
 // the reference value).
+// (jacc null: the FP64 form, which has no fixed-point sums; pack null: sweep_jw.cu, which
+// reads the inputs where they are). The same pass packs each
+// voxel's inputs of the sweep next to each other, so that a node's inputs arrive in
+// shared memory by 16-byte copies: chi, vel, rho[6], bx, by, bz (NS = 1: chi, vel, rho).
 template <typename Real, int NS>
-__global__ void jacc_prepare_kernel(long long nvox, const Real *rho, const Real *bpl, int *jexp,
-                                    unsigned long long *jacc)
+__global__ void jacc_prepare_kernel(const SweepArgs<Real> a, int *jexp, Real *pack)
 {
     const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long nvox = a.nvox;
     if (v >= nvox) return;
-    const double ref = fmax(fmax(fabs((double)rho[v]), fabs((double)bpl[v])), 1e-30);
+    using W = JW<Real, NS>;
+    if (pack) {
+        Real w[W::staged];
+        w[0] = a.chi[v];
+        w[1] = a.vel[v];
+        w[2] = a.rho[v];
+        w[W::staged - 1] = Real(0);
+        if constexpr (NS == 4) {
+#pragma unroll
+            for (int k = 1; k < 6; ++k) w[2 + k] = a.rho[k * nvox + v];
+            w[8] = a.bx[v];
+            w[9] = a.by[v];
+            w[10] = a.bz[v];
+        }
+        using V = typename V16<Real>::T;
+#pragma unroll
+        for (int h = 0; h < W::staged / W::per; ++h) chunk_put<Real>(reinterpret_cast<V *>(pack + v * W::staged) + h, w + h * W::per);
+    }
+    if (!a.jacc) return;
+    const double ref = fmax(fmax(fabs((double)a.rho[v]), fabs((double)a.bpl[v])), 1e-30);
     // kept within the FP32 exponent range, where the sweep forms 2^e exactly
     jexp[v] = min(max(kJFrac - ilogb(ref), -100), 126);
 #pragma unroll
-    for (int k = 0; k < JW<Real, NS>::nacc; ++k) jacc[k * nvox + v] = 0ULL;
+    for (int k = 0; k < W::nacc; ++k) a.jacc[k * nvox + v] = 0ULL;
 }
 
 template <int NS>
@@ -714,9 +1125,10 @@ __global__ void jacc_finalize_kernel(long long nvox, const unsigned long long *j
 template <typename Real, int NS>
 cudaError_t launch_jacc_prepare(const SweepArgs<Real> &a, cudaStream_t st)
 {
+    static_assert(JW<Real, NS>::staged == jpack_words<NS>(), "packed inputs of a voxel");
     const int bs = 256;
     const long long nb = (a.nvox + bs - 1) / bs;
-    jacc_prepare_kernel<Real, NS><<<(unsigned)nb, bs, 0, st>>>(a.nvox, a.rho, a.bpl, const_cast<int *>(a.jexp), a.jacc);
+    jacc_prepare_kernel<Real, NS><<<(unsigned)nb, bs, 0, st>>>(a, const_cast<int *>(a.jexp), const_cast<Real *>(a.pack));
     return cudaGetLastError();
 }
 
