@@ -318,7 +318,12 @@ int mlpol_tables(const std::vector<double> &J, const std::vector<double> &E, con
             }
         }
     t.cell_rc.clear(); t.cell_start.assign(1, 0); t.ent_src.clear(); t.ent_coef.clear();
-    for (auto &c : cells) {
+    // cells with as many terms next to each other: the lanes of a warp, a cell each, then add
+    // equally many
+    std::vector<std::pair<long long, std::vector<std::pair<int, double>>>> order(cells.begin(), cells.end());
+    std::stable_sort(order.begin(), order.end(),
+                     [](const auto &x, const auto &y) { return x.second.size() > y.second.size(); });
+    for (auto &c : order) {
         t.cell_rc.push_back((int)(c.first / nr));
         t.cell_rc.push_back((int)(c.first % nr));
         for (auto &e : c.second) {
@@ -485,27 +490,6 @@ __device__ __forceinline__ void cta_argmax(double &bv, int &br, double *red, int
         if (red[w] > bv || (red[w] == bv && redi[w] < br)) { bv = red[w]; br = redi[w]; }
 }
 
-// the same over FP32 values (FP32 compares: the FP64 pipe of this GPU is a small
-// fraction of its FP32 rate, and compares occupy it like arithmetic)
-__device__ __forceinline__ void cta_argmax(float &bv, int &br, float *red, int *redi)
-{
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int orr = __shfl_xor_sync(0xffffffffu, br, o);
-        if (ov > bv || (ov == bv && orr < br)) { bv = ov; br = orr; }
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
-        red[threadIdx.x >> 5] = bv;
-        redi[threadIdx.x >> 5] = br;
-    }
-    __syncthreads();
-    bv = red[0];
-    br = redi[0];
-    for (int w = 1; w < kVoxWarps; ++w)
-        if (red[w] > bv || (red[w] == bv && redi[w] < br)) { bv = red[w]; br = redi[w]; }
-}
-
 // the real system of voxel v into A [N][N + 1] (row of level 0's population =
 // the trace), sources into s; xo holds the old unknowns; lstar null: the plain
 // rates (no preconditioning). Called by all threads of the voxel's CTA.
@@ -577,123 +561,153 @@ __global__ void __launch_bounds__(kVoxThreads) mlpol_apply_kernel(const MlConst 
     }
 }
 
+// a value in FP32, truncated, by integer operations (the conversion instruction runs in the
+// FP64 pipe; the FP32 inverse need not be the nearest one); beyond FP32's range 0 or infinite
+__device__ __forceinline__ float to_float(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), m = hi & 0x7fffffffu;
+    if (m < 0x38100000u) return 0.0f;
+    const unsigned f = m < 0x47f00000u ? (m - 0x38000000u) << 3 | lo >> 29 : 0x7f800000u;
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
 // Solve of the K > 0 block B x = b (B = A restricted to the M = N - L unknowns
-// kidx[], b their right-hand sides; A itself is left unchanged) by LU factors in
+// kidx[], b their right-hand sides; A itself is left unchanged) by an inverse in
 // FP32 and iterative refinement with FP64 residuals: x = 0, r = b, then
-// d = (LU)^-1 P r, x += d, r = b - B x until the correction is below 1e-13 of x
+// d = B^-1 r, x += d, r = b - B x until the correction is below 1e-13 of x
 // (or has stopped shrinking below 1e-12 of it, the floor of FP64 residuals).
-// The factorization costs a third of the FP64 elimination's M^3 operations in
-// FP32 (64 times the FP64 rate on this GPU); each refinement step costs M^2 in
-// FP64. Returns false (the same in every thread) when a pivot vanishes or the
+// Returns false (the same in every thread) when a pivot vanishes or the
 // refinement does not converge: the caller then eliminates in FP64. On success
 // xn[kidx[i]] = x_i.
-__device__ bool mlpol_refine_solve(const double *A, int N, int M, const int *kidx, float *LU, float *y, int *piv,
-                                   double *xr, double *rr, double *xn, double *red, float *redf, int *redi)
+//
+// The inverse (Gauss-Jordan in place, partial pivoting with the rows left where they are)
+// stays in registers: MP >= M rows and columns, padded, as 8 x 16 tiles, one per thread. A
+// step publishes column k, finds the pivot (every warp for itself, one integer reduction of
+// the magnitudes' bits with the row in their low 7 bits), publishes the pivot row and updates
+// the tiles: two barriers and no pass over shared memory. Its M^3 operations in FP32 cost
+// less than the M^3 / 3 of LU factors in shared memory, and the refinement's solves are
+// products of whole tiles instead of two chains of M dependent steps in one warp: 69
+// unknowns (M = 64), 24576 voxels 11.2 -> 3.1 ms. In FP64 remain the residuals, M^2
+// operations each at 2 per cycle and SM.
+template <int MP>
+__device__ bool mlpol_refine_solve(const double *A, int N, int M, const int *kidx, float *fbuf, int *prow, double *xr,
+                                   double *rr, double *xn, unsigned *redu)
 {
-    const int N1 = N + 1, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    for (int e = tid; e < M * M; e += kVoxThreads) {
-        const int i = e / M, j = e - (e / M) * M;
-        LU[e] = (float)A[kidx[i] * N1 + kidx[j]];
-    }
+    constexpr int TR = MP / 8, TC = MP / 16;
+    const int N1 = N + 1, tid = threadIdx.x, lane = tid & 31;
+    const int tr = tid >> 4, tc = tid & 15, i0 = tr * TR, c0 = tc * TC;
+    float *col = fbuf, *row = col + 2 * MP, *y = row + 2 * MP, *d = y + MP;
+    int *qrow = prow + MP;
+    float B[TR][TC];
+#pragma unroll
+    for (int a = 0; a < TR; ++a)
+#pragma unroll
+        for (int b = 0; b < TC; ++b) {
+            const int i = i0 + a, j = c0 + b;
+            B[a][b] = i < M && j < M ? to_float(A[kidx[i] * N1 + kidx[j]]) : (i == j ? 1.0f : 0.0f);
+        }
     for (int i = tid; i < M; i += kVoxThreads) {
         rr[i] = A[kidx[i] * N1 + N];
         xr[i] = 0.0;
     }
+    unsigned used = 0;                                  // of the rows lane + 32 m, bit m
+    for (int kb = 0; kb * TR < M; ++kb) {
+#pragma unroll
+        for (int u = 0; u < TR; ++u) {
+            const int k = kb * TR + u;
+            if (k >= M) break;
+            float *ck = col + (u & 1) * MP, *rk = row + (u & 1) * MP;
+            const bool mine = tc == 2 * kb + u / TC;    // column k = 2 TC kb + u
+            if (mine) {
+#pragma unroll
+                for (int a = 0; a < TR; ++a) ck[i0 + a] = B[a][u % TC];
+            }
+            __syncthreads();
+            unsigned key = 0;
+#pragma unroll
+            for (int m = 0; m < (MP + 31) / 32; ++m) {
+                const int i = lane + 32 * m;
+                if (i < M && !(used >> m & 1u)) key = max(key, (__float_as_uint(fabsf(ck[i])) & ~127u) | (127u - i));
+            }
+            key = __reduce_max_sync(0xffffffffu, key);
+            if (key < 128u) return false;
+            const int p = 127 - (int)(key & 127u);
+            if (lane == (p & 31)) used |= 1u << (p >> 5);
+            const float inv = 1.0f / ck[p];
+            const int pa = p - i0;
+            if (pa >= 0 && pa < TR) {
+#pragma unroll
+                for (int b = 0; b < TC; ++b) {
+                    float x = 0.0f;
+#pragma unroll
+                    for (int a = 0; a < TR; ++a)
+                        if (a == pa) {
+                            x = B[a][b];
+                            B[a][b] = 0.0f;
+                        }
+                    rk[c0 + b] = mine && b == u % TC ? inv : x * inv;
+                }
+            }
+            if (tid == 0) {
+                prow[k] = p;
+                qrow[p] = k;
+            }
+            if (mine) {
+#pragma unroll
+                for (int a = 0; a < TR; ++a) B[a][u % TC] = 0.0f;
+            }
+            __syncthreads();
+            float r[TC];
+#pragma unroll
+            for (int b = 0; b < TC; ++b) r[b] = rk[c0 + b];
+#pragma unroll
+            for (int a = 0; a < TR; ++a) {
+                const float f = a == pa ? -1.0f : ck[i0 + a];
+#pragma unroll
+                for (int b = 0; b < TC; ++b) B[a][b] -= f * r[b];
+            }
+        }
+    }
     __syncthreads();
-    // LU with partial pivoting (rows swapped in place, multipliers below the diagonal).
-    // Step k: swap the pivot row in, then each warp updates its rows r = k+1+w (mod 4)
-    // with the lanes over the columns, stores the row's multiplier, and lane 0 (which
-    // holds column k+1) keeps the largest |value| of that column among the warp's rows:
-    // the next pivot comes from the four warps' candidates after one barrier (two
-    // barriers per step; the pivot is the largest |value|, the smallest row on ties).
-    constexpr int kCols = (kMlPolMaxUnk + 31) / 32;     // column slots per lane
-    float bv = -1.0f;
-    int br = 0;
-    for (int r = tid; r < M; r += kVoxThreads) {
-        const float a = fabsf(LU[r * M]);
-        if (a > bv) { bv = a; br = r; }
-    }
-    cta_argmax(bv, br, redf, redi);
-    for (int k = 0; k < M; ++k) {
-        if (!(bv > 0.0f)) return false;
-        if (tid == 0) piv[k] = br;
-        if (br != k)
-            for (int j = tid; j < M; j += kVoxThreads) {
-                const float tmp = LU[k * M + j];
-                LU[k * M + j] = LU[br * M + j];
-                LU[br * M + j] = tmp;
-            }
-        __syncthreads();
-        const float inv = 1.0f / LU[k * M + k];
-        float u[kCols];
-#pragma unroll
-        for (int m = 0; m < kCols; ++m) {
-            const int j = k + 1 + lane + 32 * m;
-            u[m] = j < M ? LU[k * M + j] : 0.0f;
-        }
-        float cv = -1.0f;
-        int cr = M;
-        for (int r = k + 1 + wid; r < M; r += kVoxWarps) {
-            const float l = LU[r * M + k] * inv;
-#pragma unroll
-            for (int m = 0; m < kCols; ++m) {
-                const int j = k + 1 + lane + 32 * m;
-                if (j < M) LU[r * M + j] -= l * u[m];
-            }
-            if (lane == 0) {                // (r > k, so column k + 1 exists)
-                const float a = fabsf(LU[r * M + k + 1]);
-                if (a > cv) { cv = a; cr = r; }
-            }
-        }
-        __syncwarp();
-        for (int r = k + 1 + wid + kVoxWarps * lane; r < M; r += 32 * kVoxWarps) LU[r * M + k] *= inv;
-        if (lane == 0) {
-            redf[wid] = cv;
-            redi[wid] = cr;
-        }
-        __syncthreads();
-        bv = redf[0];
-        br = redi[0];
-        for (int w = 1; w < kVoxWarps; ++w)
-            if (redf[w] > bv || (redf[w] == bv && redi[w] < br)) { bv = redf[w]; br = redi[w]; }
-        // (the next step writes red only after its swap barrier)
-    }
     double dprev = 1e300;
     for (int it = 0; it < 8; ++it) {
-        // d = U^-1 L^-1 P r in FP32 (warp 0)
-        if (wid == 0) {
-            for (int i = lane; i < M; i += 32) y[i] = (float)rr[i];
-            __syncwarp();
-            if (lane == 0)
-                for (int k = 0; k < M; ++k) {
-                    const int p = piv[k];
-                    if (p != k) {
-                        const float t = y[k]; y[k] = y[p]; y[p] = t;
-                    }
-                }
-            __syncwarp();
-            for (int k = 0; k + 1 < M; ++k) {
-                const float yk = y[k];
-                for (int i = k + 1 + lane; i < M; i += 32) y[i] -= LU[i * M + k] * yk;
-                __syncwarp();
-            }
-            for (int k = M - 1; k >= 0; --k) {
-                const float yk = y[k] / LU[k * M + k];
-                for (int i = lane; i < k; i += 32) y[i] -= LU[i * M + k] * yk;
-                __syncwarp();
-                if (lane == 0) y[k] = yk;
-                __syncwarp();
-            }
+        // row p_k of the tiles times the residuals in the order of the pivots is x_k
+        for (int k = tid; k < MP; k += kVoxThreads) y[k] = k < M ? (float)rr[prow[k]] : 0.0f;
+        __syncthreads();
+        float yb[TC];
+#pragma unroll
+        for (int b = 0; b < TC; ++b) yb[b] = y[c0 + b];
+#pragma unroll
+        for (int a = 0; a < TR; ++a) {
+            float t = 0.0f;
+#pragma unroll
+            for (int b = 0; b < TC; ++b) t = fmaf(B[a][b], yb[b], t);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (tc == 0) d[i0 + a] = t;
         }
         __syncthreads();
-        double dm = 0.0, xm = 0.0;
+        // largest |d| and |x| (the latter to 20 bits), by integer reductions of their bits
+        unsigned db = 0, xb = 0;
         for (int i = tid; i < M; i += kVoxThreads) {
-            xr[i] += (double)y[i];
-            dm = fmax(dm, fabs((double)y[i]));
-            xm = fmax(xm, fabs(xr[i]));
+            const int k = qrow[i];
+            const double x = xr[k] + (double)d[i];
+            xr[k] = x;
+            db = max(db, __float_as_uint(fabsf(d[i])));
+            xb = max(xb, (unsigned)__double2hiint(x) & 0x7fffffffu);
         }
-        dm = cta_max(dm, red);
-        xm = cta_max(xm, red);
+        db = __reduce_max_sync(0xffffffffu, db);
+        xb = __reduce_max_sync(0xffffffffu, xb);
+        if (lane == 0) {
+            redu[tid >> 5] = db;
+            redu[kVoxWarps + (tid >> 5)] = xb;
+        }
+        __syncthreads();
+        for (int w = 0; w < kVoxWarps; ++w) {
+            db = max(db, redu[w]);
+            xb = max(xb, redu[kVoxWarps + w]);
+        }
+        const double dm = (double)__uint_as_float(db), xm = __hiloint2double((int)xb, 0);
         if (!(dm < 1e300 && xm < 1e300)) return false;
         if (dm <= 1e-13 * xm || (dm <= 1e-12 * xm && dm > 0.5 * dprev)) {
             for (int i = tid; i < M; i += kVoxThreads) xn[kidx[i]] = xr[i];
@@ -701,12 +715,13 @@ __device__ bool mlpol_refine_solve(const double *A, int N, int M, const int *kid
             return true;
         }
         dprev = dm;
-        // r = b - B x (FP64)
-        for (int i = tid; i < M; i += kVoxThreads) {
-            const double *Ar = A + kidx[i] * N1;
-            double acc = Ar[N];
-            for (int j = 0; j < M; ++j) acc -= Ar[kidx[j]] * xr[j];
-            rr[i] = acc;
+        // r = b - B x (FP64), two threads per row
+        for (int i = tid >> 1; i < (M + 15) / 16 * 16; i += kVoxThreads / 2) {
+            const double *Ar = A + kidx[min(i, M - 1)] * N1;
+            double acc = 0.0;
+            for (int j = tid & 1; j < M; j += 2) acc += Ar[kidx[j]] * xr[j];
+            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+            if (i < M && (tid & 1) == 0) rr[i] = Ar[N] - acc;
         }
         __syncthreads();
     }
@@ -714,9 +729,10 @@ __device__ bool mlpol_refine_solve(const double *A, int N, int M, const int *kid
 }
 
 // one CTA per voxel; shared memory: A[nunk][nunk + 1], x_old, x_new, sources, and
-// for the refinement solve FP64 x and r, the FP32 LU factors and work vector,
-// pivots and the indices of the K > 0 unknowns
-__global__ void __launch_bounds__(kVoxThreads) mlpol_see_kernel(const MlConst mc, MlPolDev T, long long nvox1,
+// for the refinement solve FP64 x and r, its FP32 rows, columns and vectors, the pivots and
+// the indices of the K > 0 unknowns. MP: their number rounded up (mlpol_pad)
+template <int MP>
+__global__ void __launch_bounds__(kVoxThreads, MP <= 64 ? 5 : 1) mlpol_see_kernel(const MlConst mc, MlPolDev T, long long nvox1,
                                                                 const double *kT, const double *jkq, const double *j1,
                                                                 const double *lstar, const double *bvec,
                                                                 const double *src, double *x, unsigned long long *resid,
@@ -724,8 +740,9 @@ __global__ void __launch_bounds__(kVoxThreads) mlpol_see_kernel(const MlConst mc
 {
     extern __shared__ double sm[];
     __shared__ double red[kVoxWarps];
-    __shared__ float redf[kVoxWarps];
     __shared__ int redi[kVoxWarps];
+    __shared__ unsigned redu[2 * kVoxWarps];
+    __shared__ double m1[kMlMaxLevel][kMlMaxLevel + 1];
     const int N = T.nunk, N1 = N + 1;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     double *A = sm;
@@ -734,9 +751,8 @@ __global__ void __launch_bounds__(kVoxThreads) mlpol_see_kernel(const MlConst mc
     double *s = xn + N;
     double *xr = s + T.nsrc;
     double *rr = xr + N;
-    float *LU = reinterpret_cast<float *>(rr + N);
-    float *y = LU + N * N;
-    int *kidx = reinterpret_cast<int *>(y + N);
+    float *fbuf = reinterpret_cast<float *>(rr + N);
+    int *kidx = reinterpret_cast<int *>(fbuf + 6 * MP);
     int *piv = kidx + N;
     // the K > 0 unknowns (all but the populations)
     const int M = N - mc.nlev;
@@ -763,43 +779,47 @@ __global__ void __launch_bounds__(kVoxThreads) mlpol_see_kernel(const MlConst mc
                 if (T.pop_idx[i] == c) return true;
             return false;
         };
-        for (int i = 0; i < L; ++i) {
+        for (int i = wid; i < L; i += kVoxWarps) {
             const int r = T.pop_idx[i];
             double acc = 0.0;
-            for (int c = tid; c < N; c += kVoxThreads)
+            for (int c = lane; c < N; c += 32)
                 if (!is_k0(c)) acc += A[r * N1 + c] * xo[c];
-            acc = cta_sum(acc, red);
-            if (tid == 0) A[r * N1 + N] -= acc;
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) m1[i][L] = A[r * N1 + N] - acc;
+            if (lane < L) m1[i][lane] = A[r * N1 + T.pop_idx[lane]];
         }
         __syncthreads();
-        if (tid == 0) {
+        // elimination with partial pivoting, a lane per column (lane L: the right-hand side)
+        if (wid == 0) {
             int ok1 = 1;
-            double m[kMlMaxLevel][kMlMaxLevel + 1];
-            for (int i = 0; i < L; ++i) {
-                for (int j = 0; j < L; ++j) m[i][j] = A[T.pop_idx[i] * N1 + T.pop_idx[j]];
-                m[i][L] = A[T.pop_idx[i] * N1 + N];
-            }
-            for (int c = 0; c < L && ok1; ++c) {
+            for (int c = 0; c < L; ++c) {
                 int p = c;
                 for (int r = c + 1; r < L; ++r)
-                    if (fabs(m[r][c]) > fabs(m[p][c])) p = r;
-                if (!(fabs(m[p][c]) > 0.0)) { ok1 = 0; break; }
-                if (p != c)
-                    for (int j = 0; j <= L; ++j) {
-                        const double tmp = m[c][j]; m[c][j] = m[p][j]; m[p][j] = tmp;
-                    }
+                    if (fabs(m1[r][c]) > fabs(m1[p][c])) p = r;
+                if (!(fabs(m1[p][c]) > 0.0)) { ok1 = 0; break; }
+                __syncwarp();
+                if (p != c && lane <= L) {
+                    const double tmp = m1[c][lane]; m1[c][lane] = m1[p][lane]; m1[p][lane] = tmp;
+                }
+                __syncwarp();
+                // (lane r: the factor of row r)
+                const double fr = lane > c && lane < L ? m1[lane][c] / m1[c][c] : 0.0;
                 for (int r = c + 1; r < L; ++r) {
-                    const double f = m[r][c] / m[c][c];
-                    for (int j = c; j <= L; ++j) m[r][j] -= f * m[c][j];
+                    const double f = __shfl_sync(0xffffffffu, fr, r);
+                    if (lane >= c && lane <= L) m1[r][lane] -= f * m1[c][lane];
+                }
+                __syncwarp();
+            }
+            if (ok1) {
+                // (lane i: row i's sum)
+                double acc = lane < L ? m1[lane][L] : 0.0;
+                for (int i = L - 1; i >= 0; --i) {
+                    const double xi = __shfl_sync(0xffffffffu, acc, i) / m1[i][i];
+                    if (lane == 0) xn[T.pop_idx[i]] = xi;
+                    if (lane < i) acc -= m1[lane][i] * xi;
                 }
             }
-            if (ok1)
-                for (int i = L - 1; i >= 0; --i) {
-                    double acc = m[i][L];
-                    for (int j = i + 1; j < L; ++j) acc -= m[i][j] * xn[T.pop_idx[j]];
-                    xn[T.pop_idx[i]] = acc / m[i][i];
-                }
-            redi[0] = ok1;
+            if (lane == 0) redi[0] = ok1;
         }
         __syncthreads();
         const int ok1 = redi[0];
@@ -824,7 +844,7 @@ __global__ void __launch_bounds__(kVoxThreads) mlpol_see_kernel(const MlConst mc
         // take the columns, the warps the rows of the trailing block
         bool ok = ok1 != 0;
         const bool refined =
-            ok && M > 0 && T.solve == 0 && mlpol_refine_solve(A, N, M, kidx, LU, y, piv, xr, rr, xn, red, redf, redi);
+            ok && M > 0 && T.solve == 0 && mlpol_refine_solve<MP>(A, N, M, kidx, fbuf, piv, xr, rr, xn, redu);
         for (int k = 0; k < N && !refined; ++k) {
             double bv = -1.0;
             int br = k;
@@ -904,11 +924,14 @@ template cudaError_t run_mlpol_prepare<double>(const MlConst &, const MlPolDev &
                                                const double *, double *, double *, double *, double *, double *,
                                                unsigned long long *, cudaStream_t);
 
-size_t mlpol_see_smem(const MlPolDev &T, int voxels)
+// rows and columns of the refinement's tiles for M unknowns: a tile of (MP / 8) x (MP / 16)
+// values per thread
+static int mlpol_pad(int M) { return M <= 32 ? 32 : (M <= 64 ? 64 : (M <= 96 ? 96 : 128)); }
+
+static size_t mlpol_see_smem(const MlConst &mc, const MlPolDev &T)
 {
-    const size_t N = T.nunk;
-    return (size_t)voxels * (sizeof(double) * (N * (N + 1) + 4 * N + T.nsrc) + sizeof(float) * (N * N + N) +
-                             sizeof(int) * 2 * N);
+    const size_t N = T.nunk, MP = mlpol_pad(T.nunk - mc.nlev);
+    return sizeof(double) * (N * (N + 1) + 4 * N + T.nsrc) + sizeof(float) * 6 * MP + sizeof(int) * (N + 2 * MP);
 }
 
 namespace {
@@ -964,13 +987,13 @@ cudaError_t run_mlpol_change(const MlConst &mc, const MlPolDev &T, long long nvo
 
 // persistent launch shape of the CTA-per-voxel kernels: as many CTAs as fit on the GPU
 template <typename K>
-static cudaError_t voxel_launch_shape(K kernel, const MlPolDev &T, long long nvox1, size_t &smem, int &blocks)
+static cudaError_t voxel_launch_shape(K kernel, const MlConst &mc, const MlPolDev &T, long long nvox1, size_t &smem, int &blocks)
 {
     int dev = 0, nsm = 0, per_sm = 1, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    smem = mlpol_see_smem(T, 1);
+    smem = mlpol_see_smem(mc, T);
     if (smem > (size_t)optin) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -983,11 +1006,13 @@ cudaError_t run_mlpol_see(const MlConst &mc, const MlPolDev &T, long long nvox1,
                           const double *j1, const double *lstar, const double *bvec, double *x, unsigned long long *resid,
                           unsigned long long *bad, cudaStream_t st, const double *src)
 {
+    const int MP = mlpol_pad(T.nunk - mc.nlev);
+    const auto kernel = MP == 32 ? mlpol_see_kernel<32> : (MP == 64 ? mlpol_see_kernel<64> : (MP == 96 ? mlpol_see_kernel<96> : mlpol_see_kernel<128>));
     size_t smem = 0;
     int blocks = 1;
-    cudaError_t e = voxel_launch_shape(mlpol_see_kernel, T, nvox1, smem, blocks);
+    cudaError_t e = voxel_launch_shape(kernel, mc, T, nvox1, smem, blocks);
     if (e != cudaSuccess) return e;
-    mlpol_see_kernel<<<blocks, kVoxThreads, smem, st>>>(mc, T, nvox1, kT, jkq, j1, lstar, bvec, src, x, resid, bad);
+    kernel<<<blocks, kVoxThreads, smem, st>>>(mc, T, nvox1, kT, jkq, j1, lstar, bvec, src, x, resid, bad);
     return cudaGetLastError();
 }
 
@@ -997,7 +1022,7 @@ cudaError_t run_mlpol_apply(const MlConst &mc, const MlPolDev &T, long long nvox
 {
     size_t smem = 0;
     int blocks = 1;
-    cudaError_t e = voxel_launch_shape(mlpol_apply_kernel, T, nvox1, smem, blocks);
+    cudaError_t e = voxel_launch_shape(mlpol_apply_kernel, mc, T, nvox1, smem, blocks);
     if (e != cudaSuccess) return e;
     mlpol_apply_kernel<<<blocks, kVoxThreads, smem, st>>>(mc, T, nvox1, kT, jkq, j1, bvec, x, alpha, add, with_f, out);
     return cudaGetLastError();
