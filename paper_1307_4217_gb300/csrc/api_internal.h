@@ -112,6 +112,9 @@ void plane_geometry(int nx, int ny, int nz, double lx, double ly, const double *
 // the same for the J^K_Q sweep, which uses the bilinear weights relative to the first one:
 // in place of (tx, ty, ds, pad2) it reads u = t / (1 - t) along x and y, the first weight
 // (1 - tx) (1 - ty), and ds / 2. A factor 1 - t that rounds to 0 is held at the rounding unit of 1.
+// The first weight is what makes the rounded weights add up to 1: planes of equal spacing
+// have equal weights, and a ray through a transparent medium would gather their excess (the
+// products of the unrounded factors left 2e-8 per plane on average over a quadrature's rays).
 template <typename Real>
 PlaneGeom<Real> relative_geometry(const PlaneGeom<Real> &p)
 {
@@ -120,7 +123,8 @@ PlaneGeom<Real> relative_geometry(const PlaneGeom<Real> &p)
     PlaneGeom<Real> r = p;
     r.tx = (Real)(p.tx / mx);
     r.ty = (Real)(p.ty / my);
-    r.ds = (Real)(mx * my);
+    const Real uxy = r.tx * r.ty;        // as the sweep forms it
+    r.ds = (Real)(1.0 / (1.0 + (double)r.tx + (double)r.ty + (double)uxy));
     r.pad2 = (Real)(0.5 * p.ds);
     return r;
 }

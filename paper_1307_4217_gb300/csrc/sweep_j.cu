@@ -33,9 +33,9 @@
 // FP32; jsweep_plane_cost), whatever the strip, so a pass has few units over as many points
 // as the threads hold. Against the kernel of sweep_jw.cu, which this one replaces where it
 // fits (one frequency of one point per thread and step, one cluster barrier per plane), ms
-// per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 18.7, 33 x 27 x 41 x
-// 80 x 21 1.91 -> 1.25, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.8, 64 x 64 x 48 x 160 x 31
-// x 2 lines, unpolarized, 46.4 -> 32.6 (with the rate equations).
+// per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 18.0, 33 x 27 x 41 x
+// 80 x 21 1.91 -> 1.22, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.8, 64 x 64 x 48 x 160 x 31
+// x 2 lines, unpolarized, 46.4 -> 32.4 (with the rate equations).
 //
 // Shared memory per CTA (X: 8 bytes, a frequency unit):
 //   ring[4][nodes]        source vectors, Real
@@ -111,6 +111,16 @@ __device__ __forceinline__ bool jadd(unsigned long long *p, float y)
                                  (((unsigned long long)(__float_as_uint(h) - B) << 40) - (unsigned long long)B * ((1u << 18) + 1u));
     atomicAdd(p, k + __float_as_uint(l));
     return !(fabsf(y) < 4.6116860e18f);
+}
+// the same for |y| <= 2^45 (terms up to half the voxel's reference value) in two parts, 5
+// instructions less for each of a point's 7 terms
+__device__ __forceinline__ void jadd_small(unsigned long long *p, float y)
+{
+    constexpr float M = 12582912.0f;
+    constexpr unsigned B = 0x4b400000u;
+    const float h = fmaf(y, 0x1p-23f, M), l = fmaf(M - h, 0x1p23f, y) + M;
+    const unsigned long long k = (unsigned long long)__float_as_uint(h) * (1u << 23) - (unsigned long long)B * ((1u << 23) + 1u);
+    atomicAdd(p, k + __float_as_uint(l));
 }
 
 // per-ray partial integrals of a point (the FP64 form: summed over rays in ray
@@ -204,35 +214,55 @@ __device__ __forceinline__ double xdet(double a) { return 1.0 - a * a; }
 __device__ __forceinline__ float xlane(float2 a, int i) { return i ? a.y : a.x; }
 __device__ __forceinline__ double xlane(double a, int) { return a; }
 
-// Coefficients of the step (Eqs. 9-13) of a unit: e = e^-t and the three w. In FP32 e^-t is
-// one hardware power of two (its argument's rounding, t 2^-24 relative, is multiplied by
-// e^-t <= 1/(e t) in the step); the polynomial and the closed forms are evaluated where
-// some lane needs them.
-template <typename X> struct XCoef { X e, wm, wo, wc; };
+// Coefficients of the step (Eqs. 9-13) of a unit: e = e^-t, their sum e0 = 1 - e, and the
+// three w. With q = w_O, h = t (1 - q) / 2 gives e0 = t (1 - h), w_O + w_C = e0 - w_M (or
+// 2 h - q): below t = 1.5 two polynomials (w_M and w_O over t, minimax in relative error:
+// 5e-9 and 3e-9) yield all five, above it closed forms whose cancellation costs a factor of
+// about 3. e0 is within 1.2e-7 of its value and e + e0 = 1 to rounding, so a constant source
+// function is kept; w_M is within 2e-7, w_O + w_C and w_C, which multiply differences of
+// source functions, within 3e-7 and 8e-7. The polynomials are evaluated for both lanes
+// always; the closed forms replace them where some lane needs them. (Three polynomials, an
+// exponential per lane and the sums: 26 instructions more per unit, 3% of the sweep's time.)
+template <typename X> struct XCoef { X e, e0, wm, wo, wc; };
 __device__ __forceinline__ XCoef<double> xcoef(double t)
 {
     const Coef<double> c = coefficients(t);
-    return {c.e, c.wm, c.wo, c.wc};
+    return {c.e, c.wm + c.wo + c.wc, c.wm, c.wo, c.wc};
 }
 __device__ __forceinline__ XCoef<float2> xcoef(float2 t)
 {
     XCoef<float2> c;
-    const float2 u = xmul(t, xset(-1.4426950408889634f));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(c.e.x) : "f"(u.x));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(c.e.y) : "f"(u.y));
+    const float2 one = xset(1.0f), nt = xneg(t);
+    float2 m = xset(-9.985858924e-06f), o = xset(3.294269391e-06f);
+    m = xfma(t, m, xset(1.324526238e-04f));
+    m = xfma(t, m, xset(-1.014578040e-03f));
+    o = xfma(t, o, xset(-4.541862290e-05f));
+    m = xfma(t, m, xset(5.933146924e-03f));
+    o = xfma(t, o, xset(3.927011858e-04f));
+    m = xfma(t, m, xset(-2.777018584e-02f));
+    o = xfma(t, o, xset(-2.775641857e-03f));
+    m = xfma(t, m, xset(9.999849647e-02f));
+    o = xfma(t, o, xset(1.666613296e-02f));
+    m = xfma(t, m, xset(-2.499998808e-01f));
+    o = xfma(t, o, xset(-8.333328366e-02f));
+    m = xfma(t, m, xset(3.333333433e-01f));
+    o = xfma(t, o, xset(3.333333433e-01f));
+    c.wm = xmul(t, m);
+    c.wo = xmul(t, o);
+    const float2 ht = xms(0.5f, t);
+    c.e0 = xfma(nt, xfma(xneg(ht), c.wo, ht), t);
+    c.e = xadd(one, xneg(c.e0));
+    c.wc = xadd(xadd(c.e0, xneg(c.wm)), xneg(c.wo));
     if (fmaxf(t.x, t.y) >= 1.5f) {
-        const float2 one = xset(1.0f), two = xset(2.0f), it = xrcp(t), it2 = xmul(it, it), ne = xneg(c.e);
-        const float2 tp = xadd(t, two);
-        c.wm = xmul(xfma(ne, xfma(t, tp, two), two), it2);
-        c.wo = xfma(xmul(xadd(xadd(c.e, t), xset(-1.0f)), xset(-2.0f)), it2, one);
-        c.wc = xmul(xmul(xfma(c.e, tp, xadd(t, xset(-2.0f))), two), it2);
-    }
-    if (fminf(t.x, t.y) < 1.5f) {
-        float m, o, k;
-        wpoly(t.x, m, o, k);
-        if (t.x < 1.5f) { c.wm.x = m; c.wo.x = o; c.wc.x = k; }
-        wpoly(t.y, m, o, k);
-        if (t.y < 1.5f) { c.wm.y = m; c.wo.y = o; c.wc.y = k; }
+        const float2 two = xset(2.0f), u = xms(-1.4426950408889634f, t), it = xrcp(t);
+        float2 e;
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.x) : "f"(u.x));
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e.y) : "f"(u.y));
+        const float2 e0 = xadd(one, xneg(e)), h = xfma(xneg(e0), it, one), h2 = xadd(h, h);
+        const float2 wm = xmul(xfma(xneg(e), xfma(t, xadd(t, two), two), two), xmul(it, it));
+        const float2 wo = xfma(xneg(h2), it, one), hd = xadd(h2, xneg(e0)), wc = xmul(xadd(hd, hd), it);
+        if (t.x >= 1.5f) { c.e.x = e.x; c.e0.x = e0.x; c.wm.x = wm.x; c.wo.x = wo.x; c.wc.x = wc.x; }
+        if (t.y >= 1.5f) { c.e.y = e.y; c.e0.y = e0.y; c.wm.y = wm.y; c.wo.y = wo.y; c.wc.y = wc.y; }
     }
     return c;
 }
@@ -559,6 +589,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
             unsigned oc = opaque(sbase + sm.coef + s * FX * sm.cplane + idx * CB), of = sbase + sm.freq;
             if constexpr (NS == 1) {
                 sts(sbase + (s * nodes + idx) * SZ, d[2]);
+#pragma unroll 2
                 for (int f = 0; f < nf; ++f, oc += sm.cplane, of += 8) {
                     X x;
                     lds(of, x);
@@ -574,6 +605,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                                                                               t[6 * i + 4] * d[6] + t[6 * i + 5] * d[7]);
                 w[3] = d[2];
                 sts4(sbase + (s * W::s_chunks * nodes + idx) * 16, nodes * 16, w);
+#pragma unroll 2
                 for (int f = 0; f < nf; ++f, oc += sm.cplane, of += 8) {
                     X x;
                     lds(of, x);
@@ -598,21 +630,35 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
             return;
         }
         if constexpr (SZ == 4) {
-            bool bad = false;
-            unsigned long long *acc = a.jacc + v;
+            Real y[W::nacc], sum_abs = 0;
             if constexpr (NS == 1) {
-                bad |= jadd(acc, t[0]);
-                bad |= jadd(acc + nvox, t[1]);
+                y[0] = t[0];
+                y[1] = t[1];
             } else {
                 Real T[20];
 #pragma unroll
                 for (int i = 0; i < 5; ++i) ray4(1 + i, T + 4 * i);
 #pragma unroll
-                for (int k = 0; k < 6; ++k, acc += nvox)
-                    bad |= jadd(acc, T[k] * t[0] + T[6 + k] * t[1] + T[12 + k] * t[2]);
-                bad |= jadd(acc, t[3]);
+                for (int k = 0; k < 6; ++k) y[k] = T[k] * t[0] + T[6 + k] * t[1] + T[12 + k] * t[2];
+                y[6] = t[3];
             }
-            if (bad) atomicOr(a.jerr, 1);
+#pragma unroll
+            for (int k = 0; k < W::nacc; ++k) sum_abs += fabsf(y[k]);
+            unsigned long long *acc = a.jacc + v;
+            if (sum_abs <= 0x1p45f) {
+#pragma unroll
+                for (int k = 0; k < W::nacc; ++k, acc += nvox) jadd_small(acc, y[k]);
+            } else {
+                bool bad = false;
+#pragma unroll 1
+                for (int k = 0; k < W::nacc; ++k, acc += nvox) {
+                    Real x = y[0];
+#pragma unroll
+                    for (int i = 1; i < W::nacc; ++i) x = k == i ? y[i] : x;
+                    bad |= jadd(acc, x);
+                }
+                if (bad) atomicOr(a.jerr, 1);
+            }
         }
     };
     // the same from the totals of several groups of threads (written a phase before)
@@ -773,12 +819,12 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 // a4, a6: optical path and coefficients of the step
                 const X tMO = xms(dsM, xfs(wM, eM, eO));
                 const XCoef<X> co = xcoef(tMO);
-                const X ls = has_p ? xadd(co.wo, co.wc) : xfs(Real(0.5), co.wc, co.wo);
+                const X ls = has_p ? (XW == 1 ? xadd(co.wo, co.wc) : xadd(co.e0, xneg(co.wm))) : xfs(Real(0.5), co.wc, co.wo);
                 // a7: right-hand side of Eq. 7, e I_M + (w_M + w_O + w_C) S_O - w_M d_M - w_C (S_O - c_M),
                 // with the upwind Stokes vector over w_M (a3) and K'_V at M coupling I and V
                 X r[NS];
                 {
-                    const X wsum = xadd(xadd(co.wm, co.wo), co.wc), ew = xms(wM, co.e);
+                    const X wsum = co.e0, ew = xms(wM, co.e);
                     // without a downwind point c_M = (S_M + S_O) / 2
                     const X nwm = has_p ? xneg(co.wm) : xfs(Real(-0.5), co.wc, xneg(co.wm));
 #pragma unroll
