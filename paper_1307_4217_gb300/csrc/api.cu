@@ -292,12 +292,17 @@ void check_global_sweep(porta_ctx *c)
     if (!c->sc_faces && !c->gsweep && c->d_kexpl == nullptr && c->interp != 2 && !smem_sweep_fits(c)) c->gsweep = 2;
 }
 
+cudaError_t ensure_jpack(porta_ctx *c)
+{
+    if (c->d_jpack) return cudaSuccess;
+    return pmalloc(&c->d_jpack, (size_t)(c->ns == 1 ? jpack_words<1>() : jpack_words<4>()) * c->nvox * c->rsz);
+}
+
 cudaError_t ensure_sweep_buffers(porta_ctx *c)
 {
     check_global_sweep(c);
     cudaError_t e = cudaSuccess;
-    if (use_jk(c) && c->jk_form == 1 && !c->d_jpack)
-        e = pmalloc(&c->d_jpack, (size_t)(c->ns == 1 ? jpack_words<1>() : jpack_words<4>()) * c->nvox * c->rsz);
+    if (use_jk(c) && c->jk_form == 1) e = ensure_jpack(c);
     if (e != cudaSuccess) return e;
     if (jfixed(c)) {
         if (!c->d_jacc) e = pmalloc(&c->d_jacc, (size_t)(c->nj + 1) * c->nvox * sizeof(unsigned long long));
@@ -640,6 +645,8 @@ int autotune_t(porta_ctx *c)
 
 void free_all(porta_ctx *c)
 {
+    if (c->h_flag) cudaFreeHost(c->h_flag);
+    c->h_flag = nullptr;
     drop_graph(c);
     mg_free(c);
     it_free(c);
@@ -669,7 +676,7 @@ void free_all(porta_ctx *c)
     for (cudaEvent_t &ev : c->adj_ev)
         if (ev) cudaEventDestroy(ev);
     void *ptrs[] = {c->d_atm, c->d_eps, c->d_bpl, c->d_b, c->d_rho, c->d_rhoR, c->d_invn, c->d_geom, c->d_rays,
-                    c->d_freq, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->d_resid, c->d_err, c->d_boxes,
+                    c->d_freq, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->d_resid, c->d_err, c->d_dirs, c->d_boxes,
                     c->d_items, c->d_tune_items, c->d_tape, c->d_gpart, c->d_jacc, c->d_jexp, c->d_jpack, c->d_kexpl, c->d_sexpl,
                     c->d_partv, c->d_j1, c->d_tw1, c->d_gjR, c->d_vjp_out, c->d_faces, c->d_fdxy};
     for (void *p : ptrs)
@@ -836,7 +843,8 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
     ok(dalloc(&c->d_jkq, nvox * c->nj));
     ok(dalloc(&c->d_lstar, nvox));
     ok(dalloc(&c->d_resid, 1));
-    ok(dalloc(&c->d_err, 1));
+    ok(dalloc(&c->d_err, 2));     // formal solution; emergent sweep (sticky until read)
+    if (rc == PORTA_OK) ok(cudaMemset(c->d_err, 0, 2 * sizeof(int)));
     if (rc == PORTA_OK) {
         ok(cudaMemset(c->d_atm, 0, 6 * nvox * R));
         // geometry, rays, frequencies, angular weights
@@ -862,6 +870,13 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
         std::vector<int> tune(c->n_tune);
         for (int i = 0; i < c->n_tune; ++i) tune[i] = items[(size_t)i * items.size() / c->n_tune];
         ok(cudaMemcpy(c->d_tune_items, tune.data(), tune.size() * sizeof(int), cudaMemcpyHostToDevice));
+        auto relative_form = [&](auto &geom) {
+            for (int b = 0; b < nbox; ++b)
+                for (int m = 0; m < c->nray; ++m) {
+                    const size_t o = c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz;
+                    relative_geometry(geom.data() + o, c->boxes[b].nz, geom.data() + geom.size() / 2 + o);
+                }
+        };
         if (prec == PORTA_FP32) {
             std::vector<PlaneGeom<float>> geom(2 * (size_t)c->nray * nplane);
             std::vector<RayDev<float>> rays(c->nray);
@@ -871,7 +886,7 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
                     plane_geometry<float>(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
                                           c->bz[b].data(), c->mu[m], c->chi[m],
                                           geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz);
-            for (size_t i = 0; i < geom.size() / 2; ++i) geom[geom.size() / 2 + i] = relative_geometry(geom[i]);
+            relative_form(geom);
             for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<float>(c->mu[m], c->chi[m], c->w[m]);
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = (float)c->xf[j]; fr[c->n_nu + j] = (float)c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));
@@ -886,7 +901,7 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
                     plane_geometry<double>(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
                                            c->bz[b].data(), c->mu[m], c->chi[m],
                                            geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz);
-            for (size_t i = 0; i < geom.size() / 2; ++i) geom[geom.size() / 2 + i] = relative_geometry(geom[i]);
+            relative_form(geom);
             for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<double>(c->mu[m], c->chi[m], c->w[m]);
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = c->xf[j]; fr[c->n_nu + j] = c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));

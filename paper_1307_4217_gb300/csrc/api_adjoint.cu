@@ -89,42 +89,135 @@ int emergent_shape(porta_ctx *c, SweepArgs<Real> &a, int ndir, LaunchCfg &cfg)
     return PORTA_OK;
 }
 
+// The emergent-mode sweep (with the Stokes vectors of every node for the reverse mode, where
+// a.store is set) is that of sweep_j.cu where it fits. Against the general sweep: 48 x 48 x
+// 40, 5 directions, 21 frequencies with the store 0.32 -> 0.23 ms, 16 x 16 x 24 in FP64, 32
+// rays, 7 frequencies 1.30 -> 0.90 ms, 64 x 64 x 64, 5 directions 0.64 -> 0.64 ms; and its shape
+// need not be timed (64 x 64 x 64: 42 ms of the first call). The general sweep remains for the
+// media that the other does not know (dichroism, explicit media, biquadratic stencils), for
+// planes that do not fit, and where the packed inputs cannot be allocated.
+//
+// emergent_begin decides for ndir directions and has the inputs packed (the host can prepare
+// the directions meanwhile).
+template <typename Real>
+int emergent_begin(porta_ctx *c, int ndir, LaunchCfg &cfg, bool &packed)
+{
+    packed = false;
+    if (c->jk_form != 1 || c->d_dich || c->d_kexpl || c->interp == 2 || c->sc_faces || c->gsweep) return PORTA_OK;
+    const int fc = c->user_shape ? c->opt_cluster : 0, ff = c->user_shape ? c->opt_nu_group : 0;
+    const int rc = c->ns == 1 ? choose_launch<Real, 1>(c, cfg, fc, ff, ndir, true, c->n_nu, true)
+                              : choose_launch<Real, 4>(c, cfg, fc, ff, ndir, true, c->n_nu, true);
+    if (rc != PORTA_OK || ensure_jpack(c) != cudaSuccess) {
+        cudaGetLastError();
+        return PORTA_OK;
+    }
+    SweepArgs<Real> a = base_args<Real>(c);
+    a.pack = (const Real *)c->d_jpack;
+    const cudaError_t e = c->ns == 1 ? launch_jacc_prepare<Real, 1>(a, c->stream) : launch_jacc_prepare<Real, 4>(a, c->stream);
+    if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("emergent inputs: ") + cudaGetErrorString(e));
+    packed = true;
+    return PORTA_OK;
+}
+
+// the sweep itself: directions a.rays, their geometry in the general form a.geom and in the
+// relative form rel
+template <typename Real>
+int emergent_sweep(porta_ctx *c, SweepArgs<Real> a, const PlaneGeom<Real> *rel, int ndir, LaunchCfg cfg, bool packed)
+{
+    cudaError_t e = cudaSuccess;
+    if (packed) {
+        shape_args<Real>(c, a, cfg, true);
+        a.geom = rel;
+        a.nitems = ndir;
+        cfg.clusters = std::min(cfg.clusters, ndir * a.ngroups);
+        a.pack = (const Real *)c->d_jpack;
+        a.jerr = c->d_err + 1;
+        e = c->ns == 1 ? launch_jsweep<Real, 1>(a, cfg, c->stream) : launch_jsweep<Real, 4>(a, cfg, c->stream);
+    } else {
+        const int rc = c->ns == 1 ? emergent_shape<Real, 1>(c, a, ndir, cfg) : emergent_shape<Real, 4>(c, a, ndir, cfg);
+        if (rc) return rc;
+        e = c->ns == 1 ? launch_sweep<Real, 1>(a, MODE_EMERGENT, cfg, c->stream)
+                       : launch_sweep<Real, 4>(a, MODE_EMERGENT, cfg, c->stream);
+    }
+    return e == cudaSuccess ? PORTA_OK : fail(c, PORTA_ECUDA, std::string("emergent launch: ") + cudaGetErrorString(e));
+}
+
+// the emergent sweeps' error flag (synchronizes the stream)
+int emergent_check(porta_ctx *c)
+{
+    if (!c->h_flag) CK(cudaMallocHost((void **)&c->h_flag, sizeof(int)));
+    CK(cudaMemcpyAsync(c->h_flag, c->d_err + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    if (*c->h_flag) CK(cudaMemsetAsync(c->d_err + 1, 0, sizeof(int), c->stream));
+    if (*c->h_flag) return fail(c, PORTA_EKERNEL, "emergent: a strip's wait for its neighbour ran out");
+    return PORTA_OK;
+}
+
+// grow-only device buffer held by the context
+cudaError_t ensure_buf(void **p, size_t &cap, size_t need)
+{
+    if (need <= cap && *p) return cudaSuccess;
+    if (*p) pfree(*p);
+    *p = nullptr;
+    cap = 0;
+    cudaError_t e = pmalloc(p, need);
+    if (e == cudaSuccess) cap = need;
+    return e;
+}
+
+// The directions of a call on the device, in one buffer that the context keeps: their
+// geometry in the general form and in the relative form, the rays, and the box (with its
+// geometry at offset 0). (Three allocations and releases per call before.)
+template <typename Real>
+struct Directions {
+    const PlaneGeom<Real> *geom = nullptr, *rel = nullptr;
+    const RayDev<Real> *rays = nullptr;
+    const BoxDev *box = nullptr;
+};
+template <typename Real>
+cudaError_t put_directions(porta_ctx *c, int ndir, const double *mu, const double *chi, int box, Directions<Real> &d)
+{
+    const size_t n = (size_t)ndir * c->nz, gb = n * sizeof(PlaneGeom<Real>), rb = (size_t)ndir * sizeof(RayDev<Real>);
+    std::vector<unsigned char> h(2 * gb + sizeof(BoxDev) + rb);
+    PlaneGeom<Real> *g = reinterpret_cast<PlaneGeom<Real> *>(h.data());
+    BoxDev *b = reinterpret_cast<BoxDev *>(h.data() + 2 * gb);
+    RayDev<Real> *r = reinterpret_cast<RayDev<Real> *>(b + 1);
+    for (int i = 0; i < ndir; ++i) {
+        PlaneGeom<Real> *gi = g + (size_t)i * c->nz;
+        plane_geometry<Real>(c->nx, c->ny, c->nz, c->lx, c->ly, c->z.data(), mu[i], chi[i], gi);
+        relative_geometry(gi, c->nz, gi + n);
+        r[i] = ray_dev<Real>(mu[i], chi[i]);
+    }
+    *b = c->boxes[box];
+    b->geom0 = 0;
+    cudaError_t e = ensure_buf(&c->d_dirs, c->dirs_bytes, h.size());
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_dirs, h.data(), h.size(), cudaMemcpyHostToDevice, c->stream);
+    const unsigned char *p = static_cast<const unsigned char *>(c->d_dirs);
+    d.geom = reinterpret_cast<const PlaneGeom<Real> *>(p);
+    d.rel = d.geom + n;
+    d.box = reinterpret_cast<const BoxDev *>(p + 2 * gb);
+    d.rays = reinterpret_cast<const RayDev<Real> *>(d.box + 1);
+    return e;
+}
+
 template <typename Real>
 int emergent_t(porta_ctx *c, int ndir, const double *mu, const double *chi, double *dout, int box)
 {
-    std::vector<PlaneGeom<Real>> geom((size_t)ndir * c->nz);
-    std::vector<RayDev<Real>> rays(ndir);
-    for (int d = 0; d < ndir; ++d) {
-        plane_geometry<Real>(c->nx, c->ny, c->nz, c->lx, c->ly, c->z.data(), mu[d], chi[d], geom.data() + (size_t)d * c->nz);
-        rays[d] = ray_dev<Real>(mu[d], chi[d]);
-    }
-    PlaneGeom<Real> *dg = nullptr;
-    RayDev<Real> *dr = nullptr;
-    BoxDev *dbox = nullptr;
-    CK(dalloc(&dg, geom.size()));
-    cudaError_t e2 = dalloc(&dr, rays.size());
-    if (e2 == cudaSuccess) e2 = pmalloc(&dbox, sizeof(BoxDev));
-    if (e2 != cudaSuccess) {
-        pfree(dg);
-        if (dr) pfree(dr);
-        return fail(c, PORTA_ENOMEM, "emergent: device allocation");
-    }
-    int rc = PORTA_OK;
+    check_global_sweep(c);
+    LaunchCfg cfg{};
+    bool packed = false;
+    int rc = emergent_begin<Real>(c, ndir, cfg, packed);
+    if (rc) return rc;
+    Directions<Real> dirs;
+    cudaError_t e = put_directions<Real>(c, ndir, mu, chi, box, dirs);
+    if (e != cudaSuccess) return fail(c, PORTA_ENOMEM, "emergent: device allocation");
     do {
-        // the box of this call (a line of a multilevel context shares the grid): its
-        // voxels, with the per-direction geometry of this call (geometry offset 0)
-        BoxDev hb = c->boxes[box];
-        hb.geom0 = 0;
-        cudaError_t e = cudaMemcpyAsync(dg, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dr, rays.data(), rays.size() * sizeof(rays[0]), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dbox, &hb, sizeof(hb), cudaMemcpyHostToDevice, c->stream);
-        if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, cudaGetErrorString(e)); break; }
         SweepArgs<Real> a = base_args<Real>(c);
-        a.boxes = dbox;
-        a.geom = dg;
-        a.rays = dr;
+        // (a line of a multilevel context shares the grid: its own box's voxels)
+        a.boxes = dirs.box;
+        a.geom = dirs.geom;
+        a.rays = dirs.rays;
         a.out = dout;
-        check_global_sweep(c);
         if (c->sc_faces || c->gsweep) {
             // short characteristics on cell faces, or the plane placement of the
             // global-memory sweep (faces.cu), its own work buffer
@@ -151,32 +244,11 @@ int emergent_t(porta_ctx *c, int ndir, const double *mu, const double *chi, doub
             else if (flag & 2) rc = fail(c, PORTA_ENOTCONV, "emergent (faces): a plane of face points did not converge");
             break;
         }
-        LaunchCfg cfg{};
-        rc = c->ns == 1 ? emergent_shape<Real, 1>(c, a, ndir, cfg) : emergent_shape<Real, 4>(c, a, ndir, cfg);
-        if (rc) break;
-        e = c->ns == 1 ? launch_sweep<Real, 1>(a, MODE_EMERGENT, cfg, c->stream)
-                       : launch_sweep<Real, 4>(a, MODE_EMERGENT, cfg, c->stream);
-        if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, std::string("emergent launch: ") + cudaGetErrorString(e)); break; }
-        e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) rc = fail(c, PORTA_ECUDA, std::string("emergent: ") + cudaGetErrorString(e));
+        rc = emergent_sweep<Real>(c, a, dirs.rel, ndir, cfg, packed);
+        if (rc == PORTA_OK) rc = emergent_check(c);
     } while (0);
-    cudaStreamSynchronize(c->stream);
-    pfree(dg);
-    pfree(dr);
-    pfree(dbox);
+    if (rc != PORTA_OK) cudaStreamSynchronize(c->stream);
     return rc;
-}
-
-// grow-only device buffer held by the context
-cudaError_t ensure_buf(void **p, size_t &cap, size_t need)
-{
-    if (need <= cap && *p) return cudaSuccess;
-    if (*p) pfree(*p);
-    *p = nullptr;
-    cap = 0;
-    cudaError_t e = pmalloc(p, need);
-    if (e == cudaSuccess) cap = need;
-    return e;
 }
 
 const int kAdjThreads = 256;   // maximum threads per CTA of the adjoint kernel
@@ -246,24 +318,20 @@ template <typename Real>
 int emergent_vjp_t(porta_ctx *c, int ndir, const double *mu, const double *chi, const double *dgrad, double *dout,
                    double *dg_chi, double *dg_e, double *dg_b, double *dg_rho = nullptr)
 {
-    std::vector<PlaneGeom<Real>> geom((size_t)ndir * c->nz);
-    std::vector<RayDev<Real>> rays(ndir);
-    for (int d = 0; d < ndir; ++d) {
-        plane_geometry<Real>(c->nx, c->ny, c->nz, c->lx, c->ly, c->z.data(), mu[d], chi[d], geom.data() + (size_t)d * c->nz);
-        rays[d] = ray_dev<Real>(mu[d], chi[d]);
-    }
     const long long nxy = (long long)c->nx * c->ny;
-    PlaneGeom<Real> *dg = nullptr;
-    RayDev<Real> *dr = nullptr;
     double *scratch_out = nullptr;
-    CK(dalloc(&dg, geom.size()));
-    cudaError_t e2 = dalloc(&dr, rays.size());
+    LaunchCfg cfg{};
+    bool packed = false;
+    int rc = emergent_begin<Real>(c, ndir, cfg, packed);
+    if (rc) return rc;
+    Directions<Real> dirs;
+    cudaError_t e2 = put_directions<Real>(c, ndir, mu, chi, 0, dirs);
     if (e2 == cudaSuccess && !dout) e2 = dalloc(&scratch_out, (size_t)ndir * c->n_nu * nxy * c->ns);
-    int rc = PORTA_OK;
+    const PlaneGeom<Real> *dg = dirs.geom;
+    const RayDev<Real> *dr = dirs.rays;
     do {
         if (e2 != cudaSuccess) { rc = fail(c, PORTA_ENOMEM, "emergent_vjp: device allocation"); break; }
-        cudaError_t e = cudaMemcpyAsync(dg, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dr, rays.data(), rays.size() * sizeof(rays[0]), cudaMemcpyHostToDevice, c->stream);
+        cudaError_t e = cudaSuccess;
         if (e == cudaSuccess)
             e = ensure_buf(&c->d_tape, c->tape_bytes, (size_t)ndir * c->n_nu * c->nvox * c->ns * sizeof(Real));
         if (e != cudaSuccess) { rc = fail(c, PORTA_ENOMEM, std::string("emergent_vjp: ") + cudaGetErrorString(e)); break; }
@@ -276,14 +344,11 @@ int emergent_vjp_t(porta_ctx *c, int ndir, const double *mu, const double *chi, 
         a.rays = dr;
         a.out = dout ? dout : scratch_out;
         a.store = (Real *)c->d_tape;
-        LaunchCfg cfg{};
-        rc = c->ns == 1 ? emergent_shape<Real, 1>(c, a, ndir, cfg) : emergent_shape<Real, 4>(c, a, ndir, cfg);
-        if (rc) break;
         e = cudaEventRecord(c->adj_ev[0], c->stream);
-        if (e == cudaSuccess)
-            e = c->ns == 1 ? launch_sweep<Real, 1>(a, MODE_EMERGENT, cfg, c->stream)
-                           : launch_sweep<Real, 4>(a, MODE_EMERGENT, cfg, c->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(c->adj_ev[1], c->stream);
+        if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, std::string("emergent_vjp: ") + cudaGetErrorString(e)); break; }
+        rc = emergent_sweep<Real>(c, a, dirs.rel, ndir, cfg, packed);
+        if (rc) break;
+        e = cudaEventRecord(c->adj_ev[1], c->stream);
         if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, std::string("emergent_vjp forward: ") + cudaGetErrorString(e)); break; }
         // adjoint: launch shape forced, or timed once per direction count over
         // every fitting shape (each trial overwrites the same outputs)
@@ -361,14 +426,13 @@ int emergent_vjp_t(porta_ctx *c, int ndir, const double *mu, const double *chi, 
         if (e == cudaSuccess) e = cudaEventRecord(c->adj_ev[2], c->stream);
         if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, std::string("emergent_vjp adjoint: ") + cudaGetErrorString(e)); break; }
         c->last_adj = acfg;
-        e = cudaStreamSynchronize(c->stream);
+        rc = emergent_check(c);
+        if (rc) break;
         if (e == cudaSuccess && !tune) e = cudaEventElapsedTime(&c->adj_fwd_ms, c->adj_ev[0], c->adj_ev[1]);
         if (e == cudaSuccess) e = cudaEventElapsedTime(&c->adj_rev_ms, c->adj_ev[1], c->adj_ev[2]);
         if (e != cudaSuccess) rc = fail(c, PORTA_ECUDA, std::string("emergent_vjp: ") + cudaGetErrorString(e));
     } while (0);
     cudaStreamSynchronize(c->stream);
-    pfree(dg);
-    pfree(dr);
     if (scratch_out) pfree(scratch_out);
     return rc;
 }
@@ -418,18 +482,19 @@ int jkq_vjp_t(porta_ctx *c, const double *dgj, const double *dgl, double *dg_chi
     e = ensure_buf((void **)&c->d_gacc, c->gacc_bytes, (size_t)maxcl * 10 * c->nvox * sizeof(Real));
     if (e != cudaSuccess) return fail(c, PORTA_ENOMEM, "iterate_vjp: accumulator allocation");
     // forward: Stokes vectors of every node for rays r0 .. r0 + n - 1
+    LaunchCfg fcfg{};
+    bool packed = false;
+    rc = emergent_begin<Real>(c, nb, fcfg, packed);
+    if (rc) return rc;
     auto forward = [&](int r0, int n) -> int {
         SweepArgs<Real> a = base_args<Real>(c);
         a.geom = (const PlaneGeom<Real> *)c->d_geom + (size_t)r0 * c->nz;
         a.rays = (const RayDev<Real> *)c->d_rays + r0;
         a.out = scratch;
         a.store = (Real *)c->d_tape;
-        LaunchCfg cfg{};
-        int r = c->ns == 1 ? emergent_shape<Real, 1>(c, a, n, cfg) : emergent_shape<Real, 4>(c, a, n, cfg);
-        if (r) return r;
-        e = c->ns == 1 ? launch_sweep<Real, 1>(a, MODE_EMERGENT, cfg, c->stream)
-                       : launch_sweep<Real, 4>(a, MODE_EMERGENT, cfg, c->stream);
-        return e == cudaSuccess ? PORTA_OK : fail(c, PORTA_ECUDA, std::string("iterate_vjp: ") + cudaGetErrorString(e));
+        size_t planes = 0;
+        for (const BoxDev &b : c->boxes) planes += b.nz;
+        return emergent_sweep<Real>(c, a, a.geom + (size_t)c->nray * planes, n, fcfg, packed);
     };
     // reverse: the J^K_Q and Lambda-bar* terms of the same rays
     auto reverse = [&](int r0, int n, LaunchCfg k) -> int {
@@ -512,6 +577,7 @@ int jkq_vjp_t(porta_ctx *c, const double *dgj, const double *dgl, double *dg_chi
         c->it_ms[4] += t;
         c->last_adj = acfg;
     }
+    if (rc == PORTA_OK) rc = emergent_check(c);
     cudaStreamSynchronize(c->stream);
     return rc;
 }

@@ -10,6 +10,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -109,24 +111,52 @@ void plane_geometry(int nx, int ny, int nz, double lx, double ly, const double *
     }
 }
 
+// the next larger or smaller value of a positive normal one
+inline float neighbour(float x, bool up)
+{
+    std::int32_t b;
+    std::memcpy(&b, &x, sizeof(b));
+    b += up ? 1 : -1;
+    std::memcpy(&x, &b, sizeof(b));
+    return x;
+}
+inline double neighbour(double x, bool up)
+{
+    std::int64_t b;
+    std::memcpy(&b, &x, sizeof(b));
+    b += up ? 1 : -1;
+    std::memcpy(&x, &b, sizeof(b));
+    return x;
+}
+
 // the same for the J^K_Q sweep, which uses the bilinear weights relative to the first one:
 // in place of (tx, ty, ds, pad2) it reads u = t / (1 - t) along x and y, the first weight
 // (1 - tx) (1 - ty), and ds / 2. A factor 1 - t that rounds to 0 is held at the rounding unit of 1.
-// The first weight is what makes the rounded weights add up to 1: planes of equal spacing
-// have equal weights, and a ray through a transparent medium would gather their excess (the
-// products of the unrounded factors left 2e-8 per plane on average over a quadrature's rays).
+// The first weight is what makes the rounded weights add up to 1, rounded up or down so that
+// the sums' product over a ray's planes stays at 1: planes of equal spacing have equal
+// weights, and a ray through a transparent medium would gather their excess (2e-8 per plane
+// rms, 1e-6 after 64 planes).
 template <typename Real>
-PlaneGeom<Real> relative_geometry(const PlaneGeom<Real> &p)
+void relative_geometry(const PlaneGeom<Real> *p, int nz, PlaneGeom<Real> *r)
 {
     const double unit = sizeof(Real) == 4 ? 5.9604644775390625e-08 : 1.1102230246251565e-16;
-    const double mx = std::max(1.0 - (double)p.tx, unit), my = std::max(1.0 - (double)p.ty, unit);
-    PlaneGeom<Real> r = p;
-    r.tx = (Real)(p.tx / mx);
-    r.ty = (Real)(p.ty / my);
-    const Real uxy = r.tx * r.ty;        // as the sweep forms it
-    r.ds = (Real)(1.0 / (1.0 + (double)r.tx + (double)r.ty + (double)uxy));
-    r.pad2 = (Real)(0.5 * p.ds);
-    return r;
+    double gathered = 0.0;
+    for (int q = 0; q < nz; ++q) {
+        const double mx = std::max(1.0 - (double)p[q].tx, unit), my = std::max(1.0 - (double)p[q].ty, unit);
+        r[q] = p[q];
+        r[q].tx = (Real)(p[q].tx / mx);
+        r[q].ty = (Real)(p[q].ty / my);
+        r[q].pad2 = (Real)(0.5 * p[q].ds);
+        const Real uxy = r[q].tx * r[q].ty;        // as the sweep forms it
+        const double sum = 1.0 + (double)r[q].tx + (double)r[q].ty + (double)uxy;
+        const Real w = (Real)(1.0 / sum);
+        const double e0 = (double)w * sum - 1.0;
+        const Real other = neighbour(w, e0 < 0.0);
+        const double e1 = (double)other * sum - 1.0;
+        const bool swap = std::fabs(gathered + e1) < std::fabs(gathered + e0);
+        r[q].ds = swap ? other : w;
+        if (q > 0) gathered += swap ? e1 : e0;
+    }
 }
 
 template <typename Real>
@@ -219,11 +249,12 @@ int jsweep_tots(const porta_ctx *c, int C, int F, int *threads_out)
 // Cycles of one plane of one pass of the J^K_Q sweep in a CTA: a chain of fixed length
 // (barrier, geometry, sources of the corners, sums), the units of the points' rounds one
 // after the other, and a round of the nodes' filling, whose length grows little with the
-// frequencies; in FP64 the operations of all points besides, at 1/64 of the FP32 rate.
-// Fitted to forced shapes of boxes from 8 x 8 x 16 to 64 x 64 x 64 (C 1 to 16, every number of
-// passes): the shape it picks was the fastest of all, or within 12% of it, for each.
+// frequencies; in FP64 also the operations of all points and of `share` CTAs at 1/64 of the
+// FP32 rate, whichever is longer (smoothly). Fitted to forced shapes of boxes from 8 x 8 x 16
+// to 64 x 64 x 64 (C 1 to 16, every number of passes): the shape it picks was the fastest of
+// all, or within 13% of it, for each.
 template <typename Real, int NS>
-double jsweep_plane_cost(int nx, int R, int F, int threads)
+double jsweep_plane_cost(int nx, int R, int F, int threads, int share)
 {
     const int W = jsweep_lanes<Real>(), FX = (F + W - 1) / W;
     const int pts = R * nx, nodes = (R + 2) * nx;
@@ -233,16 +264,18 @@ double jsweep_plane_cost(int nx, int R, int F, int threads)
     if (sizeof(Real) == 4)
         return NS == 4 ? 2660.0 + 1106.0 * units + fills * (1190.0 + 151.0 * FX)
                        : 3180.0 + 778.0 * units + fills * (339.0 + 6.0 * FX);
-    const double warps = (double)((pts + 31) / 32) * FX, nwarps = (double)((nodes + 31) / 32) * FX;
-    return NS == 4 ? 5610.0 + 5520.0 * units + fills * (2790.0 + 1200.0 * FX) + 1630.0 * warps + 611.0 * nwarps
-                   : 3550.0 + 17166.0 * units + fills * 550.0 * FX + 600.0 * nwarps;
+    const double chain = NS == 4 ? 5680.0 + 10000.0 * units + fills * (2280.0 + 2330.0 * FX)
+                                 : 6720.0 + 5580.0 * units + fills * 2030.0 * FX;
+    const double pipe = share * (NS == 4 ? 3930.0 : 2120.0) * ((pts + 31) / 32) * FX;
+    // (unevenly shared SMs: the clusters on the fuller ones end last)
+    return (NS == 4 && share > 1 ? 1.2 : 1.0) * std::sqrt(std::sqrt(chain * chain * chain * chain + pipe * pipe * pipe * pipe));
 }
 
 // Launch shape of the J^K_Q sweep: every cluster size, every number of passes whose
 // frequencies fit in shared memory; the (box, ray) items, in FP32 the passes of a ray each,
 // spread over the resident clusters.
 template <typename Real, int NS>
-int choose_jsweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, int NU)
+int choose_jsweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, int NU, bool emg)
 {
     double best_cost = 1e300;
     best = LaunchCfg{};
@@ -269,23 +302,23 @@ int choose_jsweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int n
             const int smem = jsweep_smem_bytes<Real, NS>(nodes, ipts, tots, F);
             if (smem > kJSmemLimit) continue;
             const int G = jsweep_groups<Real>(NU, F);
-            const int parts = sizeof(Real) == 4 ? G : 1;
+            const int parts = sizeof(Real) == 4 || emg ? G : 1;
             const long long n = (long long)nitems * parts;
-            double total = 0.0, item_max = 0.0;
-            for (const BoxDev &b : c->boxes) {
-                const double item =
-                    (double)b.nz * (G / parts) * jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads);
-                total += item * c->nray * parts;
-                item_max = std::max(item_max, item);
-            }
-            // (CTAs on one SM hide one another's chains, but share its FP64 pipe)
             auto cost = [&](int ncl) {
-                const double share = sizeof(Real) == 8 ? std::max(1, (ncl * C + nsm - 1) / nsm) : 1;
-                return share * (c->nbox == 1 ? (double)((n + ncl - 1) / ncl) * item_max : std::max(total / ncl, item_max) * 1.05);
+                const int share = std::max(1, (ncl * C + nsm - 1) / nsm);     // CTAs on one SM
+                double total = 0.0, item_max = 0.0;
+                for (const BoxDev &b : c->boxes) {
+                    const double item = (double)b.nz * (G / parts) *
+                                        jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads, share);
+                    total += item * c->nray * parts;
+                    item_max = std::max(item_max, item);
+                }
+                return c->nbox == 1 || emg ? (double)((n + ncl - 1) / ncl) * item_max : std::max(total / ncl, item_max) * 1.05;
             };
             // no better even with every SM's thread slots taken
-            const int per_sm = std::min(2048 / threads, 227 * 1024 / (smem + 1024));
-            const double bound = cost(std::max(1, nsm * (sizeof(Real) == 8 ? 1 : std::max(1, per_sm)) / C));
+            const int per_sm = std::max(1, std::min(2048 / threads, 227 * 1024 / (smem + 1024)));
+            double bound = 1e300;
+            for (int k = 1; k <= per_sm && bound >= best_cost; ++k) bound = std::min(bound, cost(std::max(1, nsm * k / C)));
             if (best.cluster > 0 && bound >= best_cost) continue;
             int act = 0;
             if (jsweep_max_active_clusters<Real, NS>(C, smem, threads, &act) != cudaSuccess) {
@@ -383,20 +416,21 @@ int choose_sweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int ni
     return best.cluster > 0 ? PORTA_OK : PORTA_EINVAL;
 }
 
-// The shape of a context's sweep (jk: the J^K_Q sweep's). It follows from sizes and options
+// The shape of a context's sweep (jk: the J^K_Q sweep's; emg: its form for emergent profiles). It follows from sizes and options
 // alone and takes some tens of occupancy queries, so the context keeps what it chose.
 template <typename Real, int NS>
-int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, bool jk = false, int nnu = 0)
+int choose_launch(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int nitems, bool jk = false, int nnu = 0,
+                  bool emg = false)
 {
     const int NU = nnu > 0 ? nnu : c->n_nu;     // frequencies swept
     if (force_f > NU) force_f = NU;
-    const std::array<int, 8> key = {force_c, force_f, nitems, jk ? c->jk_form : 0, NU, c->d_dich != nullptr, c->interp, c->d_kexpl != nullptr};
+    const std::array<int, 8> key = {force_c, force_f, nitems, jk ? c->jk_form + (emg ? 2 : 0) : 0, NU, c->d_dich != nullptr, c->interp, c->d_kexpl != nullptr};
     for (const auto &s : c->shapes)
         if (s.first == key) {
             best = s.second;
             return PORTA_OK;
         }
-    const int rc = jk && c->jk_form == 1 ? choose_jsweep<Real, NS>(c, best, force_c, force_f, nitems, NU)
+    const int rc = jk && c->jk_form == 1 ? choose_jsweep<Real, NS>(c, best, force_c, force_f, nitems, NU, emg)
                                          : choose_sweep<Real, NS>(c, best, force_c, force_f, nitems, NU, jk);
     if (rc == PORTA_OK) {
         if (c->shapes.size() >= 64) c->shapes.clear();
@@ -454,6 +488,8 @@ void shape_args(porta_ctx *c, SweepArgs<Real> &a, const LaunchCfg &cfg, bool jk 
 }
 
 // api.cu
+// the packed inputs of sweep_j.cu, allocated on first use
+cudaError_t ensure_jpack(porta_ctx *c);
 void free_all(porta_ctx *c);
 bool finite_host(const double *x, long long n);
 // copy n doubles from a caller buffer (host or device) into device memory

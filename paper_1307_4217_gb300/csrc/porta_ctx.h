@@ -94,7 +94,10 @@ struct porta_ctx {
     int *d_items = nullptr;        // nbox*nray work items ordered by decreasing cost
     int *d_tune_items = nullptr;   // strided sample of the work items for the autotuner
     int n_tune = 0;
-    int *d_err = nullptr;
+    int *d_err = nullptr;               // error flags: formal solution, emergent sweeps
+    int *h_flag = nullptr;              // page-locked, receives the latter
+    void *d_dirs = nullptr;             // directions of the last emergent call (put_directions)
+    size_t dirs_bytes = 0;
     // CUDA graph of one Jacobi iteration (porta_run_iterations)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;

@@ -151,6 +151,7 @@ template <typename Real, int NS>
 int jsweep_smem_bytes(int nodes, int ipts, int tots, int F);
 template <typename Real, int NS>
 cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out);
+// (a.out set: the emergent Stokes profiles of the nitems directions of a.rays, a.geom)
 template <typename Real, int NS>
 cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st);
 // the same for planes too wide for sweep_j.cu's shared memory (sweep_jw.cu: three ring slots

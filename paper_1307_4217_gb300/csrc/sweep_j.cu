@@ -1,7 +1,9 @@
 // Formal solution for the radiation-field tensors (Sec. 3 of Stepan & Trujillo
 // Bueno 2013): the short-characteristics BESSER sweep of every ray direction
 // and frequency, fused with the frequency integration of the Stokes parameters
-// and Lambda* that feeds J^K_Q (Eq. 1, Eq. 14) and the Jacobi update.
+// and Lambda* that feeds J^K_Q (Eq. 1, Eq. 14) and the Jacobi update; and the same
+// sweep for emergent Stokes profiles, with the Stokes vectors of every node for the
+// reverse mode where asked.
 //
 // The decomposition is that of the general sweep (sweep.cu): one thread-block
 // cluster per ray and frequency group at a time, the plane split into strips of
@@ -33,9 +35,9 @@
 // FP32; jsweep_plane_cost), whatever the strip, so a pass has few units over as many points
 // as the threads hold. Against the kernel of sweep_jw.cu, which this one replaces where it
 // fits (one frequency of one point per thread and step, one cluster barrier per plane), ms
-// per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 18.0, 33 x 27 x 41 x
-// 80 x 21 1.91 -> 1.22, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.8, 64 x 64 x 48 x 160 x 31
-// x 2 lines, unpolarized, 46.4 -> 32.4 (with the rate equations).
+// per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 17.9, 33 x 27 x 41 x
+// 80 x 21 1.91 -> 1.21, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.4, 64 x 64 x 48 x 160 x 31
+// x 2 lines, unpolarized, 46.4 -> 31.8 (with the rate equations).
 //
 // Shared memory per CTA (X: 8 bytes, a frequency unit):
 //   ring[4][nodes]        source vectors, Real
@@ -194,10 +196,18 @@ __device__ __forceinline__ double xadd(double a, double b) { return a + b; }
 __device__ __forceinline__ float2 xneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ double xneg(double a) { return -a; }
 __device__ __forceinline__ float2 xrcp(float2 a) { return make_float2(rcp(a.x), rcp(a.y)); }
-__device__ __forceinline__ double xrcp(double a) { return rcp(a); }
+// (FP64 operations run at 2 lanes per cycle and SM here, 1/64 of the FP32 rate: the hardware's
+// 20-bit reciprocal and two Newton steps, within an ulp for normal a, are 4 of them)
+__device__ __forceinline__ double xrcp(double a)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    y = fma(y, fma(-a, y, 1.0), y);
+    return fma(y, fma(-a, y, 1.0), y);
+}
 // -1 / a
 __device__ __forceinline__ float2 xnrcp(float2 a) { return make_float2(rcp(-a.x), rcp(-a.y)); }
-__device__ __forceinline__ double xnrcp(double a) { return rcp(-a); }
+__device__ __forceinline__ double xnrcp(double a) { return xrcp(-a); }
 // the same Real times both lanes (scalar operations: a pair made of one value costs a move)
 __device__ __forceinline__ float2 xms(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
 __device__ __forceinline__ double xms(double s, double a) { return s * a; }
@@ -207,7 +217,12 @@ __device__ __forceinline__ double xfs(double s, double a, double c) { return fma
 __device__ __forceinline__ float xdot(float2 a, float2 b, float s) { return fmaf(a.y, b.y, fmaf(a.x, b.x, s)); }
 __device__ __forceinline__ double xdot(double a, double b, double s) { return fma(a, b, s); }
 __device__ __forceinline__ float2 xprofile(float2 xs) { return make_float2(profile_shape(xs.x), profile_shape(xs.y)); }
-__device__ __forceinline__ double xprofile(double xs) { return profile_shape(xs); }
+// (capped far in the wings, at 1e-282 of the line centre, so that eta_I stays a normal number)
+__device__ __forceinline__ double xprofile(double xs)
+{
+    const double x = xs * xs;
+    return exp(-(__double2hiint(x) > __double2hiint(650.0) ? 650.0 : x));
+}
 // 1 - a^2
 __device__ __forceinline__ float2 xdet(float2 a) { return make_float2(1.0f - a.x * a.x, 1.0f - a.y * a.y); }
 __device__ __forceinline__ double xdet(double a) { return 1.0 - a * a; }
@@ -223,11 +238,49 @@ __device__ __forceinline__ double xlane(double a, int) { return a; }
 // source functions, within 3e-7 and 8e-7. The polynomials are evaluated for both lanes
 // always; the closed forms replace them where some lane needs them. (Three polynomials, an
 // exponential per lane and the sums: 26 instructions more per unit, 3% of the sweep's time.)
+// (In FP64 below t = 1, to 5e-17; 26 operations instead of an exponential, a reciprocal, the
+// closed forms and, below 0.18, three series.)
 template <typename X> struct XCoef { X e, e0, wm, wo, wc; };
 __device__ __forceinline__ XCoef<double> xcoef(double t)
 {
-    const Coef<double> c = coefficients(t);
-    return {c.e, c.wm + c.wo + c.wc, c.wm, c.wo, c.wc};
+    XCoef<double> c;
+    if (t < 1.0) {
+        double m = fma(t, -1.1202256902396886e-09, 1.9558584056821613e-08), o = fma(t, 2.1752747810916859e-10, -3.9450135294101958e-09);
+        m = fma(t, m, -2.2723481708323534e-07);
+        o = fma(t, o, 4.9804374537587804e-08);
+        m = fma(t, m, 2.2524008032884722e-06);
+        o = fma(t, o, -5.5090033985190619e-07);
+        m = fma(t, m, -1.9839818101854985e-05);
+        o = fma(t, o, 5.5113331078707397e-06);
+        m = fma(t, m, 0.00015432036885733235);
+        o = fma(t, o, -4.9603129765952493e-05);
+        m = fma(t, m, -0.0010416664919878616);
+        o = fma(t, o, 0.00039682538720382121);
+        m = fma(t, m, 0.0059523809209458198);
+        o = fma(t, o, -0.0027777777765696106);
+        m = fma(t, m, -0.027777777774420587);
+        o = fma(t, o, 0.016666666666588639);
+        m = fma(t, m, 0.099999999999813557);
+        o = fma(t, o, -0.083333333333331358);
+        m = fma(t, m, -0.24999999999999592);
+        o = fma(t, o, 0.33333333333333331);
+        m = fma(t, m, 0.33333333333333331);
+        c.wm = t * m;
+        c.wo = t * o;
+        const double ht = 0.5 * t;
+        c.e0 = fma(-t, fma(-ht, c.wo, ht), t);
+        c.e = 1.0 - c.e0;
+        c.wc = (c.e0 - c.wm) - c.wo;
+    } else {
+        const double it = xrcp(t);
+        c.e = exp(-t);
+        c.e0 = 1.0 - c.e;
+        const double h2 = fma(-2.0 * c.e0, it, 2.0);
+        c.wo = fma(-h2, it, 1.0);
+        c.wc = 2.0 * it * (h2 - c.e0);
+        c.wm = fma(-c.e, fma(t, t + 2.0, 2.0), 2.0) * (it * it);
+    }
+    return c;
 }
 __device__ __forceinline__ XCoef<float2> xcoef(float2 t)
 {
@@ -273,20 +326,26 @@ __device__ __forceinline__ XCoef<float2> xcoef(float2 t)
 // both differences and w have one sign, so the interval tests compare magnitudes: |w| >
 // |d_M| is c_M outside [y_M, y_O] (steps 5-6, c_M = y_M), |w| > |r d_P| is c_P outside
 // [y_O, y_P] (steps 7-9). na = -a, nr = -r.
-template <typename Real> __device__ __forceinline__ Real cp_select(Real dm, Real w, Real rdp, Real te)
+__device__ __forceinline__ float cp_select(float dm, float w, float rdp, float te)
 {
-    Real c = fabs(w) > fabs(rdp) ? rdp : w;
-    c = fabs(w) > fabs(dm) ? dm : c;
-    return te < Real(0) ? c : Real(0);
+    float c = fabsf(w) > fabsf(rdp) ? rdp : w;
+    c = fabsf(w) > fabsf(dm) ? dm : c;
+    return te < 0.0f ? c : 0.0f;
 }
 __device__ __forceinline__ float2 xoffset(float2 dm, float2 ndp, float2 na, float2 b, float2 nr)
 {
     const float2 w = xfma(na, ndp, xmul(b, dm)), rdp = xmul(nr, ndp), te = xmul(dm, ndp);
     return make_float2(cp_select(dm.x, w.x, rdp.x, te.x), cp_select(dm.y, w.y, rdp.y, te.y));
 }
+// (the comparisons on the bits, in the integer pipe; where a difference is 0, so is the
+// selected value, and step 2 needs the signs alone)
 __device__ __forceinline__ double xoffset(double dm, double ndp, double na, double b, double nr)
 {
-    return cp_select(dm, fma(na, ndp, b * dm), nr * ndp, dm * ndp);
+    const double w = fma(na, ndp, b * dm), rdp = nr * ndp;
+    auto mag = [](double x) { return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull; };
+    double c = mag(w) > mag(rdp) ? rdp : w;
+    c = mag(w) > mag(dm) ? dm : c;
+    return (__double2hiint(dm) ^ __double2hiint(ndp)) < 0 ? c : 0.0;
 }
 
 // ---- shared memory by 32-bit address -------------------------------------------------
@@ -294,6 +353,11 @@ __device__ __forceinline__ double xoffset(double dm, double ndp, double na, doub
 // access). volatile keeps the accesses' order against barriers; stores clobber memory.
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void lds(unsigned a, int &x) { asm volatile("ld.shared.s32 %0, [%1];" : "=r"(x) : "r"(a)); }
+__device__ __forceinline__ void lds4i(unsigned a, int *x)
+{
+    asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(a));
+}
+__device__ __forceinline__ int wrap(int x, int n) { return (int)min((unsigned)x, (unsigned)(x - n)); }
 __device__ __forceinline__ void lds(unsigned a, float &x) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(a)); }
 __device__ __forceinline__ void lds(unsigned a, double &x) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(x) : "r"(a)); }
 __device__ __forceinline__ void lds(unsigned a, float2 &x)
@@ -449,13 +513,18 @@ __device__ __forceinline__ void bar_wait(unsigned bar, unsigned parity, volatile
 struct JBars { unsigned full, freed; volatile int *dead; };   // [2] words of 8 bytes each
 struct JPhase { unsigned full0, full1, freed0, freed1; };
 
-template <typename Real, int NS, bool PROBE>
+// what a sweep leaves: the J^K_Q and Lambda* sums (SUMS; with one ray's Stokes vectors and
+// Lambda*, PROBE), or the emergent Stokes profiles and, for the reverse mode, the Stokes
+// vectors of every node (EMERGENT: no sums, no profile normalization)
+enum JMode { SUMS = 0, PROBE_RAY = 1, EMERGENT = 2 };
+template <typename Real, int NS, int MODE>
 __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsigned sbase, const JSmem &sm,
                                             const JBars &bars, JPhase &ph, const unsigned sray, int box, int m, int g,
                                             int rank, int C)
 {
     using X = typename XOf<Real>::X;
     using W = JW<Real, NS>;
+    constexpr bool PROBE = MODE == PROBE_RAY, EMG = MODE == EMERGENT;
     constexpr int XW = jsweep_lanes<Real>();
     constexpr int NA = W::na;
     constexpr unsigned SZ = sizeof(Real);
@@ -533,21 +602,29 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
     };
 
     // Inputs of plane q's nodes on their way to shared memory; the thread that asked for a
-    // node's values is the one that fills the node a phase later.
+    // node's values is the one that fills the node a phase later. (Wrapped by an unsigned
+    // minimum: x - n is huge below n.)
+    const int jown = row0 + rowt - 1 + (row0 + rowt == 0 ? ny : 0) - (row0 + rowt > ny ? ny : 0);
     auto fetch = [&](int q) {
-        int lr = rowt, c = colt;
+        if (rtid >= nn) return;
+        int g4[4];
+        lds4i(geo + (q & 7) * GB, g4);
+        const int base = vox0 + g4[2] * ny * nx;
+        int j = jown, c = colt;
         for (int idx = rtid; idx < nn; idx += nt) {
-            const int v = point_voxel(q, lr - 1, c);
+            const int pi = wrap(c + g4[0], nx), pj = wrap(j + g4[1], ny);
+            const int v = base + pj * nx + pi;
             const Real *src = a.pack + (size_t)(unsigned)v * W::staged;
             const unsigned d = sbase + sm.stage + idx * 16;
             sts(sbase + sm.stv + idx * 4, v);
-            copy_async(sbase + sm.stw + idx * SZ, invn + v);
-            if (a.jacc) copy_async(sbase + sm.ste + idx * 4, a.jexp + v);
+            if (!EMG) copy_async(sbase + sm.stw + idx * SZ, invn + v);
+            if (!EMG && a.jacc) copy_async(sbase + sm.ste + idx * 4, a.jexp + v);
 #pragma unroll
             for (int h = 0; h < SCH; ++h) copy_async16(d + h * nodes * 16, src + h * W::per);
             c += dc;
-            lr += dl;
-            if (c >= nx) { c -= nx; ++lr; }
+            j += dl;
+            if (c >= nx) { c -= nx; ++j; }
+            j = wrap(wrap(j, ny), ny);      // (from the row before the strip to the one after: up to 2 ny)
         }
     };
 
@@ -573,23 +650,24 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
             Real t[20];
 #pragma unroll
             for (int i = 0; i < 5; ++i)
-                if (NS == 4 || i == 4) ray4(1 + i, t + 4 * i);
-            Real wn;
-            lds(sbase + sm.stw + idx * SZ, wn);
-            wn = quotient(wn, d[0]);
-            if (a.jacc) {
-                int ex;
-                lds(sbase + sm.ste + idx * 4, ex);
-                wn *= t[18] * pow2(Real(0), ex);
+                if (NS == 4 || (i == 4 && !EMG)) ray4(1 + i, t + 4 * i);
+            if constexpr (!EMG) {
+                Real wn;
+                lds(sbase + sm.stw + idx * SZ, wn);
+                wn = quotient(wn, d[0]);
+                if (a.jacc) {
+                    int ex;
+                    lds(sbase + sm.ste + idx * 4, ex);
+                    wn *= t[18] * pow2(Real(0), ex);
+                }
+                sts(sbase + sm.wgt + (s * nodes + idx) * SZ, wn);
             }
-            sts(sbase + sm.wgt + (s * nodes + idx) * SZ, wn);
             int v;
             lds(sbase + sm.stv + idx * 4, v);
             sts(sbase + sm.vox + (s * nodes + idx) * 4, v);
             unsigned oc = opaque(sbase + sm.coef + s * FX * sm.cplane + idx * CB), of = sbase + sm.freq;
             if constexpr (NS == 1) {
                 sts(sbase + (s * nodes + idx) * SZ, d[2]);
-#pragma unroll 2
                 for (int f = 0; f < nf; ++f, oc += sm.cplane, of += 8) {
                     X x;
                     lds(of, x);
@@ -705,7 +783,37 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
             if (q + 5 < nz && tid < GW)
                 copy_async(geo + ((q + 5) & 7) * GB + 4 * tid, reinterpret_cast<const int *>(G + q + 5) + tid);
         }
-        if (Lg > 1 && q >= 1) add_totals(q - 1);
+        if (!EMG && Lg > 1 && q >= 1) add_totals(q - 1);
+    };
+
+    // EMERGENT: a point's Stokes vectors at the frequencies of a unit, row jd of (direction,
+    // frequency), to the reverse mode's store and, at the last plane, to the output
+    auto emit = [&](int q, int jd, int v, const X *r) {
+        const int w1 = min(XW, (m + 1) * a.nnu - jd);
+#pragma unroll
+        for (int w = 0; w < XW; ++w) {
+            if (w >= w1) break;
+            Real o[NS];
+#pragma unroll
+            for (int s = 0; s < NS; ++s) o[s] = xlane(r[s], w);
+            if (a.store) {
+                Real *d = a.store + ((long long)(jd + w) * nvox + v) * NS;
+                if constexpr (NS == 1) {
+                    *d = o[0];
+                } else {
+                    using V = typename V16<Real>::T;
+#pragma unroll
+                    for (int h = 0; h < 4 / W::per; ++h) chunk_put<Real>(reinterpret_cast<V *>(d) + h, o + h * W::per);
+                }
+            }
+            if (q == nz - 1) {
+                int kz;
+                lds(geo + (q & 7) * GB + 8, kz);
+                double *d = a.out + ((long long)(jd + w) * nx * ny + (v - vox0 - kz * nx * ny)) * NS;
+#pragma unroll
+                for (int s = 0; s < NS; ++s) d[s] = (double)o[s];
+            }
+        }
     };
 
     // One plane of updates (q >= 1). The bilinear weights are used relative to the first
@@ -755,6 +863,8 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
             Real acc[NA];
 #pragma unroll
             for (int s = 0; s < NA; ++s) acc[s] = Real(0);
+            int vox = 0;
+            if constexpr (EMG) lds(sbase + sm.vox + ((q & 3) * nodes + p + nx) * 4, vox);
             // the corners' source vectors (NS = 4: I, Q, U and the S^0_0 that eta_V multiplies)
             auto source = [&](unsigned u, unsigned n, Real *r) {
                 if constexpr (NS == 1) lds(u + n / CB * SZ, r[0]);
@@ -819,7 +929,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 // a4, a6: optical path and coefficients of the step
                 const X tMO = xms(dsM, xfs(wM, eM, eO));
                 const XCoef<X> co = xcoef(tMO);
-                const X ls = has_p ? (XW == 1 ? xadd(co.wo, co.wc) : xadd(co.e0, xneg(co.wm))) : xfs(Real(0.5), co.wc, co.wo);
+                [[maybe_unused]] const X ls = has_p ? xadd(co.e0, xneg(co.wm)) : xfs(Real(0.5), co.wc, co.wo);
                 // a7: right-hand side of Eq. 7, e I_M + (w_M + w_O + w_C) S_O - w_M d_M - w_C (S_O - c_M),
                 // with the upwind Stokes vector over w_M (a3) and K'_V at M coupling I and V
                 X r[NS];
@@ -944,13 +1054,17 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                         }
                     }
                 }
-                // a8: Lambda* and frequency integration (w_nu phi / N = w_nu eta_I / (chi N))
-                X wt;
-                lds(of, wt);
-                wt = xmul(wt, eO);
+                if constexpr (EMG) {
+                    if (active) emit(q, m * a.nnu + j0 + f * XW, vox, r);
+                } else {
+                    // a8: Lambda* and frequency integration (w_nu phi / N = w_nu eta_I / (chi N))
+                    X wt;
+                    lds(of, wt);
+                    wt = xmul(wt, eO);
 #pragma unroll
-                for (int s = 0; s < NA - 1; ++s) acc[s] = xdot(wt, r[s], acc[s]);
-                acc[NA - 1] = xdot(wt, ls, acc[NA - 1]);
+                    for (int s = 0; s < NA - 1; ++s) acc[s] = xdot(wt, r[s], acc[s]);
+                    acc[NA - 1] = xdot(wt, ls, acc[NA - 1]);
+                }
                 if (PROBE && a.probe_ray == m && active) {
                     const int v = point_voxel(q, l, c);
                     for (int w = 0; w < XW && j0 + f * XW + w < a.nnu; ++w) {
@@ -962,7 +1076,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 }
                 uM += stepC; uO += stepC; uP += stepC; uI += stepI; uW += stepI; uH += stepI; of += Lg * 8;
             }
-            if (active) totals(q, p, acc);
+            if (!EMG && active) totals(q, p, acc);
         }
     };
 
@@ -999,10 +1113,17 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                         }
                     }
                 }
-                X eta, wt;
-                lds(sbase + sm.coef + f * sm.cplane + (p + nx) * CB, eta);
-                lds(sbase + sm.freq + FX * XW * SZ + f * 8, wt);
-                acc[0] = xdot(xmul(wt, eta), I0, acc[0]);
+                if constexpr (EMG) {
+                    X r[NS];
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) r[s] = s == 0 ? I0 : zero;
+                    emit(0, m * a.nnu + j0 + f * XW, v, r);
+                } else {
+                    X eta, wt;
+                    lds(sbase + sm.coef + f * sm.cplane + (p + nx) * CB, eta);
+                    lds(sbase + sm.freq + FX * XW * SZ + f * 8, wt);
+                    acc[0] = xdot(xmul(wt, eta), I0, acc[0]);
+                }
                 if (PROBE && a.probe_ray == m) {
                     for (int w = 0; w < XW && j0 + f * XW + w < a.nnu; ++w) {
                         const long long pv = (long long)(j0 + f * XW + w) * a.nvox + v;
@@ -1012,7 +1133,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                     }
                 }
             }
-            totals(0, p, acc);
+            if (!EMG) totals(0, p, acc);
         }
     };
 
@@ -1059,7 +1180,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
     }
 }
 
-template <typename Real, int NS, bool PROBE>
+template <typename Real, int NS, int MODE>
 __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kernel(const SweepArgs<Real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1086,7 +1207,7 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
     cluster.sync();
     // fixed-point sums do not depend on the order of their terms: the frequency groups of a
     // ray are items of their own; per-ray partials add their groups in order in one item
-    const int split = a.jacc ? a.ngroups : 1;
+    const int split = a.jacc || MODE == EMERGENT ? a.ngroups : 1;
     const int total = a.nitems * split;
     for (int k = 0, own = cid;; ++k, own += ncl) {
         int item = own;
@@ -1101,12 +1222,12 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
         if (item >= total) break;
         const int ray = item / split;
         const int code = a.items ? a.items[ray] : ray;
-        const int box = code / a.nray, m = code - box * a.nray;
+        const int box = MODE == EMERGENT ? 0 : code / a.nray, m = code - box * a.nray;
         const int g0 = item - ray * split;
         // the ray's constants (mu, ox, oy, oz, T[18], w, pad); the item starts with a barrier
         if (threadIdx.x < 24) sray[threadIdx.x] = reinterpret_cast<const Real *>(a.rays + m)[threadIdx.x];
         for (int g = g0; g < (split > 1 ? g0 + 1 : a.ngroups); ++g) {
-            jsweep_item<Real, NS, PROBE>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), box, m, g, rank, C);
+            jsweep_item<Real, NS, MODE>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), box, m, g, rank, C);
             // every halo row of the item has been written and read before the next one
             // (whose strips may have other neighbours)
             if (C > 1) cluster.sync();
@@ -1188,10 +1309,10 @@ cudaError_t launch_jacc_finalize(long long nvox, const unsigned long long *jacc,
     return cudaGetLastError();
 }
 
-template <typename Real, int NS, bool PROBE>
+template <typename Real, int NS, int MODE>
 static cudaError_t jprepare(int cluster, int smem)
 {
-    void *k = (void *)jsweep_kernel<Real, NS, PROBE>;
+    void *k = (void *)jsweep_kernel<Real, NS, MODE>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     if (cluster > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1201,7 +1322,7 @@ static cudaError_t jprepare(int cluster, int smem)
 template <typename Real, int NS>
 cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out)
 {
-    cudaError_t e = jprepare<Real, NS, false>(cluster, smem);
+    cudaError_t e = jprepare<Real, NS, SUMS>(cluster, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(cluster);
@@ -1214,16 +1335,15 @@ cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *
     at[0].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(out, jsweep_kernel<Real, NS, false>, &lc);
+    return cudaOccupancyMaxActiveClusters(out, jsweep_kernel<Real, NS, SUMS>, &lc);
 }
 
 // the probe variant writes one ray's Stokes vectors and Lambda* at every node and
 // frequency (porta_probe_ray); the plain one keeps no trace of that in its loop
-template <typename Real, int NS>
-cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st)
+template <typename Real, int NS, int MODE>
+static cudaError_t jlaunch(const SweepArgs<Real> &a, const LaunchCfg &cfg, cudaStream_t st)
 {
-    const bool probe = a.probe_ray >= 0;
-    cudaError_t e = probe ? jprepare<Real, NS, true>(cfg.cluster, cfg.smem) : jprepare<Real, NS, false>(cfg.cluster, cfg.smem);
+    cudaError_t e = jprepare<Real, NS, MODE>(cfg.cluster, cfg.smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(cfg.clusters * cfg.cluster);
@@ -1242,8 +1362,14 @@ cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t
         at[1].val.priority = cfg.priority;
         lc.numAttrs = 2;
     }
-    if (probe) return cudaLaunchKernelEx(&lc, jsweep_kernel<Real, NS, true>, a);
-    return cudaLaunchKernelEx(&lc, jsweep_kernel<Real, NS, false>, a);
+    return cudaLaunchKernelEx(&lc, jsweep_kernel<Real, NS, MODE>, a);
+}
+
+template <typename Real, int NS>
+cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st)
+{
+    if (a.out) return jlaunch<Real, NS, EMERGENT>(a, cfg, st);
+    return a.probe_ray >= 0 ? jlaunch<Real, NS, PROBE_RAY>(a, cfg, st) : jlaunch<Real, NS, SUMS>(a, cfg, st);
 }
 
 #define PORTA_JINST(R, N)                                                                    \
