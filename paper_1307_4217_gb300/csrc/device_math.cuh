@@ -12,76 +12,91 @@ namespace porta {
 //   psi'_M = (1 - e (1 + t)) / t,          psi'_O = (e + t - 1) / t,
 //   w_M = (2 - e (t^2 + 2t + 2)) / t^2,    w_O = 1 - 2 (e + t - 1) / t^2,
 //   w_C = 2 (t - 2 + e (t + 2)) / t^2      (Eqs. 9-13).
-// Below a crossover the closed forms lose digits to cancellation and the
-// Taylor series at t = 0 is used instead (Table 1 for double precision).
-// Series coefficients of t^k, k >= 1, from expanding the closed forms:
-//   psi'_M: (-1)^(k+1) k / (k+1)!        psi'_O: (-1)^(k+1) / (k+1)!
-//   w_M:    (-1)^(k+1) k (k+1) / (k+2)!  w_O:    2 (-1)^(k+1) / (k+2)!
-//   w_C:    2 (-1)^(k+1) k / (k+2)!
+// Near t = 0 the closed forms lose digits to cancellation; polynomials in t take their place.
 // ---------------------------------------------------------------------------
 template <typename Real>
 struct Coef {
     Real e, pm, po, wm, wo, wc;
 };
 
-__host__ __device__ constexpr double fact_d(int n) { return n <= 1 ? 1.0 : n * fact_d(n - 1); }
-__host__ __device__ constexpr double sgn_d(int k) { return (k % 2) ? 1.0 : -1.0; }  // (-1)^(k+1)
-__host__ __device__ constexpr double c_pm(int k) { return sgn_d(k) * k / fact_d(k + 1); }
-__host__ __device__ constexpr double c_po(int k) { return sgn_d(k) / fact_d(k + 1); }
-__host__ __device__ constexpr double c_wm(int k) { return sgn_d(k) * k * (k + 1.0) / fact_d(k + 2); }
-__host__ __device__ constexpr double c_wo(int k) { return 2.0 * sgn_d(k) / fact_d(k + 2); }
-__host__ __device__ constexpr double c_wc(int k) { return 2.0 * sgn_d(k) * k / fact_d(k + 2); }
-
-// t * (a_1 + t (a_2 + ... + t a_N)) with a_k = COEF(k), N = DEG; every
-// coefficient is a compile-time constant of type Real.
-template <typename Real, double (*COEF)(int), int K, int DEG>
-__device__ __forceinline__ Real horner_tail(Real t)
-{
-    constexpr double c = COEF(K);
-    if constexpr (K == DEG) {
-        return Real(c);
-    } else {
-        return Real(c) + t * horner_tail<Real, COEF, K + 1, DEG>(t);
-    }
-}
-
-template <typename Real, int DEG, double (*COEF)(int)>
-__device__ __forceinline__ Real horner(Real t)
-{
-    return t * horner_tail<Real, COEF, 1, DEG>(t);
-}
-
 // The linear-interpolation coefficients follow from the quadratic ones: a
 // linear source on MO is the Bezier curve whose control point is the midpoint
 // c_M = (y_M + y_O)/2, so psi'_M = w_M + w_C/2 and psi'_O = w_O + w_C/2 (all
 // terms positive: no cancellation). Only the three w series are evaluated.
 
-// Double precision: degree 8 (the order of Table 1), crossovers of Table 1
-// (w_M 0.14, w_O and w_C 0.18).
-__device__ __forceinline__ Coef<double> coefficients(double t)
+// reciprocal. In FP64, whose operations run at 2 lanes per cycle and SM here (1/64 of the FP32
+// rate): the hardware's 20-bit approximation and two Newton steps, 4 of them, within an ulp
+// for normal x. In FP32 the hardware approximation rcp.approx.ftz (max 1 ulp; the operands
+// here are normal numbers below 2^126), since the FP32 form's error budget is 1e-5. The bare
+// instruction saves the scaling steps of a general approximate division (4% of the J^K_Q
+// sweep's time).
+__device__ __forceinline__ double rcp(double x)
 {
-    Coef<double> c;
-    double e = exp(-t);
-    c.e = e;
-    double it = 1.0 / t, it2 = it * it;
-    c.wm = t < 0.14 ? horner<double, 8, c_wm>(t) : (2.0 - e * (t * t + 2.0 * t + 2.0)) * it2;
-    c.wo = t < 0.18 ? horner<double, 8, c_wo>(t) : 1.0 - 2.0 * (e + t - 1.0) * it2;
-    c.wc = t < 0.18 ? horner<double, 8, c_wc>(t) : 2.0 * (t - 2.0 + e * (t + 2.0)) * it2;
-    c.pm = c.wm + 0.5 * c.wc;
-    c.po = c.wo + 0.5 * c.wc;
-    return c;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
 }
-
-// reciprocal: IEEE in FP64; in FP32 the hardware approximation rcp.approx.ftz
-// (max 1 ulp; the operands here are normal numbers below 2^126), since the FP32
-// form's error budget is 1e-5. The bare instruction saves the scaling steps of a
-// general approximate division (4% of the J^K_Q sweep's time).
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float rcp(float x)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
+}
+
+// Double precision. With q = w_O, h = t (1 - q) / 2 gives e0 = 1 - e = t (1 - h) and
+// w_C = e0 - w_M - w_O. Below t = 1, w_M and w_O over t are polynomials minimax in relative
+// error (Remez exchange on the Taylor series, 5e-17); above, the closed forms in e0. Every
+// coefficient is within 2e-15 of its value. (26 operations, 34 and an exponential above,
+// where Taylor series below 0.14 and 0.18 and the closed forms above took up to 60 and left
+// 1e-13 at the crossover: 6% of the FP64 J^K_Q sweep's time.) e0 out: 1 - e.
+__device__ __forceinline__ Coef<double> coefficients(double t, double &e0)
+{
+    Coef<double> c;
+    if (t < 1.0) {
+        double m = fma(t, -1.1202256902396886e-09, 1.9558584056821613e-08), o = fma(t, 2.1752747810916859e-10, -3.9450135294101958e-09);
+        m = fma(t, m, -2.2723481708323534e-07);
+        o = fma(t, o, 4.9804374537587804e-08);
+        m = fma(t, m, 2.2524008032884722e-06);
+        o = fma(t, o, -5.5090033985190619e-07);
+        m = fma(t, m, -1.9839818101854985e-05);
+        o = fma(t, o, 5.5113331078707397e-06);
+        m = fma(t, m, 0.00015432036885733235);
+        o = fma(t, o, -4.9603129765952493e-05);
+        m = fma(t, m, -0.0010416664919878616);
+        o = fma(t, o, 0.00039682538720382121);
+        m = fma(t, m, 0.0059523809209458198);
+        o = fma(t, o, -0.0027777777765696106);
+        m = fma(t, m, -0.027777777774420587);
+        o = fma(t, o, 0.016666666666588639);
+        m = fma(t, m, 0.099999999999813557);
+        o = fma(t, o, -0.083333333333331358);
+        m = fma(t, m, -0.24999999999999592);
+        o = fma(t, o, 0.33333333333333331);
+        m = fma(t, m, 0.33333333333333331);
+        c.wm = t * m;
+        c.wo = t * o;
+        const double ht = 0.5 * t;
+        e0 = fma(-t, fma(-ht, c.wo, ht), t);
+        c.e = 1.0 - e0;
+        c.wc = (e0 - c.wm) - c.wo;
+    } else {
+        const double it = rcp(t);
+        c.e = exp(-t);
+        e0 = 1.0 - c.e;
+        const double h2 = fma(-2.0 * e0, it, 2.0);
+        c.wo = fma(-h2, it, 1.0);
+        c.wc = 2.0 * it * (h2 - e0);
+        c.wm = fma(-c.e, fma(t, t + 2.0, 2.0), 2.0) * (it * it);
+    }
+    c.pm = c.wm + 0.5 * c.wc;
+    c.po = c.wo + 0.5 * c.wc;
+    return c;
+}
+__device__ __forceinline__ Coef<double> coefficients(double t)
+{
+    double e0;
+    return coefficients(t, e0);
 }
 
 // Single precision: two regimes. Below t = 1.5, w / t as a polynomial whose relative
@@ -152,7 +167,12 @@ __device__ __forceinline__ float profile_shape(float xs)
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fminf(xs * xs, 60.0f) * -1.4426950408889634f));
     return r;
 }
-__device__ __forceinline__ double profile_shape(double xs) { return exp(-xs * xs); }
+// (FP64: capped at 1e-282 of the line centre, so that eta_I stays a normal number)
+__device__ __forceinline__ double profile_shape(double xs)
+{
+    const double x = xs * xs;
+    return exp(-(__double2hiint(x) > __double2hiint(650.0) ? 650.0 : x));
+}
 
 // ---------------------------------------------------------------------------
 // BESSER upwind control point c_M of the quadratic Bezier spline on MO
@@ -199,6 +219,28 @@ __device__ __forceinline__ Real control_point_branch(Real yM, Real yO, Real yP, 
     const bool over = (dm - w) * w < Real(0);        // steps 5-6: c_M outside [y_M, y_O] -> y_M
     const Real r = over ? yM : cM9;
     const bool ext = dm * dp <= Real(0);             // step 2: extremum at O
+    branch = ext ? 0 : (over ? 1 : (clip ? 2 : 3));
+    return ext ? yO : r;
+}
+
+// The same in FP64 with the signs of the products taken from their factors' bits, in the
+// integer pipe (6 of 16 FP64 operations less).
+__device__ __forceinline__ bool nonzero(double a) { return ((unsigned)__double2hiint(a) << 1 | (unsigned)__double2loint(a)) != 0u; }
+// a b > 0, a b < 0
+__device__ __forceinline__ bool same_sign(double a, double b) { return (__double2hiint(a) ^ __double2hiint(b)) >= 0 && nonzero(a) && nonzero(b); }
+__device__ __forceinline__ bool opposite_sign(double a, double b) { return (__double2hiint(a) ^ __double2hiint(b)) < 0 && nonzero(a) && nonzero(b); }
+__device__ __forceinline__ double control_point_branch(double yM, double yO, double yP, const BesserGeom<double> &g, int &branch)
+{
+    const double dm = yO - yM, dp = yP - yO;
+    const double yp = g.a * dp + g.b * dm;
+    const double w = g.hm2 * yp;
+    double u = g.hp2 * yp;
+    const bool clip = same_sign(u, u - dp);
+    u = clip ? dp : u;
+    const double cM9 = yO - g.r * u;
+    const bool over = opposite_sign(dm - w, w);
+    const double r = over ? yM : cM9;
+    const bool ext = !same_sign(dm, dp);
     branch = ext ? 0 : (over ? 1 : (clip ? 2 : 3));
     return ext ? yO : r;
 }

@@ -196,18 +196,10 @@ __device__ __forceinline__ double xadd(double a, double b) { return a + b; }
 __device__ __forceinline__ float2 xneg(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ double xneg(double a) { return -a; }
 __device__ __forceinline__ float2 xrcp(float2 a) { return make_float2(rcp(a.x), rcp(a.y)); }
-// (FP64 operations run at 2 lanes per cycle and SM here, 1/64 of the FP32 rate: the hardware's
-// 20-bit reciprocal and two Newton steps, within an ulp for normal a, are 4 of them)
-__device__ __forceinline__ double xrcp(double a)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    y = fma(y, fma(-a, y, 1.0), y);
-    return fma(y, fma(-a, y, 1.0), y);
-}
+__device__ __forceinline__ double xrcp(double a) { return rcp(a); }
 // -1 / a
 __device__ __forceinline__ float2 xnrcp(float2 a) { return make_float2(rcp(-a.x), rcp(-a.y)); }
-__device__ __forceinline__ double xnrcp(double a) { return xrcp(-a); }
+__device__ __forceinline__ double xnrcp(double a) { return rcp(-a); }
 // the same Real times both lanes (scalar operations: a pair made of one value costs a move)
 __device__ __forceinline__ float2 xms(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
 __device__ __forceinline__ double xms(double s, double a) { return s * a; }
@@ -217,12 +209,7 @@ __device__ __forceinline__ double xfs(double s, double a, double c) { return fma
 __device__ __forceinline__ float xdot(float2 a, float2 b, float s) { return fmaf(a.y, b.y, fmaf(a.x, b.x, s)); }
 __device__ __forceinline__ double xdot(double a, double b, double s) { return fma(a, b, s); }
 __device__ __forceinline__ float2 xprofile(float2 xs) { return make_float2(profile_shape(xs.x), profile_shape(xs.y)); }
-// (capped far in the wings, at 1e-282 of the line centre, so that eta_I stays a normal number)
-__device__ __forceinline__ double xprofile(double xs)
-{
-    const double x = xs * xs;
-    return exp(-(__double2hiint(x) > __double2hiint(650.0) ? 650.0 : x));
-}
+__device__ __forceinline__ double xprofile(double xs) { return profile_shape(xs); }
 // 1 - a^2
 __device__ __forceinline__ float2 xdet(float2 a) { return make_float2(1.0f - a.x * a.x, 1.0f - a.y * a.y); }
 __device__ __forceinline__ double xdet(double a) { return 1.0 - a * a; }
@@ -238,49 +225,12 @@ __device__ __forceinline__ double xlane(double a, int) { return a; }
 // source functions, within 3e-7 and 8e-7. The polynomials are evaluated for both lanes
 // always; the closed forms replace them where some lane needs them. (Three polynomials, an
 // exponential per lane and the sums: 26 instructions more per unit, 3% of the sweep's time.)
-// (In FP64 below t = 1, to 5e-17; 26 operations instead of an exponential, a reciprocal, the
-// closed forms and, below 0.18, three series.)
 template <typename X> struct XCoef { X e, e0, wm, wo, wc; };
 __device__ __forceinline__ XCoef<double> xcoef(double t)
 {
-    XCoef<double> c;
-    if (t < 1.0) {
-        double m = fma(t, -1.1202256902396886e-09, 1.9558584056821613e-08), o = fma(t, 2.1752747810916859e-10, -3.9450135294101958e-09);
-        m = fma(t, m, -2.2723481708323534e-07);
-        o = fma(t, o, 4.9804374537587804e-08);
-        m = fma(t, m, 2.2524008032884722e-06);
-        o = fma(t, o, -5.5090033985190619e-07);
-        m = fma(t, m, -1.9839818101854985e-05);
-        o = fma(t, o, 5.5113331078707397e-06);
-        m = fma(t, m, 0.00015432036885733235);
-        o = fma(t, o, -4.9603129765952493e-05);
-        m = fma(t, m, -0.0010416664919878616);
-        o = fma(t, o, 0.00039682538720382121);
-        m = fma(t, m, 0.0059523809209458198);
-        o = fma(t, o, -0.0027777777765696106);
-        m = fma(t, m, -0.027777777774420587);
-        o = fma(t, o, 0.016666666666588639);
-        m = fma(t, m, 0.099999999999813557);
-        o = fma(t, o, -0.083333333333331358);
-        m = fma(t, m, -0.24999999999999592);
-        o = fma(t, o, 0.33333333333333331);
-        m = fma(t, m, 0.33333333333333331);
-        c.wm = t * m;
-        c.wo = t * o;
-        const double ht = 0.5 * t;
-        c.e0 = fma(-t, fma(-ht, c.wo, ht), t);
-        c.e = 1.0 - c.e0;
-        c.wc = (c.e0 - c.wm) - c.wo;
-    } else {
-        const double it = xrcp(t);
-        c.e = exp(-t);
-        c.e0 = 1.0 - c.e;
-        const double h2 = fma(-2.0 * c.e0, it, 2.0);
-        c.wo = fma(-h2, it, 1.0);
-        c.wc = 2.0 * it * (h2 - c.e0);
-        c.wm = fma(-c.e, fma(t, t + 2.0, 2.0), 2.0) * (it * it);
-    }
-    return c;
+    double e0;
+    const Coef<double> c = coefficients(t, e0);
+    return {c.e, e0, c.wm, c.wo, c.wc};
 }
 __device__ __forceinline__ XCoef<float2> xcoef(float2 t)
 {
