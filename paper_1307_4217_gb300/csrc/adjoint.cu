@@ -889,25 +889,23 @@ cudaError_t launch_adjoint(const SweepArgs<Real> &a, const LaunchCfg &cfg, cudaS
     return cudaLaunchKernelEx(&lc, adjoint_kernel<Real, NS, 2>, a);
 }
 
-// per voxel: sum of the per-cluster accumulators in cluster order (FP64)
+// per voxel and quantity (blockIdx.y): sum of the per-cluster accumulators in cluster order
+// (FP64). One quantity per thread keeps the loads of several clusters in flight and fills the
+// chip for small boxes: 6144 voxels, 152 clusters, FP64 258 -> 25 us (75 MB).
 template <typename Real>
 __global__ void adjoint_acc_reduce_kernel(const Real *gacc, int nclusters, long long nvox, int nl, double *g_chi,
                                           double *g_b, double *g_rho)
 {
+    const int k = blockIdx.y;
+    if ((k >= 1 && k <= 3 && !g_b) || k >= 4 + nl) return;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvox; v += (long long)gridDim.x * blockDim.x) {
-        double s[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int cl = 0; cl < nclusters; ++cl) {
-            const Real *p = gacc + (long long)cl * 10 * nvox + v;
-#pragma unroll
-            for (int k = 0; k < 10; ++k) s[k] += (double)p[k * nvox];
-        }
-        g_chi[v] += s[0];
-        if (g_b) {
-            g_b[v] += s[1];
-            g_b[nvox + v] += s[2];
-            g_b[2 * nvox + v] += s[3];
-        }
-        for (int c = 0; c < nl; ++c) g_rho[v * nl + c] = s[4 + c];
+        const Real *p = gacc + k * nvox + v;
+        double s = 0.0;
+#pragma unroll 8
+        for (int cl = 0; cl < nclusters; ++cl) s += (double)p[(long long)cl * 10 * nvox];
+        if (k == 0) g_chi[v] += s;
+        else if (k < 4) g_b[(k - 1) * nvox + v] += s;
+        else g_rho[v * nl + k - 4] = s;
     }
 }
 
@@ -915,9 +913,9 @@ template <typename Real>
 cudaError_t launch_adjoint_acc_reduce(const Real *gacc, int nclusters, long long nvox, int nl, double *g_chi,
                                       double *g_b, double *g_rho, cudaStream_t st)
 {
-    const int threads = 256;
+    const int threads = 128;
     const long long blocks = std::min<long long>((nvox + threads - 1) / threads, 152LL * 16);
-    adjoint_acc_reduce_kernel<Real><<<(int)blocks, threads, 0, st>>>(gacc, nclusters, nvox, nl, g_chi, g_b, g_rho);
+    adjoint_acc_reduce_kernel<Real><<<dim3((unsigned)blocks, 10), threads, 0, st>>>(gacc, nclusters, nvox, nl, g_chi, g_b, g_rho);
     return cudaGetLastError();
 }
 template cudaError_t launch_adjoint_acc_reduce<float>(const float *, int, long long, int, double *, double *, double *,

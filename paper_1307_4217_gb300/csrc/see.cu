@@ -103,7 +103,7 @@ __global__ void jkq_finalize_kernel(long long nvox, int nray, const void *part, 
         lstar[v] = (double)L.s;
     } else {
         KahanSum<Real> J[6], L;
-#pragma unroll 2
+#pragma unroll 4
         for (int m = 0; m < nray; ++m) {
             const Real *q = p + 4 * ((long long)m * nvox + v);
             const Real *t = stw + m * 19;
@@ -267,6 +267,15 @@ __global__ void coefficients_kernel(int n, const double *t, double *out)
 }
 
 static inline unsigned nblk(long long n, int t) { return (unsigned)((n + t - 1) / t); }
+// threads per block of the kernels that work long on a voxel (sums over rays, 5 x 5 systems in
+// FP64): 256, or as few as it takes for two blocks per SM of the 152. (6144 voxels, 32 rays,
+// FP64, caches cold: the J^K_Q sums took 66 us in 24 blocks of 256, 44 us in 192 of 32.)
+static inline int spread(long long n)
+{
+    int t = 256;
+    while (t > 32 && nblk(n, t) < 2 * 152) t /= 2;
+    return t;
+}
 
 template <typename Real>
 cudaError_t run_profile_norm(long long nvox, int nray, int nnu, const double *mu, const double *xf, const double *wf,
@@ -290,7 +299,8 @@ cudaError_t run_jkq_finalize(long long nvox, int nray, const void *part, const d
     const size_t smem = (size_t)nray * 19 * sizeof(Real);
     cudaError_t e = cudaFuncSetAttribute(jkq_finalize_kernel<Real, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    jkq_finalize_kernel<Real, NS><<<nblk(nvox, 256), 256, smem, st>>>(nvox, nray, part, tw, jkq, lstar);
+    const int t = spread(nvox);
+    jkq_finalize_kernel<Real, NS><<<nblk(nvox, t), t, smem, st>>>(nvox, nray, part, tw, jkq, lstar);
     return cudaGetLastError();
 }
 
@@ -300,7 +310,8 @@ cudaError_t run_j1_finalize(long long nvox, int nray, const void *partv, const d
     const size_t smem = (size_t)nray * 3 * sizeof(Real);
     cudaError_t e = cudaFuncSetAttribute(j1_finalize_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    j1_finalize_kernel<Real><<<nblk(nvox, 256), 256, smem, st>>>(nvox, nray, (const Real *)partv, tw1, j1);
+    const int t = spread(nvox);
+    j1_finalize_kernel<Real><<<nblk(nvox, t), t, smem, st>>>(nvox, nray, (const Real *)partv, tw1, j1);
     return cudaGetLastError();
 }
 
@@ -309,7 +320,8 @@ cudaError_t run_see(long long nvox, int nl, int model, double bcrit, const doubl
                     const double *bvec, const double *jkq, const double *lstar, double *rho, void *rhoR,
                     unsigned long long *resid, cudaStream_t st, const double *src)
 {
-    see_kernel<Real><<<nblk(nvox, 256), 256, 0, st>>>(nvox, nl, model, bcrit, eps, bpl, bvec, jkq, lstar, rho,
+    const int t = spread(nvox);
+    see_kernel<Real><<<nblk(nvox, t), t, 0, st>>>(nvox, nl, model, bcrit, eps, bpl, bvec, jkq, lstar, rho,
                                                       (Real *)rhoR, resid, src);
     return cudaGetLastError();
 }
@@ -398,7 +410,8 @@ cudaError_t run_see_vjp(long long nvox, int nl, int model, double bcrit, const d
                         const double *rho, const double *g, double *g_rho, double *g_jkq, double *g_lstar,
                         double *g_f, double *g_b, cudaStream_t st)
 {
-    see_vjp_kernel<<<nblk(nvox, 256), 256, 0, st>>>(nvox, nl, model, bcrit, eps, bpl, bvec, jkq, lstar, src, rho, g,
+    const int t = spread(nvox);
+    see_vjp_kernel<<<nblk(nvox, t), t, 0, st>>>(nvox, nl, model, bcrit, eps, bpl, bvec, jkq, lstar, src, rho, g,
                                                     g_rho, g_jkq, g_lstar, g_f, g_b);
     return cudaGetLastError();
 }
@@ -407,7 +420,8 @@ cudaError_t run_see_apply(long long nvox, int nl, int model, double bcrit, const
                           const double *bvec, const double *jkq, const double *rho, double alpha, const double *add,
                           int with_eb, double *out, cudaStream_t st)
 {
-    see_apply_kernel<<<nblk(nvox, 256), 256, 0, st>>>(nvox, nl, model, bcrit, eps, bpl, bvec, jkq, rho, alpha, add,
+    const int t = spread(nvox);
+    see_apply_kernel<<<nblk(nvox, t), t, 0, st>>>(nvox, nl, model, bcrit, eps, bpl, bvec, jkq, rho, alpha, add,
                                                       with_eb, out);
     return cudaGetLastError();
 }
