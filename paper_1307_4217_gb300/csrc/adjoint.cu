@@ -171,11 +171,11 @@ __device__ __forceinline__ int row_start(int k, int ny, int C) { return (int)(((
 // parameter gradients (chi, e, b) of one node at reduced frequency x from the
 // node's total adjoint t = dL/d(eta_I, [eta_V], eps[NS])
 template <typename Real, int NS>
-__device__ __forceinline__ void node_param_grad(const Node<Real, NS> &n, Real x, const Real *t, Real &gchi, Real &ge,
-                                                Real &gb)
+__device__ __forceinline__ void node_param_grad(const Node<Real, NS> &n, Real x, unsigned stab, const Real *t, Real &gchi,
+                                                Real &ge, Real &gb)
 {
     const Real xs = x - n.s;
-    const Real ph = profile_shape(xs);
+    const Real ph = profile_shape(xs, stab);
     if constexpr (NS == 1) {
         gchi += ph * t[0];
         ge += ph * t[1];
@@ -189,40 +189,54 @@ __device__ __forceinline__ void node_param_grad(const Node<Real, NS> &n, Real x,
 }
 
 // the same in the unknowns: dL/dchi at fixed rho, dL/dB (3) and dL/drho (up to 6)
-// added to o[10] (eps_i = chi phi S_i(rho), eps_V = S00 eta_V, S_i = sum_c T_ic rho_c
-// with the real multipole layout's factor 2 for Q != 0); o in the sweep's precision
-// over one frequency group (the per-cluster sums across items are FP64)
+// (eps_i = chi phi S_i(rho), eps_V = S00 eta_V, S_i = sum_c T_ic rho_c with the real
+// multipole layout's factor 2 for Q != 0), in the sweep's precision over one frequency
+// group (the per-cluster sums across items are FP64). Over the frequencies are summed what
+// depends on them, o: dL/dchi, dL/db, dL/dS_I, dL/dS_Q, dL/dS_U and eps_V's part of dL/drho_0;
+// the ray's factors follow once per node (node_rho: 28 operations less per frequency).
 template <typename Real, int NS>
-__device__ __forceinline__ void node_param_grad_rho(const Node<Real, NS> &n, const RayDev<Real> &ray, Real bfac, Real x,
-                                                    const Real *t, Real *o)
+__device__ __forceinline__ void node_param_grad_rho(const Node<Real, NS> &n, Real x, unsigned stab, const Real *t, Real *o)
 {
     const Real xs = x - n.s;
-    const Real ph = profile_shape(xs);
+    const Real ph = profile_shape(xs, stab);
+    const Real cp = n.chi * ph;
     if constexpr (NS == 1) {
         o[0] += ph * (t[0] + n.S * t[1]);
-        o[4] += n.chi * ph * t[1];
+        o[2] += cp * t[1];
     } else {
         const Real bxs = n.b * xs;
         o[0] += ph * (t[0] + bxs * t[1] + n.SI * t[2] + n.SQ * t[3] + n.SU * t[4] + bxs * n.S00 * t[5]);
-        const Real gb = bfac * xs * ph * n.chi * (t[1] + n.S00 * t[5]);
-        o[1] += gb * ray.ox;
-        o[2] += gb * ray.oy;
-        o[3] += gb * ray.oz;
-        const Real cp = n.chi * ph;
-        const Real gS[3] = {cp * t[2], cp * t[3], cp * t[4]};
+        o[1] += xs * cp * (t[1] + n.S00 * t[5]);
+        o[2] += cp * t[2];
+        o[3] += cp * t[3];
+        o[4] += cp * t[4];
+        o[5] += cp * bxs * t[5];
+    }
+}
+template <typename Real, int NS>
+__device__ __forceinline__ void node_rho(const RayDev<Real> &ray, Real bfac, const Real *o, Real *out)
+{
+    out[0] = o[0];
+    if constexpr (NS == 1) {
+        out[4] = o[2];
+    } else {
+        const Real gb = bfac * o[1];
+        out[1] = gb * ray.ox;
+        out[2] = gb * ray.oy;
+        out[3] = gb * ray.oz;
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const Real f2 = c >= 2 ? Real(2) : Real(1);
-            o[4 + c] += f2 * (ray.t[c] * gS[0] + ray.t[6 + c] * gS[1] + ray.t[12 + c] * gS[2]);
+            out[4 + c] = f2 * (ray.t[c] * o[2] + ray.t[6 + c] * o[3] + ray.t[12 + c] * o[4]);
         }
-        o[4] += cp * bxs * t[5];
+        out[4] += o[5];
     }
 }
 
 template <typename Real, int NS, int FORM>
 __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::cluster_group &cluster,
                                              typename V16<Real>::T *ring, Real *gI, Real *gM, Real *gP, Real *T,
-                                             Real *tt, int d, int g, int rank, int C, int item, int cid)
+                                             Real *tt, unsigned stab, int d, int g, int rank, int C, int item, int cid)
 {
     constexpr int NM = adj_nm<NS>(), NP = adj_np<NS>();
     constexpr int NCH = node_words<NS>() * (int)sizeof(Real) / 16;
@@ -325,7 +339,7 @@ __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::clust
             const Real *ph = last ? gP_next : gP;
             const int lh = last ? 0 : (l + 1) * nx;
             Real gchi = 0, ge = 0, gb = 0;
-            Real o[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+            Real o[6] = {0, 0, 0, 0, 0, 0};
             for (int f = 0; f < nf; ++f) {
                 Real t[NM];
                 VM::load(T + oT(par, f), ipa, p, t);
@@ -344,9 +358,9 @@ __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::clust
                     for (int s = 0; s < NS; ++s) t[NM - NS + s] += gp[1 + s];
                 }
                 if constexpr (FORM == 0)
-                    node_param_grad<Real, NS>(n, xsh[f], t, gchi, ge, gb);
+                    node_param_grad<Real, NS>(n, xsh[f], stab, t, gchi, ge, gb);
                 else
-                    node_param_grad_rho<Real, NS>(n, ray, a.bfac, xsh[f], t, o);
+                    node_param_grad_rho<Real, NS>(n, xsh[f], stab, t, o);
             }
             const long long v = B.vox0 + voxel(gq, c, l);
             if constexpr (FORM == 0) {
@@ -360,8 +374,10 @@ __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::clust
                 // node is finalized by one thread per item and the cluster's items are
                 // separated by cluster barriers (release / acquire), so the additions
                 // into each accumulator happen in item order: the sums are reproducible.
+                Real out[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+                node_rho<Real, NS>(ray, a.bfac, o, out);
 #pragma unroll
-                for (int k = 0; k < 10; ++k) atomicAdd(acc + k * a.nvox + v, o[k]);
+                for (int k = 0; k < 10; ++k) atomicAdd(acc + k * a.nvox + v, out[k]);
             }
         }
     };
@@ -502,7 +518,7 @@ __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::clust
                 for (int k = 0; k < 4; ++k) {
                     const CornerM<Real, NS> km = corner_m<Real, NS>(ring_load<Real, NS>(ring, plane, chunk, sM, rM[k]), wM[k]);
                     const Real xs = x - km.s;
-                    const Real we = km.wchi * profile_shape(xs);
+                    const Real we = km.wchi * profile_shape(xs, stab);
                     etaM += we;
                     if constexpr (NS == 1) {
                         epsM[0] += we * km.S;
@@ -524,7 +540,7 @@ __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::clust
                         const CornerP<Real, NS> kp =
                             corner_p<Real, NS>(ring_load<Real, NS>(ring, plane, chunk, sP, rP[k]), wP[k]);
                         const Real xs = x - kp.s;
-                        const Real we = kp.wchi * profile_shape(xs);
+                        const Real we = kp.wchi * profile_shape(xs, stab);
                         etaP += we;
                         if constexpr (NS == 1) {
                             epsP[0] += we * kp.S;
@@ -537,7 +553,7 @@ __device__ __forceinline__ void adjoint_item(const SweepArgs<Real> &a, cg::clust
                     }
                 }
                 const Real xsO = x - nO.s;
-                const Real phO = profile_shape(xsO);
+                const Real phO = profile_shape(xsO, stab);
                 const Real etaO = nO.chi * phO;
                 Real SO[NS], SM[NS], SP[NS];
                 const Real iM = rcp(etaM), iO = rcp(etaO);
@@ -739,6 +755,8 @@ template <typename Real, int NS, int FORM>
 __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 2 : 1) adjoint_kernel(const SweepArgs<Real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double s_exp[sizeof(Real) == 8 ? 64 : 1];
+    profile_table<Real>(s_exp);
     constexpr int NM = adj_nm<NS>(), NP = adj_np<NS>();
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
@@ -756,7 +774,8 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 2 : 1) adjoint_kernel
     cluster.sync();
     for (int item = cid; item < a.nitems; item += ncl) {
         const int d = item / a.ngroups, g = item - d * a.ngroups;
-        adjoint_item<Real, NS, FORM>(a, cluster, ring, gI, gM, gP, T, tt, d, g, rank, C, item, cid);
+        adjoint_item<Real, NS, FORM>(a, cluster, ring, gI, gM, gP, T, tt, (unsigned)__cvta_generic_to_shared(s_exp), d, g, rank, C,
+                                     item, cid);
         cluster.sync();
     }
 }

@@ -209,25 +209,7 @@ __device__ __forceinline__ double xfs(double s, double a, double c) { return fma
 __device__ __forceinline__ float xdot(float2 a, float2 b, float s) { return fmaf(a.y, b.y, fmaf(a.x, b.x, s)); }
 __device__ __forceinline__ double xdot(double a, double b, double s) { return fma(a, b, s); }
 __device__ __forceinline__ float2 xprofile(float2 xs, unsigned) { return make_float2(profile_shape(xs.x), profile_shape(xs.y)); }
-// exp(-x^2) in FP64 by a table of 2^(j/64) at the shared-memory address tab (Tang, ACM TOMS 15,
-// 1989): -x^2 = (64 m + j) ln 2 / 64 + r with |r| < 0.0055, e^r by its Taylor polynomial of
-// degree 5 (4e-17), 10 operations of the FP64 pipe and 2^m by the exponent. Capped as
-// profile_shape is. (Every node and frequency takes one: 16 x 16 x 32, unpolarized, 48 rays, 11
-// frequencies, ten iterations 14.3 -> 13.4 ms.)
-__device__ __forceinline__ double xprofile(double xs, unsigned tab)
-{
-    double y = -xs * xs;
-    y = __double2hiint(y) > __double2hiint(-650.0) ? -650.0 : y;      // (both negative: the larger magnitude)
-    double k = fma(y, 92.33248261689366, 6755399441055744.0);
-    const int n = __double2loint(k);
-    k -= 6755399441055744.0;
-    const double r = fma(k, -3.623510646634843e-19, fma(k, -0.010830424696249145, y));
-    const double q = fma(r, fma(r, fma(r, 1.0 / 120, 1.0 / 24), 1.0 / 6), 0.5);
-    double t;
-    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(t) : "r"(tab + 8 * (n & 63)));
-    t = fma(t, fma(r * r, q, r), t);
-    return __hiloint2double(__double2hiint(t) + ((n >> 6) << 20), __double2loint(t));
-}
+__device__ __forceinline__ double xprofile(double xs, unsigned tab) { return profile_shape(xs, tab); }
 // 1 - a^2
 __device__ __forceinline__ float2 xdet(float2 a) { return make_float2(1.0f - a.x * a.x, 1.0f - a.y * a.y); }
 __device__ __forceinline__ double xdet(double a) { return 1.0 - a * a; }
@@ -1155,8 +1137,8 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
     __shared__ __align__(16) Real sray[24];
     __shared__ __align__(8) unsigned long long s_bar[4];
     __shared__ int s_dead, s_item[2];
-    __shared__ double s_exp[sizeof(Real) == 8 ? 64 : 1];      // 2^(j/64) (xprofile)
-    if (sizeof(Real) == 8 && threadIdx.x < 64) s_exp[threadIdx.x] = exp2(threadIdx.x / 64.0);
+    __shared__ double s_exp[sizeof(Real) == 8 ? 64 : 1];
+    profile_table<Real>(s_exp);
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
