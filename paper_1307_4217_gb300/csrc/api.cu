@@ -298,18 +298,35 @@ cudaError_t ensure_jpack(porta_ctx *c)
     return pmalloc(&c->d_jpack, (size_t)(c->ns == 1 ? jpack_words<1>() : jpack_words<4>()) * c->nvox * c->rsz);
 }
 
+// the packed inputs of sweep_j.cu; where there is no room for them, the kernel for wide planes,
+// which reads the inputs where they are (or the general sweep) takes over
+static void jpack_or_wide(porta_ctx *c)
+{
+    if (!use_jk(c) || c->jk_form != 1 || ensure_jpack(c) == cudaSuccess) return;
+    cudaGetLastError();
+    LaunchCfg cfg{};
+    const int n = c->nbox * c->nray, fc = c->opt_cluster, ff = c->opt_nu_group;
+    c->jk_form = 2;
+    const int rc = c->precision == PORTA_FP32
+                       ? (c->ns == 1 ? choose_launch<float, 1>(c, cfg, fc, ff, n, true, jnu(c))
+                                     : choose_launch<float, 4>(c, cfg, fc, ff, n, true, jnu(c)))
+                       : (c->ns == 1 ? choose_launch<double, 1>(c, cfg, fc, ff, n, true, jnu(c))
+                                     : choose_launch<double, 4>(c, cfg, fc, ff, n, true, jnu(c)));
+    if (rc != PORTA_OK) c->jk_form = 0;
+}
+
 cudaError_t ensure_sweep_buffers(porta_ctx *c)
 {
     check_global_sweep(c);
     cudaError_t e = cudaSuccess;
-    if (use_jk(c) && c->jk_form == 1) e = ensure_jpack(c);
-    if (e != cudaSuccess) return e;
     if (jfixed(c)) {
         if (!c->d_jacc) e = pmalloc(&c->d_jacc, (size_t)(c->nj + 1) * c->nvox * sizeof(unsigned long long));
         if (e == cudaSuccess && !c->d_jexp) e = pmalloc(&c->d_jexp, (size_t)c->nvox * sizeof(int));
-        return e;
+        if (e == cudaSuccess) jpack_or_wide(c);
+        if (jfixed(c)) return e;
     }
     if (!c->d_part) e = pmalloc(&c->d_part, (size_t)c->nray * c->nvox * (c->ns == 1 ? 2 : 4) * c->rsz);
+    if (e == cudaSuccess && !jfixed(c)) jpack_or_wide(c);
     // polarized lines of a multilevel atom: the per-ray integrals of Stokes V (J^1_Q)
     if (e == cudaSuccess && c->d_dich && !c->d_partv) e = pmalloc(&c->d_partv, (size_t)c->nray * c->nvox * c->rsz);
     // short characteristics on cell faces: the work planes and per-group partials
@@ -468,6 +485,12 @@ int formal_solve_t(porta_ctx *c, int probe_ray, Real *probe, Real *probe_ls)
         if (probe_ray >= 0) return fail(c, PORTA_EINVAL, "probe ray: not with the global-memory sweep");
         return faces_solve_t<Real>(c, !c->sc_faces);
     }
+    cudaError_t e = ensure_sweep_buffers(c);
+    if (e != cudaSuccess) return fail(c, PORTA_ENOMEM, std::string("formal solution buffers: ") + cudaGetErrorString(e));
+    if (c->gsweep) {
+        if (probe_ray >= 0) return fail(c, PORTA_EINVAL, "probe ray: not with the global-memory sweep");
+        return faces_solve_t<Real>(c, true);
+    }
     SweepArgs<Real> a = jkq_args<Real>(c);
     a.probe_ray = probe_ray;
     a.probe = probe;
@@ -485,13 +508,6 @@ int formal_solve_t(porta_ctx *c, int probe_ray, Real *probe, Real *probe_ls)
         return faces_solve_t<Real>(c, true);
     }
     shape_args<Real>(c, a, cfg, use_jk(c));
-    cudaError_t e = ensure_sweep_buffers(c);
-    if (e != cudaSuccess) return fail(c, PORTA_ENOMEM, std::string("formal solution buffers: ") + cudaGetErrorString(e));
-    a.part = jfixed(c) ? nullptr : c->d_part;
-    a.partv = (Real *)c->d_partv;
-    a.jacc = jfixed(c) ? c->d_jacc : nullptr;
-    a.jexp = c->d_jexp;
-    a.pack = (const Real *)c->d_jpack;
     e = jacc_prepare<Real>(c, a);
     if (e == cudaSuccess) e = sweep_jkq<Real>(c, a, cfg, a.items, a.nitems, probe_ray < 0);
     if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
@@ -503,13 +519,14 @@ template <typename Real>
 int autotune_t(porta_ctx *c)
 {
     const int nitems = c->nbox * c->nray;
+    cudaError_t eb = ensure_sweep_buffers(c);
+    if (eb != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("autotune: ") + cudaGetErrorString(eb));
     std::vector<LaunchCfg> cand = c->ns == 1 ? candidates<Real, 1>(c, nitems) : candidates<Real, 4>(c, nitems);
     if (cand.empty()) return fail(c, PORTA_EINVAL, "autotune: no launch shape fits");
     {
         // the timing launches write the formal solution's buffers (their sums are
         // discarded: every formal solution starts from zero)
-        cudaError_t eb = ensure_sweep_buffers(c);
-        if (eb == cudaSuccess) eb = jacc_prepare<Real>(c, jkq_args<Real>(c));
+        eb = jacc_prepare<Real>(c, jkq_args<Real>(c));
         if (eb != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("autotune: ") + cudaGetErrorString(eb));
     }
     cudaEvent_t e0, e1;

@@ -36,7 +36,7 @@
 // as the threads hold. Against the kernel of sweep_jw.cu, which this one replaces where it
 // fits (one frequency of one point per thread and step, one cluster barrier per plane), ms
 // per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 17.9, 33 x 27 x 41 x
-// 80 x 21 1.91 -> 1.21, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.4, 64 x 64 x 48 x 160 x 31
+// 80 x 21 1.91 -> 1.21, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.1, 64 x 64 x 48 x 160 x 31
 // x 2 lines, unpolarized, 46.4 -> 31.8 (with the rate equations).
 //
 // Shared memory per CTA (X: 8 bytes, a frequency unit):

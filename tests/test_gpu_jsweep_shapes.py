@@ -53,3 +53,21 @@ def test_wide_plane(nx, ny, prec):
     jg, lg = ctx.accumulate_jkq()
     _, (jo, lo) = oracle_fs(atm, 1, 2, 4, 3, rho)
     _check(jg, lg, jo, lo, 1e-5 if prec == F32 else 1e-10)
+
+
+@pytest.mark.parametrize("prec", [F32, F64])
+def test_no_room_for_packed_inputs(prec):
+    """The sums fit the device limit, the packed inputs do not: another kernel takes over."""
+    atm = polarized_case(12, 10, 8, seed=3)
+    rho = initial_rho(atm, 1, seed=4)
+    ctx = make_ctx(atm, 1, 2, 4, 5, prec, rho=rho)
+    nvox = 12 * 10 * 8
+    sums = nvox * (7 * 8 + 4) if prec == F32 else nvox * 16 * 4 * 8      # rays x 4 partials in FP64
+    assert P.porta_set_device_limit(P.porta_device_bytes() + sums + 4096) == P.PORTA_OK
+    try:
+        ctx.formal_solve()
+        jg, lg = ctx.accumulate_jkq()
+    finally:
+        assert P.porta_set_device_limit(0) == P.PORTA_OK
+    _, (jo, lo) = oracle_fs(atm, 1, 2, 4, 5, rho)
+    _check(jg, lg, jo, lo, 1e-5 if prec == F32 else 1e-10)
