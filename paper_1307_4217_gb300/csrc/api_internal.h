@@ -248,13 +248,14 @@ int jsweep_tots(const porta_ctx *c, int C, int F, int *threads_out)
 
 // Cycles of one plane of one pass of the J^K_Q sweep in a CTA: a chain of fixed length
 // (barrier, geometry, sources of the corners, sums), the units of the points' rounds one
-// after the other, and a round of the nodes' filling, whose length grows little with the
-// frequencies; in FP64 also the operations of all points and of `share` CTAs at 1/64 of the
-// FP32 rate, whichever is longer (smoothly). Fitted to forced shapes of boxes from 8 x 8 x 16
-// to 64 x 64 x 64 (C 1 to 16, every number of passes): the shape it picks was the fastest of
-// all, or within 13% of it, for each.
+// after the other, a round of the nodes' filling, whose length grows little with the
+// frequencies, and a little for the exchange between CTAs (without it two CTAs tie with one on
+// 8 x 8 planes: 58 and 50 us per call); in FP64 also the operations of all points and of
+// `share` CTAs at 1/64 of the FP32 rate, whichever is longer (smoothly). Fitted to forced
+// shapes of boxes from 8 x 8 x 16 to 64 x 64 x 64 (C 1 to 16, every number of passes): the
+// shape it picks was the fastest of all, or within 2% of it (FP64: 4%), for each.
 template <typename Real, int NS>
-double jsweep_plane_cost(int nx, int R, int F, int threads, int share)
+double jsweep_plane_cost(int nx, int R, int F, int threads, int share, bool exchange)
 {
     const int W = jsweep_lanes<Real>(), FX = (F + W - 1) / W;
     const int pts = R * nx, nodes = (R + 2) * nx;
@@ -262,8 +263,8 @@ double jsweep_plane_cost(int nx, int R, int F, int threads, int share)
     const double units = (double)((pts + pw - 1) / pw) * ((FX + Lg - 1) / Lg);
     const double fills = (nodes + threads - 1) / threads;
     if (sizeof(Real) == 4)
-        return NS == 4 ? 2660.0 + 1106.0 * units + fills * (1190.0 + 151.0 * FX)
-                       : 3180.0 + 778.0 * units + fills * (339.0 + 6.0 * FX);
+        return (exchange ? 120.0 : 0.0) + (NS == 4 ? 2660.0 + 1106.0 * units + fills * (1190.0 + 151.0 * FX)
+                                                   : 3180.0 + 778.0 * units + fills * (339.0 + 6.0 * FX));
     const double chain = NS == 4 ? 5680.0 + 10000.0 * units + fills * (2280.0 + 2330.0 * FX)
                                  : 6720.0 + 5580.0 * units + fills * 2030.0 * FX;
     const double pipe = share * (NS == 4 ? 3930.0 : 2120.0) * ((pts + 31) / 32) * FX;
@@ -309,7 +310,7 @@ int choose_jsweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int n
                 double total = 0.0, item_max = 0.0;
                 for (const BoxDev &b : c->boxes) {
                     const double item = (double)b.nz * (G / parts) *
-                                        jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads, share);
+                                        jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads, share, C > 1);
                     total += item * c->nray * parts;
                     item_max = std::max(item_max, item);
                 }
