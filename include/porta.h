@@ -382,9 +382,10 @@ int porta_fill_info(const porta_ctx *c, int *cluster_size, int *nu_group, double
    work list in (0, 1) it takes. PORTA_EINVAL if the shape does not fit. */
 int porta_set_fill(porta_ctx *c, int cluster_size, int nu_group, double fraction);
 
-/* Diagnostic: the coefficients of the BESSER-DELO step (Eqs. 9-13; Table 1
-   series at small optical path) exactly as the sweep kernels of the given
-   precision evaluate them, for n upwind optical paths t (host array, t > 0):
+/* Diagnostic: the coefficients of the BESSER-DELO step (Eqs. 9-13; polynomials
+   at small optical path) exactly as the general sweep and the adjoint of the given
+   precision evaluate them (the J^K_Q sweep in FP32 takes the same polynomials for
+   omega_M and omega_O and forms the others from them), for n upwind optical paths t (host array, t > 0):
    out[6*i + 0..5] = e^-t, psi'_M, psi'_O, omega_M, omega_O, omega_C (host).
    Synchronous; uses the current device. */
 int porta_eval_coefficients(int precision, int n, const double *t, double *out);
