@@ -170,6 +170,7 @@ cudaError_t ensure_buf(void **p, size_t &cap, size_t need)
 // geometry at offset 0). (Three allocations and releases per call before.)
 template <typename Real>
 struct Directions {
+    std::vector<unsigned char> host;     // lives until the caller has synchronized
     const PlaneGeom<Real> *geom = nullptr, *rel = nullptr;
     const RayDev<Real> *rays = nullptr;
     const BoxDev *box = nullptr;
@@ -178,7 +179,8 @@ template <typename Real>
 cudaError_t put_directions(porta_ctx *c, int ndir, const double *mu, const double *chi, int box, Directions<Real> &d)
 {
     const size_t n = (size_t)ndir * c->nz, gb = n * sizeof(PlaneGeom<Real>), rb = (size_t)ndir * sizeof(RayDev<Real>);
-    std::vector<unsigned char> h(2 * gb + sizeof(BoxDev) + rb);
+    std::vector<unsigned char> &h = d.host;
+    h.resize(2 * gb + sizeof(BoxDev) + rb);
     PlaneGeom<Real> *g = reinterpret_cast<PlaneGeom<Real> *>(h.data());
     BoxDev *b = reinterpret_cast<BoxDev *>(h.data() + 2 * gb);
     RayDev<Real> *r = reinterpret_cast<RayDev<Real> *>(b + 1);
