@@ -292,27 +292,24 @@ void check_global_sweep(porta_ctx *c)
     if (!c->sc_faces && !c->gsweep && c->d_kexpl == nullptr && c->interp != 2 && !smem_sweep_fits(c)) c->gsweep = 2;
 }
 
-cudaError_t ensure_jpack(porta_ctx *c)
+// The packed inputs of sweep_j.cu. Where there is no room for them the sweep copies the same
+// values word by word from where they are, with the same results, so nothing else depends on
+// them: not the launch shapes, not a graph captured without them. After a failure the next try
+// follows new unknowns or a new atmosphere. Never inside a capture.
+void ensure_jpack(porta_ctx *c)
 {
-    if (c->d_jpack) return cudaSuccess;
-    return pmalloc(&c->d_jpack, (size_t)(c->ns == 1 ? jpack_words<1>() : jpack_words<4>()) * c->nvox * c->rsz);
-}
-
-// the packed inputs of sweep_j.cu; where there is no room for them, the kernel for wide planes,
-// which reads the inputs where they are (or the general sweep) takes over
-static void jpack_or_wide(porta_ctx *c)
-{
-    if (!use_jk(c) || c->jk_form != 1 || ensure_jpack(c) == cudaSuccess) return;
-    cudaGetLastError();
-    LaunchCfg cfg{};
-    const int n = c->nbox * c->nray, fc = c->opt_cluster, ff = c->opt_nu_group;
-    c->jk_form = 2;
-    const int rc = c->precision == PORTA_FP32
-                       ? (c->ns == 1 ? choose_launch<float, 1>(c, cfg, fc, ff, n, true, jnu(c))
-                                     : choose_launch<float, 4>(c, cfg, fc, ff, n, true, jnu(c)))
-                       : (c->ns == 1 ? choose_launch<double, 1>(c, cfg, fc, ff, n, true, jnu(c))
-                                     : choose_launch<double, 4>(c, cfg, fc, ff, n, true, jnu(c)));
-    if (rc != PORTA_OK) c->jk_form = 0;
+    if (c->d_jpack || c->jpack_failed) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return;
+    }
+    const size_t words = c->ns == 1 ? jpack_words<1>() : jpack_words<4>();
+    c->jpack_failed = pmalloc(&c->d_jpack, words * c->nvox * c->rsz) != cudaSuccess;
+    if (c->jpack_failed) {
+        cudaGetLastError();
+        c->d_jpack = nullptr;
+    }
 }
 
 cudaError_t ensure_sweep_buffers(porta_ctx *c)
@@ -322,11 +319,11 @@ cudaError_t ensure_sweep_buffers(porta_ctx *c)
     if (jfixed(c)) {
         if (!c->d_jacc) e = pmalloc(&c->d_jacc, (size_t)(c->nj + 1) * c->nvox * sizeof(unsigned long long));
         if (e == cudaSuccess && !c->d_jexp) e = pmalloc(&c->d_jexp, (size_t)c->nvox * sizeof(int));
-        if (e == cudaSuccess) jpack_or_wide(c);
-        if (jfixed(c)) return e;
+        if (e == cudaSuccess && c->jk_form == 1) ensure_jpack(c);
+        return e;
     }
     if (!c->d_part) e = pmalloc(&c->d_part, (size_t)c->nray * c->nvox * (c->ns == 1 ? 2 : 4) * c->rsz);
-    if (e == cudaSuccess && !jfixed(c)) jpack_or_wide(c);
+    if (e == cudaSuccess && use_jk(c) && c->jk_form == 1) ensure_jpack(c);
     // polarized lines of a multilevel atom: the per-ray integrals of Stokes V (J^1_Q)
     if (e == cudaSuccess && c->d_dich && !c->d_partv) e = pmalloc(&c->d_partv, (size_t)c->nray * c->nvox * c->rsz);
     // short characteristics on cell faces: the work planes and per-group partials
@@ -1092,6 +1089,7 @@ int porta_set_atmosphere(porta_ctx *c, const porta_atmos *a, int where)
     cudaStreamSynchronize(c->stream);
     if (rc == PORTA_OK) {
         c->have_atm = true;
+        c->jpack_failed = false;
         c->have_fs = c->have_jkq = false;
     }
     return rc;
@@ -1108,6 +1106,7 @@ int porta_set_rho(porta_ctx *c, const double *rho, int where)
         for (long long v = 0; v < c->nvox; ++v)
             if (!(rho[v * c->nl] > 0)) return fail(c, PORTA_EINVAL, "set_rho: S^0_0 must be > 0");
     }
+    c->jpack_failed = false;
     int rc = copy_in(c, c->d_rho, rho, n, where);
     if (rc) return rc;
     if (where == PORTA_DEVICE) {
@@ -1294,6 +1293,10 @@ int porta_run_iterations(porta_ctx *c, int iterations, double *max_change)
     if (!c->have_atm || !c->have_rho) return fail(c, PORTA_ESTATE, "run_iterations: atmosphere or rho not set");
     if (!c->stream) return fail(c, PORTA_ESTATE, "run_iterations: needs a non-default stream (porta_set_stream)");
     if (c->graph_exec && c->graph_stream != c->stream) drop_graph(c);
+    if (c->graph_exec && use_jk(c) && c->jk_form == 1 && !c->d_jpack) {
+        ensure_jpack(c);
+        if (c->d_jpack) drop_graph(c);          // (captured without the packed inputs)
+    }
     if (!c->graph_exec) {
         cudaError_t eb = ensure_sweep_buffers(c);   // no allocation inside the capture
         if (eb != cudaSuccess) return fail(c, PORTA_ENOMEM, std::string("run_iterations: ") + cudaGetErrorString(eb));

@@ -94,38 +94,37 @@ int emergent_shape(porta_ctx *c, SweepArgs<Real> &a, int ndir, LaunchCfg &cfg)
 // 40, 5 directions, 21 frequencies with the store 0.32 -> 0.23 ms, 16 x 16 x 24 in FP64, 32
 // rays, 7 frequencies 1.30 -> 0.90 ms, 64 x 64 x 64, 5 directions 0.64 -> 0.64 ms; and its shape
 // need not be timed (64 x 64 x 64: 42 ms of the first call). The general sweep remains for the
-// media that the other does not know (dichroism, explicit media, biquadratic stencils), for
-// planes that do not fit, and where the packed inputs cannot be allocated.
+// media that the other does not know (dichroism, explicit media, biquadratic stencils) and for
+// planes that do not fit.
 //
-// emergent_begin decides for ndir directions and has the inputs packed (the host can prepare
-// the directions meanwhile).
+// emergent_begin decides for ndir directions (jform: sweep_j.cu) and has the inputs packed
+// (the host can prepare the directions meanwhile).
 template <typename Real>
-int emergent_begin(porta_ctx *c, int ndir, LaunchCfg &cfg, bool &packed)
+int emergent_begin(porta_ctx *c, int ndir, LaunchCfg &cfg, bool &jform)
 {
-    packed = false;
+    jform = false;
     if (c->jk_form != 1 || c->d_dich || c->d_kexpl || c->interp == 2 || c->sc_faces || c->gsweep) return PORTA_OK;
     const int fc = c->user_shape ? c->opt_cluster : 0, ff = c->user_shape ? c->opt_nu_group : 0;
     const int rc = c->ns == 1 ? choose_launch<Real, 1>(c, cfg, fc, ff, ndir, true, c->n_nu, true)
                               : choose_launch<Real, 4>(c, cfg, fc, ff, ndir, true, c->n_nu, true);
-    if (rc != PORTA_OK || ensure_jpack(c) != cudaSuccess) {
-        cudaGetLastError();
-        return PORTA_OK;
-    }
+    if (rc != PORTA_OK) return PORTA_OK;
+    ensure_jpack(c);
+    jform = true;
+    if (!c->d_jpack) return PORTA_OK;
     SweepArgs<Real> a = base_args<Real>(c);
     a.pack = (const Real *)c->d_jpack;
     const cudaError_t e = c->ns == 1 ? launch_jacc_prepare<Real, 1>(a, c->stream) : launch_jacc_prepare<Real, 4>(a, c->stream);
     if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("emergent inputs: ") + cudaGetErrorString(e));
-    packed = true;
     return PORTA_OK;
 }
 
 // the sweep itself: directions a.rays, their geometry in the general form a.geom and in the
 // relative form rel
 template <typename Real>
-int emergent_sweep(porta_ctx *c, SweepArgs<Real> a, const PlaneGeom<Real> *rel, int ndir, LaunchCfg cfg, bool packed)
+int emergent_sweep(porta_ctx *c, SweepArgs<Real> a, const PlaneGeom<Real> *rel, int ndir, LaunchCfg cfg, bool jform)
 {
     cudaError_t e = cudaSuccess;
-    if (packed) {
+    if (jform) {
         shape_args<Real>(c, a, cfg, true);
         a.geom = rel;
         a.nitems = ndir;
@@ -207,8 +206,8 @@ int emergent_t(porta_ctx *c, int ndir, const double *mu, const double *chi, doub
 {
     check_global_sweep(c);
     LaunchCfg cfg{};
-    bool packed = false;
-    int rc = emergent_begin<Real>(c, ndir, cfg, packed);
+    bool jform = false;
+    int rc = emergent_begin<Real>(c, ndir, cfg, jform);
     if (rc) return rc;
     Directions<Real> dirs;
     cudaError_t e = put_directions<Real>(c, ndir, mu, chi, box, dirs);
@@ -246,7 +245,7 @@ int emergent_t(porta_ctx *c, int ndir, const double *mu, const double *chi, doub
             else if (flag & 2) rc = fail(c, PORTA_ENOTCONV, "emergent (faces): a plane of face points did not converge");
             break;
         }
-        rc = emergent_sweep<Real>(c, a, dirs.rel, ndir, cfg, packed);
+        rc = emergent_sweep<Real>(c, a, dirs.rel, ndir, cfg, jform);
         if (rc == PORTA_OK) rc = emergent_check(c);
     } while (0);
     if (rc != PORTA_OK) cudaStreamSynchronize(c->stream);
@@ -323,8 +322,8 @@ int emergent_vjp_t(porta_ctx *c, int ndir, const double *mu, const double *chi, 
     const long long nxy = (long long)c->nx * c->ny;
     double *scratch_out = nullptr;
     LaunchCfg cfg{};
-    bool packed = false;
-    int rc = emergent_begin<Real>(c, ndir, cfg, packed);
+    bool jform = false;
+    int rc = emergent_begin<Real>(c, ndir, cfg, jform);
     if (rc) return rc;
     Directions<Real> dirs;
     cudaError_t e2 = put_directions<Real>(c, ndir, mu, chi, 0, dirs);
@@ -348,7 +347,7 @@ int emergent_vjp_t(porta_ctx *c, int ndir, const double *mu, const double *chi, 
         a.store = (Real *)c->d_tape;
         e = cudaEventRecord(c->adj_ev[0], c->stream);
         if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, std::string("emergent_vjp: ") + cudaGetErrorString(e)); break; }
-        rc = emergent_sweep<Real>(c, a, dirs.rel, ndir, cfg, packed);
+        rc = emergent_sweep<Real>(c, a, dirs.rel, ndir, cfg, jform);
         if (rc) break;
         e = cudaEventRecord(c->adj_ev[1], c->stream);
         if (e != cudaSuccess) { rc = fail(c, PORTA_ECUDA, std::string("emergent_vjp forward: ") + cudaGetErrorString(e)); break; }
@@ -485,8 +484,8 @@ int jkq_vjp_t(porta_ctx *c, const double *dgj, const double *dgl, double *dg_chi
     if (e != cudaSuccess) return fail(c, PORTA_ENOMEM, "iterate_vjp: accumulator allocation");
     // forward: Stokes vectors of every node for rays r0 .. r0 + n - 1
     LaunchCfg fcfg{};
-    bool packed = false;
-    rc = emergent_begin<Real>(c, nb, fcfg, packed);
+    bool jform = false;
+    rc = emergent_begin<Real>(c, nb, fcfg, jform);
     if (rc) return rc;
     auto forward = [&](int r0, int n) -> int {
         SweepArgs<Real> a = base_args<Real>(c);
@@ -496,7 +495,7 @@ int jkq_vjp_t(porta_ctx *c, const double *dgj, const double *dgl, double *dg_chi
         a.store = (Real *)c->d_tape;
         size_t planes = 0;
         for (const BoxDev &b : c->boxes) planes += b.nz;
-        return emergent_sweep<Real>(c, a, a.geom + (size_t)c->nray * planes, n, fcfg, packed);
+        return emergent_sweep<Real>(c, a, a.geom + (size_t)c->nray * planes, n, fcfg, jform);
     };
     // reverse: the J^K_Q and Lambda-bar* terms of the same rays
     auto reverse = [&](int r0, int n, LaunchCfg k) -> int {

@@ -489,8 +489,8 @@ void shape_args(porta_ctx *c, SweepArgs<Real> &a, const LaunchCfg &cfg, bool jk 
 }
 
 // api.cu
-// the packed inputs of sweep_j.cu, allocated on first use
-cudaError_t ensure_jpack(porta_ctx *c);
+// the packed inputs of sweep_j.cu, allocated on first use (d_jpack stays null without room)
+void ensure_jpack(porta_ctx *c);
 void free_all(porta_ctx *c);
 bool finite_host(const double *x, long long n);
 // copy n doubles from a caller buffer (host or device) into device memory

@@ -256,6 +256,7 @@ int porta_ml_set_atmosphere(porta_ctx *c, const double *chi, const double *kT, c
     rc = porta_set_atmosphere(c, &at, PORTA_HOST);
     if (rc) return rc;
     m->have_atm = true;
+    c->jpack_failed = false;
     if (m->have_pops) {
         cudaError_t e = ml_prepare(c);
         if (e != cudaSuccess) return fail(c, PORTA_ECUDA, cudaGetErrorString(e));
@@ -293,6 +294,7 @@ int porta_ml_set_pops(porta_ctx *c, const double *pops, int where)
     CK(cudaStreamSynchronize(c->stream));
     if (hb) return fail(c, PORTA_EINVAL, "ml_set_pops: a line has a non-positive opacity (population inversion)");
     m->have_pops = true;
+    c->jpack_failed = false;
     c->have_rho = true;
     c->have_fs = c->have_jkq = false;
     return PORTA_OK;
@@ -389,6 +391,7 @@ int porta_ml_set_unknowns(porta_ctx *c, const double *x, int where)
     CK(cudaStreamSynchronize(c->stream));
     if (hb) return fail(c, PORTA_EINVAL, "ml_set_unknowns: non-positive population or line opacity");
     m->have_pops = true;
+    c->jpack_failed = false;
     c->have_rho = true;
     c->have_fs = c->have_jkq = false;
     return PORTA_OK;

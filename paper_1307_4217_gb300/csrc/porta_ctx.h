@@ -81,7 +81,8 @@ struct porta_ctx {
     void *d_part = nullptr;         // nray*nvox*(ns==1 ? 2 : 4) Real (general sweep only; allocated on first use)
     unsigned long long *d_jacc = nullptr;   // J^K_Q sweep: fixed-point sums [nj + 1][nvox] (allocated on first use)
     int *d_jexp = nullptr;                  // J^K_Q sweep: per-voxel fixed-point exponent
-    void *d_jpack = nullptr;                // J^K_Q sweep: packed inputs, jpack_words Reals per voxel
+    void *d_jpack = nullptr;                // J^K_Q sweep: packed inputs, jpack_words Reals per voxel (null: no room)
+    bool jpack_failed = false;              // their last allocation failed (ensure_jpack)
     double *d_tw = nullptr;         // nray*19 FP64: w_m, T (18)
     double *d_jkq = nullptr, *d_lstar = nullptr;
     unsigned long long *d_resid = nullptr;

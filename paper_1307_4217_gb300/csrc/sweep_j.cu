@@ -467,7 +467,9 @@ struct JPhase { unsigned full0, full1, freed0, freed1; };
 // Lambda*, PROBE), or the emergent Stokes profiles and, for the reverse mode, the Stokes
 // vectors of every node (EMERGENT: no sums, no profile normalization)
 enum JMode { SUMS = 0, PROBE_RAY = 1, EMERGENT = 2 };
-template <typename Real, int NS, int MODE>
+// PACKED: the voxels' inputs lie side by side in a.pack. (A form of its own: the test of
+// a.pack in one kernel cost 1.2% of a 64 x 64 x 64 formal solution, 17.89 -> 18.11 ms.)
+template <typename Real, int NS, int MODE, bool PACKED>
 __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsigned sbase, const JSmem &sm,
                                             const JBars &bars, JPhase &ph, const unsigned sray, const unsigned stab, int box, int m, int g,
                                             int rank, int C)
@@ -554,6 +556,22 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
     // Inputs of plane q's nodes on their way to shared memory; the thread that asked for a
     // node's values is the one that fills the node a phase later. (Wrapped by an unsigned
     // minimum: x - n is huge below n.)
+    // (no room for the packed inputs: a node's words one by one from where they are, into the
+    // places of the packed ones)
+    auto fetch_words = [&](unsigned d, int v) {
+        auto put = [&](int w, const Real *src) {
+            copy_async(d + w / W::per * nodes * 16 + w % W::per * SZ, src + v);
+        };
+        put(0, a.chi);
+        put(1, a.vel);
+#pragma unroll 1
+        for (int k = 0; k < (NS == 1 ? 1 : 6); ++k) put(2 + k, a.rho + (size_t)k * a.nvox);
+        if constexpr (NS == 4) {
+            put(8, a.bx);
+            put(9, a.by);
+            put(10, a.bz);
+        }
+    };
     const int jown = row0 + rowt - 1 + (row0 + rowt == 0 ? ny : 0) - (row0 + rowt > ny ? ny : 0);
     auto fetch = [&](int q) {
         if (rtid >= nn) return;
@@ -564,13 +582,17 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
         for (int idx = rtid; idx < nn; idx += nt) {
             const int pi = wrap(c + g4[0], nx), pj = wrap(j + g4[1], ny);
             const int v = base + pj * nx + pi;
-            const Real *src = a.pack + (size_t)(unsigned)v * W::staged;
             const unsigned d = sbase + sm.stage + idx * 16;
             sts(sbase + sm.stv + idx * 4, v);
             if (!EMG) copy_async(sbase + sm.stw + idx * SZ, invn + v);
             if (!EMG && a.jacc) copy_async(sbase + sm.ste + idx * 4, a.jexp + v);
+            if constexpr (PACKED) {
+                const Real *src = a.pack + (size_t)(unsigned)v * W::staged;
 #pragma unroll
-            for (int h = 0; h < SCH; ++h) copy_async16(d + h * nodes * 16, src + h * W::per);
+                for (int h = 0; h < SCH; ++h) copy_async16(d + h * nodes * 16, src + h * W::per);
+            } else {
+                fetch_words(d, v);
+            }
             c += dc;
             j += dl;
             if (c >= nx) { c -= nx; ++j; }
@@ -1130,7 +1152,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
     }
 }
 
-template <typename Real, int NS, int MODE>
+template <typename Real, int NS, int MODE, bool PACKED>
 __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kernel(const SweepArgs<Real> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1179,7 +1201,7 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
         // the ray's constants (mu, ox, oy, oz, T[18], w, pad); the item starts with a barrier
         if (threadIdx.x < 24) sray[threadIdx.x] = reinterpret_cast<const Real *>(a.rays + m)[threadIdx.x];
         for (int g = g0; g < (split > 1 ? g0 + 1 : a.ngroups); ++g) {
-            jsweep_item<Real, NS, MODE>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), smem_u32(s_exp), box, m, g, rank, C);
+            jsweep_item<Real, NS, MODE, PACKED>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), smem_u32(s_exp), box, m, g, rank, C);
             // every halo row of the item has been written and read before the next one
             // (whose strips may have other neighbours)
             if (C > 1) cluster.sync();
@@ -1192,8 +1214,8 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
 // carries 46 fraction bits and the accumulator has 2^16 of headroom above it
 // (an FP32 term then converts without rounding; an FP64 term rounds at 2^-47 of
 // the reference value).
-// (jacc null: the FP64 form, which has no fixed-point sums; pack null: sweep_jw.cu, which
-// reads the inputs where they are). The same pass packs each
+// (jacc null: the FP64 form, which has no fixed-point sums; pack null: sweep_jw.cu, or no
+// room for them: the inputs are read where they are). The same pass packs each
 // voxel's inputs of the sweep next to each other, so that a node's inputs arrive in
 // shared memory by 16-byte copies: chi, vel, rho[6], bx, by, bz (NS = 1: chi, vel, rho).
 template <typename Real, int NS>
@@ -1261,10 +1283,10 @@ cudaError_t launch_jacc_finalize(long long nvox, const unsigned long long *jacc,
     return cudaGetLastError();
 }
 
-template <typename Real, int NS, int MODE>
+template <typename Real, int NS, int MODE, bool PACKED>
 static cudaError_t jprepare(int cluster, int smem)
 {
-    void *k = (void *)jsweep_kernel<Real, NS, MODE>;
+    void *k = (void *)jsweep_kernel<Real, NS, MODE, PACKED>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     if (cluster > 8) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1274,7 +1296,7 @@ static cudaError_t jprepare(int cluster, int smem)
 template <typename Real, int NS>
 cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out)
 {
-    cudaError_t e = jprepare<Real, NS, SUMS>(cluster, smem);
+    cudaError_t e = jprepare<Real, NS, SUMS, true>(cluster, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(cluster);
@@ -1287,15 +1309,16 @@ cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *
     at[0].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(out, jsweep_kernel<Real, NS, SUMS>, &lc);
+    return cudaOccupancyMaxActiveClusters(out, jsweep_kernel<Real, NS, SUMS, true>, &lc);
 }
 
 // the probe variant writes one ray's Stokes vectors and Lambda* at every node and
-// frequency (porta_probe_ray); the plain one keeps no trace of that in its loop
-template <typename Real, int NS, int MODE>
+// frequency (porta_probe_ray); the plain one keeps no trace of that in its loop. A diagnostic,
+// it has the form that needs no packed inputs only.
+template <typename Real, int NS, int MODE, bool PACKED>
 static cudaError_t jlaunch(const SweepArgs<Real> &a, const LaunchCfg &cfg, cudaStream_t st)
 {
-    cudaError_t e = jprepare<Real, NS, MODE>(cfg.cluster, cfg.smem);
+    cudaError_t e = jprepare<Real, NS, MODE, PACKED>(cfg.cluster, cfg.smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(cfg.clusters * cfg.cluster);
@@ -1314,14 +1337,15 @@ static cudaError_t jlaunch(const SweepArgs<Real> &a, const LaunchCfg &cfg, cudaS
         at[1].val.priority = cfg.priority;
         lc.numAttrs = 2;
     }
-    return cudaLaunchKernelEx(&lc, jsweep_kernel<Real, NS, MODE>, a);
+    return cudaLaunchKernelEx(&lc, jsweep_kernel<Real, NS, MODE, PACKED>, a);
 }
 
 template <typename Real, int NS>
 cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st)
 {
-    if (a.out) return jlaunch<Real, NS, EMERGENT>(a, cfg, st);
-    return a.probe_ray >= 0 ? jlaunch<Real, NS, PROBE_RAY>(a, cfg, st) : jlaunch<Real, NS, SUMS>(a, cfg, st);
+    if (a.out) return a.pack ? jlaunch<Real, NS, EMERGENT, true>(a, cfg, st) : jlaunch<Real, NS, EMERGENT, false>(a, cfg, st);
+    if (a.probe_ray >= 0) return jlaunch<Real, NS, PROBE_RAY, false>(a, cfg, st);
+    return a.pack ? jlaunch<Real, NS, SUMS, true>(a, cfg, st) : jlaunch<Real, NS, SUMS, false>(a, cfg, st);
 }
 
 #define PORTA_JINST(R, N)                                                                    \
