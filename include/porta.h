@@ -56,7 +56,12 @@
  *     synchronize that stream.
  *   * Errors: every int-returning function returns PORTA_OK (0) or a negative
  *     status; porta_last_error gives a message. Invalid arguments are rejected
- *     before anything is launched. A context is not thread-safe.
+ *     before anything is launched. A context is not thread-safe. What a formal
+ *     solution finds out on the device (PORTA_EKERNEL, PORTA_ENOTCONV) is
+ *     reported by the call that hands its sums to the host; where they went on
+ *     on the device (into the unknowns, a device buffer, another rank), by the
+ *     next call on the context that synchronizes for a residual, the unknowns
+ *     or J^K_Q. Each is reported once.
  */
 #ifndef PORTA_H
 #define PORTA_H
@@ -389,6 +394,12 @@ int porta_set_fill(porta_ctx *c, int cluster_size, int nu_group, double fraction
    out[6*i + 0..5] = e^-t, psi'_M, psi'_O, omega_M, omega_O, omega_C (host).
    Synchronous; uses the current device. */
 int porta_eval_coefficients(int precision, int n, const double *t, double *out);
+
+/* Diagnostic: the bounded wait with which the strips of a J^K_Q sweep wait for one
+   another, on a row that never arrives. seconds (host) receives how long it
+   waited. PORTA_EKERNEL: the wait ran out and set the error flag, as it must.
+   Synchronous; uses the current device. */
+int porta_eval_halo_wait(double *seconds);
 
 /* Allocation-free formal solution. (The paper has no counterpart: this entry
    point exists for callers that cannot allocate device memory, e.g. a host

@@ -83,6 +83,7 @@ _SIGS = {
     "porta_fma_peak": (_I, [_I, ctypes.c_double, _P, _P]),
     "porta_set_freq_range": (_I, [_P, _I, _I]),
     "porta_residual": (_I, [_P, _P]),
+    "porta_eval_halo_wait": (_I, [_P]),
     "porta_eval_step": (_I, [_I, _I, _P, _P]),
     "porta_sigmoid_error": (_I, [_I, _I, _P, _P, _P, _P]),
     "porta_set_interpolation": (_I, [_P, _I]),
@@ -279,6 +280,11 @@ def porta_eval_coefficients(precision, t):
     out = np.zeros((len(t), 6))
     rc = lib().porta_eval_coefficients(precision, len(t), t.ctypes.data, out.ctypes.data)
     return rc, out
+
+
+def porta_eval_halo_wait():
+    s = ctypes.c_double()
+    return lib().porta_eval_halo_wait(ctypes.byref(s)), s.value
 
 
 def porta_formal_solve_noalloc(atm, model, n_mu, n_chi, n_nu, x_max, datm, rho_ptr, jkq_ptr, lstar_ptr, stream=None):

@@ -351,18 +351,17 @@ cudaError_t ensure_sweep_buffers(porta_ctx *c)
     return e;
 }
 
-// zero the fixed-point sums and set the voxels' scales before a J^K_Q sweep
+// zero the error flag and the fixed-point sums and set the voxels' scales before a J^K_Q sweep
 template <typename Real>
 cudaError_t jacc_prepare(porta_ctx *c, const SweepArgs<Real> &a)
 {
-    if (!use_jk(c) || (c->jk_form == 2 && !jfixed(c))) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
-    if (e != cudaSuccess) return e;
+    if (!use_jk(c) || (c->jk_form == 2 && !jfixed(c))) return cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
     return c->ns == 1 ? launch_jacc_prepare<Real, 1>(a, c->stream) : launch_jacc_prepare<Real, 4>(a, c->stream);
 }
 
 // J^K_Q and Lambda-bar* (FP64) from the sums of the last formal solution; for the
-// polarized lines of a multilevel atom also J^1_Q (d_j1)
+// polarized lines of a multilevel atom also J^1_Q (d_j1). The solution's error flag goes with
+// them: the next formal solution clears its own, while these sums are in the unknowns.
 cudaError_t finalize_jkq(porta_ctx *c)
 {
     if (c->d_j1) {
@@ -372,27 +371,34 @@ cudaError_t finalize_jkq(porta_ctx *c)
         if (e != cudaSuccess) return e;
     }
     if (jfixed(c))
-        return c->ns == 1 ? launch_jacc_finalize<1>(c->nvox, c->d_jacc, c->d_jexp, c->d_jkq, c->d_lstar, c->stream)
-                          : launch_jacc_finalize<4>(c->nvox, c->d_jacc, c->d_jexp, c->d_jkq, c->d_lstar, c->stream);
+        return c->ns == 1 ? launch_jacc_finalize<1>(c->nvox, c->d_jacc, c->d_jexp, c->d_jkq, c->d_lstar, c->d_err, c->d_handed, c->stream)
+                          : launch_jacc_finalize<4>(c->nvox, c->d_jacc, c->d_jexp, c->d_jkq, c->d_lstar, c->d_err, c->d_handed, c->stream);
     if (c->precision == PORTA_FP32)
-        return c->ns == 1 ? run_jkq_finalize<float, 1>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream)
-                          : run_jkq_finalize<float, 4>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream);
-    return c->ns == 1 ? run_jkq_finalize<double, 1>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream)
-                      : run_jkq_finalize<double, 4>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream);
+        return c->ns == 1 ? run_jkq_finalize<float, 1>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream, c->d_err, c->d_handed)
+                          : run_jkq_finalize<float, 4>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream, c->d_err, c->d_handed);
+    return c->ns == 1 ? run_jkq_finalize<double, 1>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream, c->d_err, c->d_handed)
+                      : run_jkq_finalize<double, 4>(c->nvox, c->nray, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->stream, c->d_err, c->d_handed);
 }
 
-// the fixed-point sums' overflow flag (reads device memory: synchronizes the stream)
-int check_jacc(porta_ctx *c)
+// The value of the last residual (value may be null) and the errors of the formal solutions
+// whose sums were handed on since the last report: to the unknowns, to the caller or to
+// another rank. One read, which synchronizes the stream; what it reports it clears.
+int read_status(porta_ctx *c, double *value)
 {
-    if ((!use_jk(c) || (c->jk_form == 2 && !jfixed(c))) && !c->sc_faces && !c->gsweep && !c->d_kexpl) return PORTA_OK;
-    int flag = 0;
-    CK(cudaMemcpyAsync(&flag, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    struct {
+        unsigned long long bits;
+        int err[4];
+    } s;
+    CK(cudaMemcpyAsync(&s, c->d_resid, sizeof(s), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    if (value) std::memcpy(value, &s.bits, sizeof(double));
+    const int flag = s.err[2];
+    if (!flag) return PORTA_OK;
+    CK(cudaMemsetAsync(c->d_handed, 0, sizeof(int), c->stream));
     if (flag & 2) return fail(c, PORTA_ENOTCONV, "formal solution: a plane of face points did not converge");
     if (flag & 4) return fail(c, PORTA_EKERNEL, "formal solution: a strip's wait for its neighbour ran out");
-    if (flag) return fail(c, PORTA_EKERNEL, "formal solution: a J^K_Q term exceeded the fixed-point range (2^16 times "
-                                            "max(|S^0_0|, |B|) of its voxel), or was not finite");
-    return PORTA_OK;
+    return fail(c, PORTA_EKERNEL, "formal solution: a J^K_Q term exceeded the fixed-point range (2^16 times "
+                                  "max(|S^0_0|, |B|) of its voxel), or was not finite");
 }
 
 cudaError_t ensure_fill(porta_ctx *c)
@@ -690,7 +696,7 @@ void free_all(porta_ctx *c)
     for (cudaEvent_t &ev : c->adj_ev)
         if (ev) cudaEventDestroy(ev);
     void *ptrs[] = {c->d_atm, c->d_eps, c->d_bpl, c->d_b, c->d_rho, c->d_rhoR, c->d_invn, c->d_geom, c->d_rays,
-                    c->d_freq, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->d_resid, c->d_err, c->d_dirs, c->d_boxes,
+                    c->d_freq, c->d_part, c->d_tw, c->d_jkq, c->d_lstar, c->d_resid, c->d_dirs, c->d_boxes,
                     c->d_items, c->d_tune_items, c->d_tape, c->d_gpart, c->d_jacc, c->d_jexp, c->d_jpack, c->d_kexpl, c->d_sexpl,
                     c->d_partv, c->d_j1, c->d_tw1, c->d_gjR, c->d_vjp_out, c->d_faces, c->d_fdxy};
     for (void *p : ptrs)
@@ -856,9 +862,12 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
     ok(dalloc(&c->d_tw, (size_t)c->nray * 19));
     ok(dalloc(&c->d_jkq, nvox * c->nj));
     ok(dalloc(&c->d_lstar, nvox));
-    ok(dalloc(&c->d_resid, 1));
-    ok(dalloc(&c->d_err, 2));     // formal solution; emergent sweep (sticky until read)
-    if (rc == PORTA_OK) ok(cudaMemset(c->d_err, 0, 2 * sizeof(int)));
+    ok(dalloc(&c->d_resid, 3));
+    if (rc == PORTA_OK) {
+        c->d_err = reinterpret_cast<int *>(c->d_resid + 1);
+        c->d_handed = c->d_err + 2;
+        ok(cudaMemset(c->d_resid, 0, 24));
+    }
     if (rc == PORTA_OK) {
         ok(cudaMemset(c->d_atm, 0, 6 * nvox * R));
         // geometry, rays, frequencies, angular weights
@@ -1130,8 +1139,7 @@ int porta_get_rho(porta_ctx *c, double *rho, int where)
     if (!c->have_rho) return fail(c, PORTA_ESTATE, "get_rho: rho has not been set");
     CK(cudaMemcpyAsync(rho, c->d_rho, c->nvox * c->nl * sizeof(double),
                        where == PORTA_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-    if (where == PORTA_HOST) CK(cudaStreamSynchronize(c->stream));
-    return PORTA_OK;
+    return where == PORTA_HOST ? read_status(c, nullptr) : PORTA_OK;
 }
 
 int porta_formal_solve(porta_ctx *c)
@@ -1161,7 +1169,7 @@ int porta_accumulate_jkq(porta_ctx *c, double *jkq, double *lstar, int where)
     if (jkq) CK(cudaMemcpyAsync(jkq, c->d_jkq, c->nvox * c->nj * sizeof(double), k, c->stream));
     if (lstar) CK(cudaMemcpyAsync(lstar, c->d_lstar, c->nvox * sizeof(double), k, c->stream));
     if (where == PORTA_HOST && (jkq || lstar)) {
-        int rc = check_jacc(c);
+        int rc = read_status(c, nullptr);
         if (rc != PORTA_OK) return rc;
     }
     c->have_jkq = true;
@@ -1175,15 +1183,7 @@ int porta_see_update(porta_ctx *c, double *max_change)
     cudaError_t e = enqueue_update(c);
     if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("see_update: ") + cudaGetErrorString(e));
     c->have_fs = c->have_jkq = false;
-    if (max_change) {
-        unsigned long long bits = 0;
-        CK(cudaMemcpyAsync(&bits, c->d_resid, sizeof(bits), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        double v;
-        std::memcpy(&v, &bits, sizeof(v));
-        *max_change = v;
-    }
-    return PORTA_OK;
+    return max_change ? read_status(c, max_change) : PORTA_OK;
 }
 
 int porta_probe_ray(porta_ctx *c, int m, double *out, double *lstar, int where)
@@ -1223,9 +1223,12 @@ int porta_probe_ray(porta_ctx *c, int m, double *out, double *lstar, int where)
         cudaMemcpyKind k = where == PORTA_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, d1, n * c->ns * sizeof(double), k, c->stream);
         if (e == cudaSuccess && lstar) e = cudaMemcpyAsync(lstar, d2, n * sizeof(double), k, c->stream);
+        int flag = 0;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
         cudaError_t e2 = cudaStreamSynchronize(c->stream);
         if (e == cudaSuccess) e = e2;
         if (e != cudaSuccess) rc = fail(c, PORTA_ECUDA, std::string("probe_ray: ") + cudaGetErrorString(e));
+        else if (flag & 4) rc = fail(c, PORTA_EKERNEL, "probe_ray: a strip's wait for its neighbour ran out");
     }
     cudaStreamSynchronize(c->stream);
     pfree(pr);
@@ -1253,6 +1256,24 @@ int porta_eval_coefficients(int precision, int n, const double *t, double *out)
     if (e == cudaSuccess) e = cudaMemcpy(out, d + n, sizeof(double) * 6 * (size_t)n, cudaMemcpyDeviceToHost);
     pfree(d);
     return e == cudaSuccess ? PORTA_OK : PORTA_ECUDA;
+}
+
+int porta_eval_halo_wait(double *seconds)
+{
+    if (!seconds) return PORTA_EINVAL;
+    int *d = nullptr;
+    if (dalloc(&d, 4) != cudaSuccess) return PORTA_ENOMEM;
+    struct {
+        int err, pad;
+        unsigned long long ns;
+    } h = {};
+    cudaError_t e = cudaMemset(d, 0, sizeof(h));
+    if (e == cudaSuccess) e = run_halo_wait(d, reinterpret_cast<unsigned long long *>(d + 2), nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(&h, d, sizeof(h), cudaMemcpyDeviceToHost);
+    pfree(d);
+    if (e != cudaSuccess) return PORTA_ECUDA;
+    *seconds = 1e-9 * (double)h.ns;
+    return h.err & 4 ? PORTA_EKERNEL : PORTA_OK;
 }
 
 int porta_eval_step(int precision, int n, const double *in, double *out)
@@ -1327,17 +1348,7 @@ int porta_run_iterations(porta_ctx *c, int iterations, double *max_change)
     }
     for (int it = 0; it < iterations; ++it) CK(cudaGraphLaunch(c->graph_exec, c->stream));
     c->have_fs = c->have_jkq = false;
-    if (max_change) {
-        unsigned long long bits = 0;
-        CK(cudaMemcpyAsync(&bits, c->d_resid, sizeof(bits), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        double v;
-        std::memcpy(&v, &bits, sizeof(v));
-        *max_change = v;
-        int rc = check_jacc(c);
-        if (rc != PORTA_OK) return rc;
-    }
-    return PORTA_OK;
+    return max_change ? read_status(c, max_change) : PORTA_OK;
 }
 
 int porta_set_device_limit(long long bytes)

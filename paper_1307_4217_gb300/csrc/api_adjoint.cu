@@ -232,12 +232,12 @@ int emergent_t(porta_ctx *c, int ndir, const double *mu, const double *chi, doub
                                                  : faces_scratch_bytes<Real, 4>(1, ndir, c->n_nu, nxy, c->nvox, c->d_dich ? 1 : (c->d_kexpl ? 2 : 0)));
             if (e == cudaSuccess) e = pmalloc((void **)&ddxy, sizeof(dxy));
             if (e == cudaSuccess) e = cudaMemcpyAsync(ddxy, dxy, sizeof(dxy), cudaMemcpyHostToDevice, c->stream);
-            if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err + 3, 0, sizeof(int), c->stream);
             if (e == cudaSuccess)
-                e = c->ns == 1 ? launch_faces<Real, 1>(a, ws, 1, nxy, ddxy, 100000, c->d_err, c->stream, true, !c->sc_faces)
-                               : launch_faces<Real, 4>(a, ws, 1, nxy, ddxy, 100000, c->d_err, c->stream, true, !c->sc_faces);
+                e = c->ns == 1 ? launch_faces<Real, 1>(a, ws, 1, nxy, ddxy, 100000, c->d_err + 3, c->stream, true, !c->sc_faces)
+                               : launch_faces<Real, 4>(a, ws, 1, nxy, ddxy, 100000, c->d_err + 3, c->stream, true, !c->sc_faces);
             int flag = 0;
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, c->d_err + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
             if (ws) pfree(ws);
             if (ddxy) pfree(ddxy);
@@ -697,10 +697,10 @@ int iterate_vjp_t(porta_ctx *c, int ndir, const double *mu, const double *chi, c
     }
     // leave the context at the final unknowns
     int rc2 = it_load(c, c->it_final);
-    cudaStreamSynchronize(c->stream);
+    const int rc3 = read_status(c, nullptr);
     pfree(blk);
     if (seg) pfree(seg);
-    return rc ? rc : rc2;
+    return rc ? rc : (rc2 ? rc2 : rc3);
 }
 
 }  // namespace porta_api
@@ -810,8 +810,9 @@ int porta_iterate_ckpt(porta_ctx *c, int niter, int ckpt, double *max_change)
     }
     if (rc == PORTA_OK) {
         cudaError_t e = cudaMemcpyAsync(c->it_final, c->d_rho, sizeof(double) * nr, cudaMemcpyDeviceToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) rc = fail(c, PORTA_ECUDA, std::string("iterate_ckpt: ") + cudaGetErrorString(e));
+        const int rs = read_status(c, nullptr);
+        if (rc == PORTA_OK) rc = rs;
     }
     if (rc) {
         it_free(c);

@@ -489,6 +489,8 @@ void shape_args(porta_ctx *c, SweepArgs<Real> &a, const LaunchCfg &cfg, bool jk 
 }
 
 // api.cu
+// residual and errors of the formal solutions handed on (synchronizes)
+int read_status(porta_ctx *c, double *value);
 // the packed inputs of sweep_j.cu, allocated on first use (d_jpack stays null without room)
 void ensure_jpack(porta_ctx *c);
 void free_all(porta_ctx *c);

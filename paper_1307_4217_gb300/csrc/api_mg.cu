@@ -275,6 +275,7 @@ int porta_mg_setup(porta_ctx *c, int nlevels)
             }
             c->mg.push_back(L);
             porta_set_stream(L, c->stream);
+            L->d_handed = c->d_handed;      // (reported with the finest level's)
             const MlState *mf = F->ml;
             const long long ncv = L->ml->nvox1;
             double *tmp = nullptr;
@@ -321,6 +322,7 @@ int porta_mg_setup(porta_ctx *c, int nlevels)
         }
         c->mg.push_back(L);
         porta_set_stream(L, c->stream);
+        L->d_handed = c->d_handed;      // (reported with the finest level's)
         // coarse atmosphere: the finer level's values at the coincident nodes
         const long long nf = F->nvox, ncv = L->nvox;
         double *tmp = nullptr;
@@ -406,11 +408,8 @@ int porta_residual(porta_ctx *c, double *rnorm)
         e = mg_apply(c, -1.0, nullptr, 1, r);                    // r = f - A(x)
         if (e == cudaSuccess) e = cudaMemsetAsync(c->d_resid, 0, sizeof(unsigned long long), c->stream);
         if (e == cudaSuccess) e = run_rel_residual(nu, nc, r, mg_unk(c), c->d_resid, c->stream);
-        unsigned long long bits = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bits, c->d_resid, sizeof(bits), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e == cudaSuccess) std::memcpy(rnorm, &bits, sizeof(double));
-        else rc = fail(c, PORTA_ECUDA, std::string("residual: ") + cudaGetErrorString(e));
+        rc = read_status(c, rnorm);
+        if (e != cudaSuccess) rc = fail(c, PORTA_ECUDA, std::string("residual: ") + cudaGetErrorString(e));
     }
     pfree(r);
     c->have_fs = c->have_jkq = false;
@@ -440,12 +439,7 @@ int porta_mg_vcycle(porta_ctx *c, int npre, int npost, int ncoarse, double *max_
                         ? run_mlpol_change(c->ml->mc, c->ml->dev, nu, c->mg_prev, mg_unk(c), c->d_resid, c->stream)
                         : run_change(nu, nc, c->mg_prev, mg_unk(c), c->d_resid, c->stream, c->ml ? 1 : 0);
     if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("mg_vcycle: ") + cudaGetErrorString(e));
-    if (max_change) {
-        unsigned long long bits = 0;
-        CK(cudaMemcpyAsync(&bits, c->d_resid, sizeof(bits), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        std::memcpy(max_change, &bits, sizeof(double));
-    }
+    if ((max_change || c->ml) && (rc = read_status(c, max_change))) return rc;
     if (c->ml) {
         for (porta_ctx *L : levels)
             if ((rc = ml_check(L, "mg_vcycle"))) return L == c ? rc : fail(c, rc, L->err);
@@ -521,12 +515,7 @@ int porta_mg_nested(porta_ctx *c, int ncycles, int npre, int npost, int ncoarse,
     e = c->ml && c->ml->pol ? run_mlpol_change(c->ml->mc, c->ml->dev, nu, c->mg_prev, mg_unk(c), c->d_resid, c->stream)
                             : run_change(nu, nc, c->mg_prev, mg_unk(c), c->d_resid, c->stream, c->ml ? 1 : 0);
     if (e != cudaSuccess) return fail(c, PORTA_ECUDA, std::string("mg_nested: ") + cudaGetErrorString(e));
-    if (max_change) {
-        unsigned long long bits = 0;
-        CK(cudaMemcpyAsync(&bits, c->d_resid, sizeof(bits), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        std::memcpy(max_change, &bits, sizeof(double));
-    }
+    if ((max_change || c->ml) && (rc = read_status(c, max_change))) return rc;
     if (c->ml) {
         for (porta_ctx *L : levels)
             if ((rc = ml_check(L, "mg_nested"))) return L == c ? rc : fail(c, rc, L->err);

@@ -310,7 +310,8 @@ int porta_ml_get_pops(porta_ctx *c, double *pops, int where)
     if (m->pol) {
         std::vector<double> hx((size_t)m->nvox1 * m->nunk), hp((size_t)m->nvox1 * m->mc.nlev);
         CK(cudaMemcpyAsync(hx.data(), m->d_x, hx.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        const int rc = read_status(c, nullptr);
+        if (rc != PORTA_OK) return rc;
         for (long long v = 0; v < m->nvox1; ++v)
             for (int i = 0; i < m->mc.nlev; ++i)
                 hp[v * m->mc.nlev + i] = std::sqrt(m->mc.g[i]) * hx[v * m->nunk + m->tab.pop_idx[i]];
@@ -320,8 +321,7 @@ int porta_ml_get_pops(porta_ctx *c, double *pops, int where)
     }
     CK(cudaMemcpyAsync(pops, m->d_pops, m->nvox1 * m->mc.nlev * sizeof(double),
                        where == PORTA_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-    if (where == PORTA_HOST) CK(cudaStreamSynchronize(c->stream));
-    return PORTA_OK;
+    return where == PORTA_HOST ? read_status(c, nullptr) : PORTA_OK;
 }
 
 int porta_ml_emergent_stokes(porta_ctx *c, int line, int ndir, const double *mu, const double *chi, double *out,
@@ -407,8 +407,7 @@ int porta_ml_get_unknowns(porta_ctx *c, double *x, int where)
     if (!m->have_pops) return fail(c, PORTA_ESTATE, "ml_get_unknowns: unknowns not set");
     CK(cudaMemcpyAsync(x, m->d_x, m->nvox1 * m->nunk * sizeof(double),
                        where == PORTA_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-    if (where == PORTA_HOST) CK(cudaStreamSynchronize(c->stream));
-    return PORTA_OK;
+    return where == PORTA_HOST ? read_status(c, nullptr) : PORTA_OK;
 }
 
 int porta_ml_formal_solve(porta_ctx *c, double *jbar, double *lstar, int where)
@@ -456,6 +455,7 @@ int porta_ml_iterate(porta_ctx *c, int iterations, double *max_change)
         rc = porta_ml_formal_solve(c, nullptr, nullptr, PORTA_DEVICE);
         if (rc == PORTA_OK) rc = porta_see_update(c, it == iterations - 1 ? max_change : nullptr);
     }
+    if (rc == PORTA_OK && !max_change) rc = read_status(c, nullptr);
     if (rc == PORTA_OK) rc = ml_check(c, "ml_iterate");
     return rc;
 }

@@ -85,7 +85,7 @@ struct porta_ctx {
     bool jpack_failed = false;              // their last allocation failed (ensure_jpack)
     double *d_tw = nullptr;         // nray*19 FP64: w_m, T (18)
     double *d_jkq = nullptr, *d_lstar = nullptr;
-    unsigned long long *d_resid = nullptr;
+    unsigned long long *d_resid = nullptr;   // residual; the four words of d_err follow
     // batched problems: per-box sizes, grids and offsets
     int nbox = 1;
     std::vector<porta::BoxDev> boxes;
@@ -95,7 +95,10 @@ struct porta_ctx {
     int *d_items = nullptr;        // nbox*nray work items ordered by decreasing cost
     int *d_tune_items = nullptr;   // strided sample of the work items for the autotuner
     int n_tune = 0;
-    int *d_err = nullptr;               // error flags: formal solution, emergent sweeps
+    // error flags: 0 the formal solution in flight, 1 emergent sweeps, 2 formal solutions whose sums
+    // were handed on (stays set until a synchronizing call has reported it), 3 emergent face sweeps
+    int *d_err = nullptr;
+    int *d_handed = nullptr;            // word 2; of a multigrid level: the finest level's
     int *h_flag = nullptr;              // page-locked, receives the latter
     void *d_dirs = nullptr;             // directions of the last emergent call (put_directions)
     size_t dirs_bytes = 0;

@@ -149,6 +149,8 @@ __host__ __device__ inline int jsweep_threads(int nx, int R, int FX, int tmax)
 template <typename Real, int NS> constexpr int jsweep_max_threads() { return NS == 4 && sizeof(Real) == 8 ? 256 : 512; }
 template <typename Real, int NS>
 int jsweep_smem_bytes(int nodes, int ipts, int tots, int F);
+// (diagnostic: the halo exchange's bounded wait on a row that never arrives)
+cudaError_t run_halo_wait(int *err, unsigned long long *ns, cudaStream_t st);
 template <typename Real, int NS>
 cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out);
 // (a.out set: the emergent Stokes profiles of the nitems directions of a.rays, a.geom)
@@ -178,7 +180,7 @@ template <typename Real, int NS>
 cudaError_t launch_jacc_prepare(const SweepArgs<Real> &a, cudaStream_t st);
 template <int NS>
 cudaError_t launch_jacc_finalize(long long nvox, const unsigned long long *jacc, const int *jexp, double *jkq,
-                                 double *lstar, cudaStream_t st);
+                                 double *lstar, const int *err, int *handed, cudaStream_t st);
 
 // adjoint of the emergent sweep (adjoint.cu): shared memory of a launch with
 // ring plane `ring_plane` (16-byte chunks), `ipts` points per strip, tape

@@ -80,7 +80,8 @@ struct KahanSum {
 
 template <typename Real, int NS>
 __global__ void jkq_finalize_kernel(long long nvox, int nray, const void *part, const double *tw,
-                                    double *jkq, double *lstar)
+                                    double *jkq, double *lstar,
+                                    const int *err, int *handed)
 {
     // the ray weights and tensors in the sums' precision, converted once per block
     extern __shared__ __align__(16) unsigned char fin_smem[];
@@ -89,6 +90,7 @@ __global__ void jkq_finalize_kernel(long long nvox, int nray, const void *part, 
     __syncthreads();
     long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (v >= nvox) return;
+    const int flag = v == 0 && err ? *err : 0;
     const Real *p = reinterpret_cast<const Real *>(part);
     if constexpr (NS == 1) {
         KahanSum<Real> J, L;
@@ -117,6 +119,7 @@ __global__ void jkq_finalize_kernel(long long nvox, int nray, const void *part, 
         for (int c = 0; c < 6; ++c) jkq[v * 6 + c] = (double)J[c].s;
         lstar[v] = (double)L.s;
     }
+    if (flag) atomicOr(handed, flag);
 }
 
 // J^1_Q of polarized lines from the per-ray frequency integrals of Stokes V:
@@ -294,13 +297,13 @@ cudaError_t run_rho_convert(long long nvox, int nl, const double *rho, void *out
 
 template <typename Real, int NS>
 cudaError_t run_jkq_finalize(long long nvox, int nray, const void *part, const double *tw, double *jkq, double *lstar,
-                             cudaStream_t st)
+                             cudaStream_t st, const int *err, int *handed)
 {
     const size_t smem = (size_t)nray * 19 * sizeof(Real);
     cudaError_t e = cudaFuncSetAttribute(jkq_finalize_kernel<Real, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int t = spread(nvox);
-    jkq_finalize_kernel<Real, NS><<<nblk(nvox, t), t, smem, st>>>(nvox, nray, part, tw, jkq, lstar);
+    jkq_finalize_kernel<Real, NS><<<nblk(nvox, t), t, smem, st>>>(nvox, nray, part, tw, jkq, lstar, err, handed);
     return cudaGetLastError();
 }
 
@@ -454,9 +457,9 @@ template cudaError_t run_coefficients<double>(int, const double *, double *, cud
                                              const double *, void *, cudaStream_t);                           \
     template cudaError_t run_rho_convert<R>(long long, int, const double *, void *, cudaStream_t);              \
     template cudaError_t run_jkq_finalize<R, 1>(long long, int, const void *, const double *, double *, double *, \
-                                                cudaStream_t);                                                 \
+                                                cudaStream_t, const int *, int *);                                                 \
     template cudaError_t run_jkq_finalize<R, 4>(long long, int, const void *, const double *, double *, double *, \
-                                                cudaStream_t);                                                 \
+                                                cudaStream_t, const int *, int *);                                                 \
     template cudaError_t run_j1_finalize<R>(long long, int, const void *, const double *, double *, cudaStream_t); \
     template cudaError_t run_see<R>(long long, int, int, double, const double *, const double *, const double *, \
                                     const double *, const double *, double *, void *, unsigned long long *,     \

@@ -13,7 +13,7 @@ template <typename Real>
 cudaError_t run_rho_convert(long long nvox, int nl, const double *rho, void *out, cudaStream_t st);
 template <typename Real, int NS>
 cudaError_t run_jkq_finalize(long long nvox, int nray, const void *part, const double *tw, double *jkq, double *lstar,
-                             cudaStream_t st);
+                             cudaStream_t st, const int *err = nullptr, int *handed = nullptr);
 // J^1_Q [v][3] (J10, Re J11, Im J11) = sum_m tw1[m][c] partv[m][v]: tw1 = w_m T^1_Q(V, Omega_m),
 // partv (Real [ray][nvox]) the per-ray frequency integrals of Stokes V
 template <typename Real>

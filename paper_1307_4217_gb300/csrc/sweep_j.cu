@@ -442,12 +442,23 @@ __device__ __forceinline__ unsigned bar_try(unsigned bar, unsigned parity)
 // Bounded wait for the phase of the given parity. A wait that runs out (the neighbouring
 // CTA stopped) marks the CTA, which from then on waits for and signals nothing (its
 // neighbours' waits run out in turn), and sets the error flag; the kernel then ends with
-// wrong sums and the host reports the flag.
+// wrong sums and the next call that synchronizes reports the flag. The limit is a time, a
+// hundred thousand times a plane's: the tries themselves may sleep. It is read after the
+// waits of ordinary length only (read at once it cost 1 to 2% of every sweep).
+constexpr unsigned long long kHaloWaitNs = 2000000000ull;
+__device__ __forceinline__ unsigned long long global_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
 __device__ __noinline__ void bar_wait_long(unsigned bar, unsigned parity, volatile int *dead, int *err)
 {
-    for (int i = 0; i < (1 << 21); ++i) {
+    for (int i = 0; i < 1024; ++i)
         if (bar_try(bar, parity) || *dead) return;
-    }
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < kHaloWaitNs)
+        if (bar_try(bar, parity) || *dead) return;
     *dead = 1;
     atomicOr(err, 4);
 }
@@ -1201,7 +1212,10 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
         // the ray's constants (mu, ox, oy, oz, T[18], w, pad); the item starts with a barrier
         if (threadIdx.x < 24) sray[threadIdx.x] = reinterpret_cast<const Real *>(a.rays + m)[threadIdx.x];
         for (int g = g0; g < (split > 1 ? g0 + 1 : a.ngroups); ++g) {
-            jsweep_item<Real, NS, MODE, PACKED>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), smem_u32(s_exp), box, m, g, rank, C);
+            // (a CTA whose wait ran out signals nothing any more)
+            if (C == 1 || !*bars.dead)
+                jsweep_item<Real, NS, MODE, PACKED>(a, smem_u32(smem_raw), sm, bars, ph, smem_u32(sray), smem_u32(s_exp), box, m, g,
+                                                    rank, C);
             // every halo row of the item has been written and read before the next one
             // (whose strips may have other neighbours)
             if (C > 1) cluster.sync();
@@ -1209,7 +1223,8 @@ __global__ void __launch_bounds__(jsweep_max_threads<Real, NS>(), 1) jsweep_kern
     }
 }
 
-// Fixed-point scale of each voxel: 2^e with e = 46 - ilogb(max(|S^0_0|, |B|)),
+// Before a formal solution: the error flag (where jerr is set) to 0, and the
+// fixed-point scale of each voxel: 2^e with e = 46 - ilogb(max(|S^0_0|, |B|)),
 // so that a term of the size of the voxel's source function or Planck function
 // carries 46 fraction bits and the accumulator has 2^16 of headroom above it
 // (an FP32 term then converts without rounding; an FP64 term rounds at 2^-47 of
@@ -1224,6 +1239,7 @@ __global__ void jacc_prepare_kernel(const SweepArgs<Real> a, int *jexp, Real *pa
     const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long nvox = a.nvox;
     if (v >= nvox) return;
+    if (v == 0 && a.jerr) *a.jerr = 0;
     using W = JW<Real, NS>;
     if (pack) {
         Real w[W::staged];
@@ -1252,15 +1268,34 @@ __global__ void jacc_prepare_kernel(const SweepArgs<Real> a, int *jexp, Real *pa
 
 template <int NS>
 __global__ void jacc_finalize_kernel(long long nvox, const unsigned long long *jacc, const int *jexp, double *jkq,
-                                     double *lstar)
+                                     double *lstar, const int *err, int *handed)
 {
     const long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const int flag = v == 0 ? *err : 0;
     if (v >= nvox) return;
     const double inv = ldexp(1.0, -jexp[v]);
     constexpr int NJ = NS == 1 ? 1 : 6;
 #pragma unroll
     for (int k = 0; k < NJ; ++k) jkq[v * NJ + k] = (double)(long long)jacc[k * nvox + v] * inv;
     lstar[v] = (double)(long long)jacc[NJ * nvox + v] * inv;
+    if (flag) atomicOr(handed, flag);
+}
+
+// bar_wait_long on an mbarrier at which nothing arrives
+__global__ void halo_wait_kernel(int *err, unsigned long long *ns)
+{
+    __shared__ __align__(8) unsigned long long s_bar;
+    __shared__ int s_dead;
+    s_dead = 0;
+    bar_init(smem_u32(&s_bar));
+    const unsigned long long t0 = global_ns();
+    bar_wait_long(smem_u32(&s_bar), 0, &s_dead, err);
+    *ns = global_ns() - t0;
+}
+cudaError_t run_halo_wait(int *err, unsigned long long *ns, cudaStream_t st)
+{
+    halo_wait_kernel<<<1, 1, 0, st>>>(err, ns);
+    return cudaGetLastError();
 }
 
 template <typename Real, int NS>
@@ -1275,11 +1310,11 @@ cudaError_t launch_jacc_prepare(const SweepArgs<Real> &a, cudaStream_t st)
 
 template <int NS>
 cudaError_t launch_jacc_finalize(long long nvox, const unsigned long long *jacc, const int *jexp, double *jkq,
-                                 double *lstar, cudaStream_t st)
+                                 double *lstar, const int *err, int *handed, cudaStream_t st)
 {
     const int bs = 256;
     const long long nb = (nvox + bs - 1) / bs;
-    jacc_finalize_kernel<NS><<<(unsigned)nb, bs, 0, st>>>(nvox, jacc, jexp, jkq, lstar);
+    jacc_finalize_kernel<NS><<<(unsigned)nb, bs, 0, st>>>(nvox, jacc, jexp, jkq, lstar, err, handed);
     return cudaGetLastError();
 }
 
@@ -1359,8 +1394,8 @@ PORTA_JINST(double, 1)
 PORTA_JINST(double, 4)
 #undef PORTA_JINST
 template cudaError_t launch_jacc_finalize<1>(long long, const unsigned long long *, const int *, double *, double *,
-                                             cudaStream_t);
+                                             const int *, int *, cudaStream_t);
 template cudaError_t launch_jacc_finalize<4>(long long, const unsigned long long *, const int *, double *, double *,
-                                             cudaStream_t);
+                                             const int *, int *, cudaStream_t);
 
 }  // namespace porta
