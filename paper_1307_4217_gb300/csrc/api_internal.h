@@ -285,56 +285,64 @@ int choose_jsweep(porta_ctx *c, LaunchCfg &best, int force_c, int force_f, int n
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    for (int C = 1; C <= std::min(16, ny_max); ++C) {
-        if (force_c > 0 && C != force_c) continue;
-        int nodes, ipts;
-        launch_caps<Real, NS>(c, C, nodes, ipts, true);
-        int last_units = 0;
-        for (int g = 1; g <= NU; ++g) {
-            // (a forced number of frequencies per pass is spread evenly over as many passes, or
-            // over the fewest that fit)
-            if (force_f > 0) g = std::max(g, (NU + force_f - 1) / force_f);
-            const int F = even(g);
-            const int units = (F + jsweep_lanes<Real>() - 1) / jsweep_lanes<Real>();
-            if (units == last_units) continue;
-            last_units = units;
-            int threads = 0;
-            const int tots = jsweep_tots<Real, NS>(c, C, F, &threads);
-            const int smem = jsweep_smem_bytes<Real, NS>(nodes, ipts, tots, F);
-            if (smem > kJSmemLimit) continue;
-            const int G = jsweep_groups<Real>(NU, F);
-            const int parts = sizeof(Real) == 4 || emg ? G : 1;
-            const long long n = (long long)nitems * parts;
-            auto cost = [&](int ncl) {
-                const int share = std::max(1, (ncl * C + nsm - 1) / nsm);     // CTAs on one SM
-                double total = 0.0, item_max = 0.0;
-                for (const BoxDev &b : c->boxes) {
-                    const double item = (double)b.nz * (G / parts) *
-                                        jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads, share, C > 1);
-                    total += item * c->nray * parts;
-                    item_max = std::max(item_max, item);
+    // A forced number of frequencies per pass gives the number of passes, over which they are
+    // spread evenly; only where no cluster size holds them, the fewest passes that fit.
+    const int g0 = force_f > 0 ? (NU + force_f - 1) / force_f : 1;
+    auto search = [&](int g_last) {
+        for (int C = 1; C <= std::min(16, ny_max); ++C) {
+            if (force_c > 0 && C != force_c) continue;
+            int nodes, ipts;
+            launch_caps<Real, NS>(c, C, nodes, ipts, true);
+            int last_units = 0;
+            bool fits = false;
+            for (int g = g0; g <= g_last && !(force_f > 0 && fits); ++g) {
+                const int F = even(g);
+                const int units = (F + jsweep_lanes<Real>() - 1) / jsweep_lanes<Real>();
+                if (units == last_units) continue;
+                last_units = units;
+                int threads = 0;
+                const int tots = jsweep_tots<Real, NS>(c, C, F, &threads);
+                const int smem = jsweep_smem_bytes<Real, NS>(nodes, ipts, tots, F);
+                if (smem > kJSmemLimit) continue;
+                const int G = jsweep_groups<Real>(NU, F);
+                const int parts = sizeof(Real) == 4 || emg ? G : 1;
+                const long long n = (long long)nitems * parts;
+                auto cost = [&](int ncl) {
+                    const int share = std::max(1, (ncl * C + nsm - 1) / nsm);     // CTAs on one SM
+                    double total = 0.0, item_max = 0.0;
+                    for (const BoxDev &b : c->boxes) {
+                        const double item = (double)b.nz * (G / parts) *
+                                            jsweep_plane_cost<Real, NS>(b.nx, (b.ny + C - 1) / C, F, threads, share, C > 1);
+                        total += item * c->nray * parts;
+                        item_max = std::max(item_max, item);
+                    }
+                    return c->nbox == 1 || emg ? (double)((n + ncl - 1) / ncl) * item_max : std::max(total / ncl, item_max) * 1.05;
+                };
+                // no better even with every SM's thread slots taken
+                const int per_sm = std::max(1, std::min(2048 / threads, 227 * 1024 / (smem + 1024)));
+                double bound = 1e300;
+                for (int k = 1; k <= per_sm && bound >= best_cost; ++k) bound = std::min(bound, cost(std::max(1, nsm * k / C)));
+                if (best.cluster > 0 && bound >= best_cost) {
+                    fits = true;
+                    continue;
                 }
-                return c->nbox == 1 || emg ? (double)((n + ncl - 1) / ncl) * item_max : std::max(total / ncl, item_max) * 1.05;
-            };
-            // no better even with every SM's thread slots taken
-            const int per_sm = std::max(1, std::min(2048 / threads, 227 * 1024 / (smem + 1024)));
-            double bound = 1e300;
-            for (int k = 1; k <= per_sm && bound >= best_cost; ++k) bound = std::min(bound, cost(std::max(1, nsm * k / C)));
-            if (best.cluster > 0 && bound >= best_cost) continue;
-            int act = 0;
-            if (jsweep_max_active_clusters<Real, NS>(C, smem, threads, &act) != cudaSuccess) {
-                cudaGetLastError();
-                continue;
+                int act = 0;
+                if (jsweep_max_active_clusters<Real, NS>(C, smem, threads, &act) != cudaSuccess) {
+                    cudaGetLastError();
+                    continue;
+                }
+                if (act < 1) continue;
+                fits = true;
+                const int ncl = (int)std::min<long long>(act, n);
+                if (cost(ncl) < best_cost) {
+                    best_cost = cost(ncl);
+                    best = {C, F, threads, smem, ncl, 0};
+                }
             }
-            if (act < 1) continue;
-            const int ncl = (int)std::min<long long>(act, n);
-            if (cost(ncl) < best_cost) {
-                best_cost = cost(ncl);
-                best = {C, F, threads, smem, ncl, 0};
-            }
-            if (force_f > 0) break;
         }
-    }
+    };
+    search(force_f > 0 ? g0 : NU);
+    if (force_f > 0 && best.cluster == 0) search(NU);
     return best.cluster > 0 ? PORTA_OK : PORTA_EINVAL;
 }
 
