@@ -893,23 +893,19 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
         std::vector<int> tune(c->n_tune);
         for (int i = 0; i < c->n_tune; ++i) tune[i] = items[(size_t)i * items.size() / c->n_tune];
         ok(cudaMemcpy(c->d_tune_items, tune.data(), tune.size() * sizeof(int), cudaMemcpyHostToDevice));
-        auto relative_form = [&](auto &geom) {
+        auto geometry = [&](auto &geom) {       // the general form, then the relative one
             for (int b = 0; b < nbox; ++b)
                 for (int m = 0; m < c->nray; ++m) {
-                    const size_t o = c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz;
-                    relative_geometry(geom.data() + o, c->boxes[b].nz, geom.data() + geom.size() / 2 + o);
+                    auto *g = geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz;
+                    plane_geometry(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
+                                   c->bz[b].data(), c->mu[m], c->chi[m], g, g + geom.size() / 2);
                 }
         };
         if (prec == PORTA_FP32) {
             std::vector<PlaneGeom<float>> geom(2 * (size_t)c->nray * nplane);
             std::vector<RayDev<float>> rays(c->nray);
             std::vector<float> fr(2 * c->n_nu);
-            for (int b = 0; b < nbox; ++b)
-                for (int m = 0; m < c->nray; ++m)
-                    plane_geometry<float>(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
-                                          c->bz[b].data(), c->mu[m], c->chi[m],
-                                          geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz);
-            relative_form(geom);
+            geometry(geom);
             for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<float>(c->mu[m], c->chi[m], c->w[m]);
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = (float)c->xf[j]; fr[c->n_nu + j] = (float)c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));
@@ -919,12 +915,7 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
             std::vector<PlaneGeom<double>> geom(2 * (size_t)c->nray * nplane);
             std::vector<RayDev<double>> rays(c->nray);
             std::vector<double> fr(2 * c->n_nu);
-            for (int b = 0; b < nbox; ++b)
-                for (int m = 0; m < c->nray; ++m)
-                    plane_geometry<double>(c->boxes[b].nx, c->boxes[b].ny, c->boxes[b].nz, c->blx[b], c->bly[b],
-                                           c->bz[b].data(), c->mu[m], c->chi[m],
-                                           geom.data() + c->boxes[b].geom0 + (size_t)m * c->boxes[b].nz);
-            relative_form(geom);
+            geometry(geom);
             for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<double>(c->mu[m], c->chi[m], c->w[m]);
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = c->xf[j]; fr[c->n_nu + j] = c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));

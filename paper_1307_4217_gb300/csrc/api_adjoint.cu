@@ -185,8 +185,7 @@ cudaError_t put_directions(porta_ctx *c, int ndir, const double *mu, const doubl
     RayDev<Real> *r = reinterpret_cast<RayDev<Real> *>(b + 1);
     for (int i = 0; i < ndir; ++i) {
         PlaneGeom<Real> *gi = g + (size_t)i * c->nz;
-        plane_geometry<Real>(c->nx, c->ny, c->nz, c->lx, c->ly, c->z.data(), mu[i], chi[i], gi);
-        relative_geometry(gi, c->nz, gi + n);
+        plane_geometry(c->nx, c->ny, c->nz, c->lx, c->ly, c->z.data(), mu[i], chi[i], gi, gi + n);
         r[i] = ray_dev<Real>(mu[i], chi[i]);
     }
     *b = c->boxes[box];

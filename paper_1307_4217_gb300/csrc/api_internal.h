@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <limits>
 #include <string>
 #include <vector>
 
@@ -131,21 +132,50 @@ inline double neighbour(double x, bool up)
 
 // the same for the J^K_Q sweep, which uses the bilinear weights relative to the first one:
 // in place of (tx, ty, ds, pad2) it reads u = t / (1 - t) along x and y, the first weight
-// (1 - tx) (1 - ty), and ds / 2. A factor 1 - t that rounds to 0 is held at the rounding unit of 1.
-// The first weight is what makes the rounded weights add up to 1, rounded up or down so that
-// the sums' product over a ray's planes stays at 1: planes of equal spacing have equal
-// weights, and a ray through a transparent medium would gather their excess (2e-8 per plane
-// rms, 1e-6 after 64 planes).
+// (1 - tx) (1 - ty), and ds / 2, each from FP64.
+//
+// A point within half a rounding unit of the next node (t = 1: a ray along a grid axis whose
+// other component is 1e-17 and not 0) is taken there, t = 0, with the plane's offset ax or ay
+// one less from here on. (Held at 1 - t = 2^-24 it moved by that much at every plane: 64 planes,
+// the profiles along two axes 37e-7 from their values in Q and U, along the others 3e-7.)
+//
+// What is rounded goes up or down so that the errors do not gather along a ray: planes of
+// equal spacing have equal values, whose errors would add up with one sign. u keeps the sum
+// of the point's displacements near 0, and the first weight, which is what makes the rounded
+// weights add up to 1, keeps the product of their sums at 1 (a ray through a transparent
+// medium would gather their excess, 2e-8 per plane rms, 1e-6 after 64 planes).
 template <typename Real>
-void relative_geometry(const PlaneGeom<Real> *p, int nz, PlaneGeom<Real> *r)
+void relative_geometry(const PlaneGeom<double> *p, int nx, int ny, int nz, PlaneGeom<Real> *r)
 {
-    const double unit = sizeof(Real) == 4 ? 5.9604644775390625e-08 : 1.1102230246251565e-16;
+    const double half = sizeof(Real) == 4 ? 2.98023223876953125e-08 : 5.551115123125783e-17;
     double gathered = 0.0;
+    struct Axis {
+        double moved = 0.0;     // sum of the displacements so far, in cells
+        long long back = 0;     // how much less the offset is than the general form's
+    } x, y;
+    auto ratio = [&](double t, Axis &a) {
+        if (1.0 - t <= half) {
+            a.moved += 1.0 - t;
+            ++a.back;
+            return Real(0);
+        }
+        const double u = t / (1.0 - t);
+        const Real n = (Real)u;
+        if (!(n > std::numeric_limits<Real>::min())) return n;
+        const Real o = neighbour(n, (double)n < u);
+        auto off = [&](Real v) { return ((double)v - u) / ((1.0 + (double)v) * (1.0 + u)); };
+        const double en = a.moved + off(n), eo = a.moved + off(o);
+        const bool swap = std::fabs(eo) < std::fabs(en);
+        a.moved = swap ? eo : en;
+        return swap ? o : n;
+    };
     for (int q = 0; q < nz; ++q) {
-        const double mx = std::max(1.0 - (double)p[q].tx, unit), my = std::max(1.0 - (double)p[q].ty, unit);
-        r[q] = p[q];
-        r[q].tx = (Real)(p[q].tx / mx);
-        r[q].ty = (Real)(p[q].ty / my);
+        r[q] = {};
+        r[q].kz = p[q].kz;
+        r[q].tx = ratio(p[q].tx, x);
+        r[q].ty = ratio(p[q].ty, y);
+        r[q].ax = (int)wrapll(p[q].ax - x.back, nx);
+        r[q].ay = (int)wrapll(p[q].ay - y.back, ny);
         r[q].pad2 = (Real)(0.5 * p[q].ds);
         const Real uxy = r[q].tx * r[q].ty;        // as the sweep forms it
         const double sum = 1.0 + (double)r[q].tx + (double)r[q].ty + (double)uxy;
@@ -157,6 +187,25 @@ void relative_geometry(const PlaneGeom<Real> *p, int nz, PlaneGeom<Real> *r)
         r[q].ds = swap ? other : w;
         if (q > 0) gathered += swap ? e1 : e0;
     }
+}
+
+// both forms of one direction
+template <typename Real>
+void plane_geometry(int nx, int ny, int nz, double lx, double ly, const double *z, double mu, double chi,
+                    PlaneGeom<Real> *g, PlaneGeom<Real> *rel)
+{
+    std::vector<PlaneGeom<double>> d(nz);
+    plane_geometry(nx, ny, nz, lx, ly, z, mu, chi, d.data());
+    for (int q = 0; q < nz; ++q) {
+        g[q] = {};
+        g[q].ax = d[q].ax;
+        g[q].ay = d[q].ay;
+        g[q].kz = d[q].kz;
+        g[q].tx = (Real)d[q].tx;
+        g[q].ty = (Real)d[q].ty;
+        g[q].ds = (Real)d[q].ds;
+    }
+    relative_geometry(d.data(), nx, ny, nz, rel);
 }
 
 template <typename Real>
