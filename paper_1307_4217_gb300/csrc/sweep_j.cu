@@ -369,14 +369,17 @@ __device__ __forceinline__ void copy_async16(unsigned dst, const void *src)
 }
 __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// a / b with the approximate reciprocal's error removed by one residual step (the error of a
-// node's weight is common to all rays: unlike a step's rounding it would not average out)
-__device__ __forceinline__ float quotient(float a, float b)
+// a w / b rounded up or down: to the nearest of the exact value plus `shift` (-1/2 to 1/2) of
+// its last place. The rounding of a node's weight w_m / (chi N) would be the same for all rays
+// of one w_m, N being nearly so, and go into J and Lambda* undiminished (2e-8, which Lambda*
+// near 1 multiplies in the update: 64 x 64 x 48, Lambda-bar* 3.5e-8 from its value in place of
+// 2.5e-8, populations 1.3 times as far); with a shift of its own for every ray it averages out.
+__device__ __forceinline__ float quotient(float a, float w, float b, float shift)
 {
-    const float r = rcp(b), q = a * r;
-    return fmaf(fmaf(-q, b, a), r, q);
+    const float aw = __fmul_rn(a, w), r = rcp(b), q = __fmul_rn(aw, r);
+    const float place = __uint_as_float(__float_as_uint(q) & 0x7f800000u) * 0x1p-23f;
+    return __fadd_rn(q, fmaf(fmaf(-q, b, aw) + fmaf(a, w, -aw), r, shift * place));
 }
-__device__ __forceinline__ double quotient(double a, double b) { return a * rcp(b); }
 
 // keeps the compiler from rebuilding a corner's address from its parts at every use
 __device__ __forceinline__ unsigned opaque(unsigned x)
@@ -628,8 +631,8 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 else lds2(src + h * nodes * 16, d[2 * h], d[2 * h + 1]);
             }
             const X chi_n = xset(d[0]), ns_n = xset(-d[1] * o[0]);
-            // weight of the node's frequency sums, 1 / (chi N) and, for the fixed-point sums,
-            // the ray's weight and the voxel's power of two
+            // weight of the node's frequency sums, 1 / (chi N) and, for the fixed-point sums
+            // (FP32), the ray's weight and the voxel's power of two
             Real t[20];
 #pragma unroll
             for (int i = 0; i < 5; ++i)
@@ -637,11 +640,17 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
             if constexpr (!EMG) {
                 Real wn;
                 lds(sbase + sm.stw + idx * SZ, wn);
-                wn = quotient(wn, d[0]);
-                if (a.jacc) {
+                if constexpr (SZ == 4) {
                     int ex;
                     lds(sbase + sm.ste + idx * 4, ex);
-                    wn *= t[18] * pow2(Real(0), ex);
+                    // (multiples of the golden ratio, modulo 1, fill the interval evenly; formed
+                    // here for every node: kept through the updates it is one register too many)
+                    unsigned ray = m;
+                    asm volatile("" : "+r"(ray));
+                    const float shift = (float)(ray * 2654435769u >> 8) * 0x1p-24f - 0.5f;
+                    wn = quotient(wn, t[18], d[0], shift) * pow2(Real(0), ex);
+                } else {
+                    wn *= rcp(d[0]);
                 }
                 sts(sbase + sm.wgt + (s * nodes + idx) * SZ, wn);
             }
