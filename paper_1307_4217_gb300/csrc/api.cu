@@ -906,7 +906,12 @@ int create_impl(int nbox, const porta_grid *grids, const porta_atom *at, const p
             std::vector<RayDev<float>> rays(c->nray);
             std::vector<float> fr(2 * c->n_nu);
             geometry(geom);
-            for (int m = 0; m < c->nray; ++m) rays[m] = ray_dev<float>(c->mu[m], c->chi[m], c->w[m]);
+            // (what a weight's rounding leaves goes to the next ray, so that they add up to 1)
+            double left = 0.0;
+            for (int m = 0; m < c->nray; ++m) {
+                rays[m] = ray_dev<float>(c->mu[m], c->chi[m], c->w[m] + left);
+                left += c->w[m] - (double)rays[m].w;
+            }
             for (int j = 0; j < c->n_nu; ++j) { fr[j] = (float)c->xf[j]; fr[c->n_nu + j] = (float)c->wf[j]; }
             ok(cudaMemcpy(c->d_geom, geom.data(), geom.size() * sizeof(geom[0]), cudaMemcpyHostToDevice));
             ok(cudaMemcpy(c->d_rays, rays.data(), rays.size() * sizeof(rays[0]), cudaMemcpyHostToDevice));

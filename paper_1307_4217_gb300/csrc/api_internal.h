@@ -151,20 +151,19 @@ void relative_geometry(const PlaneGeom<double> *p, int nx, int ny, int nz, Plane
     double gathered = 0.0;
     struct Axis {
         double moved = 0.0;     // sum of the displacements so far, in cells
-        long long back = 0;     // how much less the offset is than the general form's
+        int back = 0;           // how much less the offset is than the general form's, modulo the cells
     } x, y;
-    auto ratio = [&](double t, Axis &a) {
+    auto ratio = [&](double t, Axis &a, int n_cell) {
         if (1.0 - t <= half) {
             a.moved += 1.0 - t;
-            ++a.back;
+            a.back = a.back + 1 == n_cell ? 0 : a.back + 1;
             return Real(0);
         }
-        const double u = t / (1.0 - t);
+        const double u = t / (1.0 - t), dt = (1.0 - t) * (1.0 - t);      // (dt / du)
         const Real n = (Real)u;
         if (!(n > std::numeric_limits<Real>::min())) return n;
         const Real o = neighbour(n, (double)n < u);
-        auto off = [&](Real v) { return ((double)v - u) / ((1.0 + (double)v) * (1.0 + u)); };
-        const double en = a.moved + off(n), eo = a.moved + off(o);
+        const double en = a.moved + ((double)n - u) * dt, eo = a.moved + ((double)o - u) * dt;
         const bool swap = std::fabs(eo) < std::fabs(en);
         a.moved = swap ? eo : en;
         return swap ? o : n;
@@ -172,10 +171,10 @@ void relative_geometry(const PlaneGeom<double> *p, int nx, int ny, int nz, Plane
     for (int q = 0; q < nz; ++q) {
         r[q] = {};
         r[q].kz = p[q].kz;
-        r[q].tx = ratio(p[q].tx, x);
-        r[q].ty = ratio(p[q].ty, y);
-        r[q].ax = (int)wrapll(p[q].ax - x.back, nx);
-        r[q].ay = (int)wrapll(p[q].ay - y.back, ny);
+        r[q].tx = ratio(p[q].tx, x, nx);
+        r[q].ty = ratio(p[q].ty, y, ny);
+        r[q].ax = p[q].ax - x.back + (p[q].ax < x.back ? nx : 0);
+        r[q].ay = p[q].ay - y.back + (p[q].ay < y.back ? ny : 0);
         r[q].pad2 = (Real)(0.5 * p[q].ds);
         const Real uxy = r[q].tx * r[q].ty;        // as the sweep forms it
         const double sum = 1.0 + (double)r[q].tx + (double)r[q].ty + (double)uxy;

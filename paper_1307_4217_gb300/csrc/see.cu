@@ -37,7 +37,12 @@ __global__ void profile_norm_kernel(long long nvox, int nray, int nnu, const dou
             comp = (t - sum) - y;
             sum = t;
         }
-        invn[idx] = (Real)(1.0f / sum);
+        // 1 / (sum - comp) rounded up or down by the ray's place in a sequence that fills the unit
+        // interval evenly (multiples of the square root of 2): N is nearly the same for all rays,
+        // and a rounding common to them would not average out of J and Lambda*
+        const float q = 1.0f / sum, place = __uint_as_float(__float_as_uint(q) & 0x7f800000u) * 0x1p-23f;
+        const float shift = (float)((unsigned)m * 1779033704u >> 8) * 0x1p-24f - 0.5f;
+        invn[idx] = (Real)__fadd_rn(q, fmaf(q, fmaf(q, comp, fmaf(-q, sum, 1.0f)), shift * place));
     } else {
         double s = vel[v] * mu[m], sum = 0.0;
         for (int j = 0; j < nnu; ++j) {
