@@ -35,3 +35,9 @@ def test_lambda_of_thick_planes(quad):
     _, err, lam = _errors(quad)
     assert np.sum(lam > 0.9) >= 4
     assert np.max(np.abs(err[lam > 0.9])) < 1e-8
+
+
+@pytest.mark.parametrize("quad", QUADS)
+def test_mean_intensity(quad):
+    err, _, _ = _errors(quad)
+    assert np.max(np.abs(err)) < 1e-8
