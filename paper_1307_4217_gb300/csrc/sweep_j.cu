@@ -378,6 +378,14 @@ __device__ __forceinline__ float quotient(float a, float w, float b, float shift
     return __fadd_rn(q, fmaf(fmaf(-q, b, aw) + fmaf(a, w, -aw), r, shift * place));
 }
 
+// the shift of ray m: multiples of the golden ratio, modulo 1, fill the interval evenly (formed
+// anew for every node: kept through the updates it is one register too many)
+__device__ __forceinline__ float ray_shift(unsigned m)
+{
+    asm volatile("" : "+r"(m));
+    return (float)(m * 2654435769u >> 8) * 0x1p-24f - 0.5f;
+}
+
 // keeps the compiler from rebuilding a corner's address from its parts at every use
 __device__ __forceinline__ unsigned opaque(unsigned x)
 {
@@ -640,12 +648,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 if constexpr (SZ == 4) {
                     int ex;
                     lds(sbase + sm.ste + idx * 4, ex);
-                    // (multiples of the golden ratio, modulo 1, fill the interval evenly; formed
-                    // here for every node: kept through the updates it is one register too many)
-                    unsigned ray = m;
-                    asm volatile("" : "+r"(ray));
-                    const float shift = (float)(ray * 2654435769u >> 8) * 0x1p-24f - 0.5f;
-                    wn = quotient(wn, t[18], d[0], shift) * pow2(Real(0), ex);
+                    wn = quotient(wn, t[18], d[0], ray_shift(m)) * pow2(Real(0), ex);
                 } else {
                     wn *= rcp(d[0]);
                 }
@@ -716,12 +719,26 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
 #pragma unroll
                 for (int k = 0; k < W::nacc; ++k, acc += nvox) jadd_small(acc, y[k]);
             } else {
+                // large terms, one after the other; or the weight is beyond FP32, as it is where chi
+                // times the voxel's reference value is below 1e-27 or so: the sums are then as far
+                // below, and 2^64 goes from one to the other
+                if (!(wn < __int_as_float(0x7f800000))) {
+                    Real w[4];
+                    ray4(5, w);
+                    wn = quotient(invn[v], w[2], a.chi[v], ray_shift(m)) * pow2(Real(0), a.jexp[v] - 64);
+#pragma unroll
+                    for (int s = 0; s < NA; ++s) t[s] = sum[s] * Real(0x1p64) * wn;
+                }
                 bool bad = false;
 #pragma unroll 1
                 for (int k = 0; k < W::nacc; ++k, acc += nvox) {
-                    Real x = y[0];
+                    Real x = k + 1 < W::nacc ? t[0] : t[NA - 1];
+                    if (NS == 4 && k < 6) {
+                        Real T[3];
 #pragma unroll
-                    for (int i = 1; i < W::nacc; ++i) x = k == i ? y[i] : x;
+                        for (int i = 0; i < 3; ++i) lds(sray + (4 + 6 * i + k) * SZ, T[i]);
+                        x = T[0] * t[0] + T[1] * t[1] + T[2] * t[2];
+                    }
                     bad |= jadd(acc, x);
                 }
                 if (bad) atomicOr(a.jerr, 1);
