@@ -218,4 +218,44 @@ __device__ __forceinline__ void cluster_wait_acquire()
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
+// 16-byte chunks of a node's source vector and of a Stokes vector (the J^K_Q sweeps)
+template <typename Real>
+__device__ __forceinline__ void chunk_put(typename V16<Real>::T *p, const Real *w)
+{
+    if constexpr (sizeof(Real) == 4) *p = make_float4(w[0], w[1], w[2], w[3]);
+    else *p = make_double2(w[0], w[1]);
+}
+template <typename Real>
+__device__ __forceinline__ void chunk_get(const typename V16<Real>::T *p, Real *w)
+{
+    if constexpr (sizeof(Real) == 4) {
+        const float4 v = *p;
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+    } else {
+        const double2 v = *p;
+        w[0] = v.x; w[1] = v.y;
+    }
+}
+
+// 2^e as an exact FP32 value (e within the normal exponent range)
+__device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
+
+// per-ray partial integrals of a point (the FP64 form: summed over rays in ray
+// order afterwards): store on the first frequency pass, add on later ones
+template <typename Real, int NS>
+__device__ __forceinline__ void store_partial(const SweepArgs<Real> &a, int m, long long v, int g, const Real *acc)
+{
+    if constexpr (NS == 1) {
+        R2<Real> *pp = reinterpret_cast<R2<Real> *>(a.part) + (long long)m * a.nvox + v;
+        R2<Real> o = {acc[0], acc[1]};
+        if (g > 0) { R2<Real> old = *pp; o.x += old.x; o.y += old.y; }
+        *pp = o;
+    } else {
+        R4<Real> *pp = reinterpret_cast<R4<Real> *>(a.part) + (long long)m * a.nvox + v;
+        R4<Real> o = {acc[0], acc[1], acc[2], acc[3]};
+        if (g > 0) { R4<Real> old = *pp; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
+        *pp = o;
+    }
+}
+
 }  // namespace porta

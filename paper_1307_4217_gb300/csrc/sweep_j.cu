@@ -70,29 +70,7 @@ struct JW {
     static constexpr int nacc = NS == 1 ? 2 : 7;               // fixed-point accumulators per voxel
 };
 
-template <typename Real>
-__device__ __forceinline__ void chunk_put(typename V16<Real>::T *p, const Real *w)
-{
-    if constexpr (sizeof(Real) == 4) *p = make_float4(w[0], w[1], w[2], w[3]);
-    else *p = make_double2(w[0], w[1]);
-}
-template <typename Real>
-__device__ __forceinline__ void chunk_get(const typename V16<Real>::T *p, Real *w)
-{
-    if constexpr (sizeof(Real) == 4) {
-        const float4 v = *p;
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    } else {
-        const double2 v = *p;
-        w[0] = v.x; w[1] = v.y;
-    }
-}
-
 constexpr int kJFrac = 46;   // fixed-point fraction bits below a voxel's reference value
-
-// 2^e as an exact floating-point value (e within the type's normal exponent range)
-__device__ __forceinline__ float pow2(float, int e) { return __int_as_float((e + 127) << 23); }
-__device__ __forceinline__ double pow2(double, int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
 // one term of the fixed-point sum: the integer nearest to y (an FP32 value times a power of
 // two) added to *p. Integer additions are exact and commute, so the sums do not depend on
@@ -123,24 +101,6 @@ __device__ __forceinline__ void jadd_small(unsigned long long *p, float y)
     const float h = fmaf(y, 0x1p-23f, M), l = fmaf(M - h, 0x1p23f, y) + M;
     const unsigned long long k = (unsigned long long)__float_as_uint(h) * (1u << 23) - (unsigned long long)B * ((1u << 23) + 1u);
     atomicAdd(p, k + __float_as_uint(l));
-}
-
-// per-ray partial integrals of a point (the FP64 form: summed over rays in ray
-// order afterwards): store on the first frequency pass, add on later ones
-template <typename Real, int NS>
-__device__ __forceinline__ void store_partial(const SweepArgs<Real> &a, int m, long long v, int g, const Real *acc)
-{
-    if constexpr (NS == 1) {
-        R2<Real> *pp = reinterpret_cast<R2<Real> *>(a.part) + (long long)m * a.nvox + v;
-        R2<Real> o = {acc[0], acc[1]};
-        if (g > 0) { R2<Real> old = *pp; o.x += old.x; o.y += old.y; }
-        *pp = o;
-    } else {
-        R4<Real> *pp = reinterpret_cast<R4<Real> *>(a.part) + (long long)m * a.nvox + v;
-        R4<Real> o = {acc[0], acc[1], acc[2], acc[3]};
-        if (g > 0) { R4<Real> old = *pp; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
-        *pp = o;
-    }
 }
 
 // byte offsets of the dynamic shared memory (the ring of source vectors comes first) and
@@ -648,7 +608,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 if constexpr (SZ == 4) {
                     int ex;
                     lds(sbase + sm.ste + idx * 4, ex);
-                    wn = quotient(wn, t[18], d[0], ray_shift(m)) * pow2(Real(0), ex);
+                    wn = quotient(wn, t[18], d[0], ray_shift(m)) * pow2(ex);
                 } else {
                     wn *= rcp(d[0]);
                 }
@@ -725,7 +685,7 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 if (!(wn < __int_as_float(0x7f800000))) {
                     Real w[4];
                     ray4(5, w);
-                    wn = quotient(invn[v], w[2], a.chi[v], ray_shift(m)) * pow2(Real(0), a.jexp[v] - 64);
+                    wn = quotient(invn[v], w[2], a.chi[v], ray_shift(m)) * pow2(a.jexp[v] - 64);
 #pragma unroll
                     for (int s = 0; s < NA; ++s) t[s] = sum[s] * Real(0x1p64) * wn;
                 }

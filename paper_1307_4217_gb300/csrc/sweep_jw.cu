@@ -61,30 +61,6 @@ struct JW {
     static constexpr int nacc = NS == 1 ? 2 : 7;               // fixed-point accumulators per voxel
 };
 
-template <typename Real>
-__device__ __forceinline__ void chunk_put(typename V16<Real>::T *p, const Real *w)
-{
-    if constexpr (sizeof(Real) == 4) *p = make_float4(w[0], w[1], w[2], w[3]);
-    else *p = make_double2(w[0], w[1]);
-}
-template <typename Real>
-__device__ __forceinline__ void chunk_get(const typename V16<Real>::T *p, Real *w)
-{
-    if constexpr (sizeof(Real) == 4) {
-        const float4 v = *p;
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-    } else {
-        const double2 v = *p;
-        w[0] = v.x; w[1] = v.y;
-    }
-}
-
-constexpr int kJFrac = 46;   // fixed-point fraction bits below a voxel's reference value
-
-// 2^e as an exact floating-point value (e within the type's normal exponent range)
-__device__ __forceinline__ float pow2(float, int e) { return __int_as_float((e + 127) << 23); }
-__device__ __forceinline__ double pow2(double, int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
-
 // one term of the fixed-point sum: x * 2^e (exact) rounded to an integer. Integer
 // additions are exact and commute, so the sums do not depend on the order in which
 // rays, frequency passes and concurrent launches add their terms. A term beyond
@@ -105,32 +81,6 @@ __device__ __forceinline__ void jadd(unsigned long long *p, float y, int *err)
     else if (ex > -25) n = (long long)((m + (1u << (-ex - 1))) >> (-ex));
     if (b >> 31) n = -n;
     atomicAdd(p, (unsigned long long)n);
-}
-__device__ __forceinline__ void jadd(unsigned long long *p, double y, int *err)
-{
-    if (!(fabs(y) < 4.611686018427387904e18)) {
-        atomicOr(err, 1);
-        return;
-    }
-    atomicAdd(p, (unsigned long long)__double2ll_rn(y));
-}
-
-// per-ray partial integrals of a point (the FP64 form: summed over rays in ray
-// order afterwards): store on the first frequency pass, add on later ones
-template <typename Real, int NS>
-__device__ __forceinline__ void store_partial(const SweepArgs<Real> &a, int m, long long v, int g, const Real *acc)
-{
-    if constexpr (NS == 1) {
-        R2<Real> *pp = reinterpret_cast<R2<Real> *>(a.part) + (long long)m * a.nvox + v;
-        R2<Real> o = {acc[0], acc[1]};
-        if (g > 0) { R2<Real> old = *pp; o.x += old.x; o.y += old.y; }
-        *pp = o;
-    } else {
-        R4<Real> *pp = reinterpret_cast<R4<Real> *>(a.part) + (long long)m * a.nvox + v;
-        R4<Real> o = {acc[0], acc[1], acc[2], acc[3]};
-        if (g > 0) { R4<Real> old = *pp; o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w; }
-        *pp = o;
-    }
 }
 
 }  // namespace
@@ -323,19 +273,22 @@ __device__ __forceinline__ void jwide_item(const SweepArgs<Real> &a, cg::cluster
     // Lambda* for this pass: J^K_Q += w_m sum_p T^K_Q(p, m) I_p, Lambda-bar* += w_m L
     // (the ray's weight and tensors in the sweep's precision; FP32 terms convert
     // to fixed point without rounding). The L frequency lanes of a point hold the
-    // same totals and share the terms: lane k adds the components c = k mod L.
-    auto add_terms = [&](int v, const Real *tot) {
-        const Real scale = pow2(Real(0), a.jexp[v]);
-        const Real w = sray[22];
-        unsigned long long *acc = a.jacc + v;
-        if constexpr (NS == 1) {
-            if (lane == 0) jadd(acc, w * tot[0] * scale, a.jerr);
-            if (lane == (L > 1 ? 1 : 0)) jadd(acc + nvox, w * tot[1] * scale, a.jerr);
-        } else {
-            const Real pI = w * tot[0] * scale, pQ = w * tot[1] * scale, pU = w * tot[2] * scale;
-            for (int k = lane; k < 6; k += L)
-                jadd(acc + (size_t)k * nvox, sray[4 + k] * pI + sray[10 + k] * pQ + sray[16 + k] * pU, a.jerr);
-            if (lane == 6 % L) jadd(acc + (size_t)6 * nvox, w * tot[3] * scale, a.jerr);
+    // same totals and share the terms: lane k adds the components c = k mod L. (FP32 only:
+    // the FP64 form has no fixed-point sums.)
+    auto add_terms = [&]([[maybe_unused]] int v, [[maybe_unused]] const Real *tot) {
+        if constexpr (sizeof(Real) == 4) {
+            const float scale = pow2(a.jexp[v]);
+            const float w = sray[22];
+            unsigned long long *acc = a.jacc + v;
+            if constexpr (NS == 1) {
+                if (lane == 0) jadd(acc, w * tot[0] * scale, a.jerr);
+                if (lane == (L > 1 ? 1 : 0)) jadd(acc + nvox, w * tot[1] * scale, a.jerr);
+            } else {
+                const Real pI = w * tot[0] * scale, pQ = w * tot[1] * scale, pU = w * tot[2] * scale;
+                for (int k = lane; k < 6; k += L)
+                    jadd(acc + (size_t)k * nvox, sray[4 + k] * pI + sray[10 + k] * pQ + sray[16 + k] * pU, a.jerr);
+                if (lane == 6 % L) jadd(acc + (size_t)6 * nvox, w * tot[3] * scale, a.jerr);
+            }
         }
     };
 
