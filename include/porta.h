@@ -395,6 +395,13 @@ int porta_set_fill(porta_ctx *c, int cluster_size, int nu_group, double fraction
    Synchronous; uses the current device. */
 int porta_eval_coefficients(int precision, int n, const double *t, double *out);
 
+/* Diagnostic: the same and the profile exactly as the J^K_Q sweep and the emergent sweep of the
+   same kernel evaluate them; in FP32 two neighbouring elements are one pair of
+   frequencies. t, x: n optical paths (> 0) and shifts (host);
+   out[6*i + 0..5] = e^-t, 1 - e^-t, omega_M, omega_O, omega_C, exp(-x^2) (host).
+   Synchronous; uses the current device. */
+int porta_eval_unit(int precision, int n, const double *t, const double *x, double *out);
+
 /* Diagnostic: the bounded wait with which the strips of a J^K_Q sweep wait for one
    another, on a row that never arrives. seconds (host) receives how long it
    waited. PORTA_EKERNEL: the wait ran out and set the error flag, as it must.

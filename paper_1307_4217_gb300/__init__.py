@@ -14,7 +14,7 @@ from .binding import (  # noqa: F401
     porta_create, porta_batch_create, porta_destroy, porta_last_error, porta_set_stream, porta_sizes, porta_rays,
     porta_set_atmosphere, porta_set_rho, porta_get_rho, porta_formal_solve, porta_accumulate_jkq,
     porta_see_update, porta_emergent_stokes, porta_probe_ray, porta_launch_info, porta_autotune, porta_eval_coefficients,
-    porta_eval_halo_wait,
+    porta_eval_halo_wait, porta_eval_unit,
     porta_formal_solve_noalloc, porta_run_iterations, porta_iterate_to, PORTA_ENOTCONV, porta_set_device_limit, porta_device_bytes, porta_fma_peak,
     porta_set_freq_range, porta_partial_size, porta_get_partial, porta_set_partial, porta_residual, porta_eval_step, porta_sigmoid_error, porta_mg_set_prolongation, porta_mg_nested,
     porta_set_interpolation, porta_set_sc_faces, porta_set_global_sweep, porta_set_explicit_medium,

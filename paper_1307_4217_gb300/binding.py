@@ -84,6 +84,7 @@ _SIGS = {
     "porta_set_freq_range": (_I, [_P, _I, _I]),
     "porta_residual": (_I, [_P, _P]),
     "porta_eval_halo_wait": (_I, [_P]),
+    "porta_eval_unit": (_I, [_I, _I, _P, _P, _P]),
     "porta_eval_step": (_I, [_I, _I, _P, _P]),
     "porta_sigmoid_error": (_I, [_I, _I, _P, _P, _P, _P]),
     "porta_set_interpolation": (_I, [_P, _I]),
@@ -279,6 +280,13 @@ def porta_eval_coefficients(precision, t):
     t = np.ascontiguousarray(t, dtype=np.float64)
     out = np.zeros((len(t), 6))
     rc = lib().porta_eval_coefficients(precision, len(t), t.ctypes.data, out.ctypes.data)
+    return rc, out
+
+
+def porta_eval_unit(precision, t, x):
+    t, x = np.ascontiguousarray(t, dtype=np.float64), np.ascontiguousarray(x, dtype=np.float64)
+    out = np.zeros((len(t), 6))
+    rc = lib().porta_eval_unit(precision, len(t), t.ctypes.data, x.ctypes.data, out.ctypes.data)
     return rc, out
 
 

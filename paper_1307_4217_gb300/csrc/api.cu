@@ -1254,6 +1254,23 @@ int porta_eval_coefficients(int precision, int n, const double *t, double *out)
     return e == cudaSuccess ? PORTA_OK : PORTA_ECUDA;
 }
 
+int porta_eval_unit(int precision, int n, const double *t, const double *x, double *out)
+{
+    if (n < 1 || !t || !x || !out || (precision != PORTA_FP32 && precision != PORTA_FP64)) return PORTA_EINVAL;
+    for (int i = 0; i < n; ++i)
+        if (!(t[i] > 0) || !std::isfinite(t[i]) || !std::isfinite(x[i])) return PORTA_EINVAL;
+    double *d = nullptr;
+    if (dalloc(&d, 8 * (size_t)n) != cudaSuccess) return PORTA_ENOMEM;
+    cudaError_t e = cudaMemcpy(d, t, sizeof(double) * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d + n, x, sizeof(double) * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = precision == PORTA_FP32 ? run_unit<float>(n, d, d + n, d + 2 * (size_t)n, nullptr)
+                                    : run_unit<double>(n, d, d + n, d + 2 * (size_t)n, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpy(out, d + 2 * (size_t)n, sizeof(double) * 6 * (size_t)n, cudaMemcpyDeviceToHost);
+    pfree(d);
+    return e == cudaSuccess ? PORTA_OK : PORTA_ECUDA;
+}
+
 int porta_eval_halo_wait(double *seconds)
 {
     if (!seconds) return PORTA_EINVAL;

@@ -149,6 +149,8 @@ __host__ __device__ inline int jsweep_threads(int nx, int R, int FX, int tmax)
 template <typename Real, int NS> constexpr int jsweep_max_threads() { return NS == 4 && sizeof(Real) == 8 ? 256 : 512; }
 template <typename Real, int NS>
 int jsweep_smem_bytes(int nodes, int ipts, int tots, int F);
+template <typename Real>
+cudaError_t run_unit(int n, const double *t, const double *x, double *out, cudaStream_t st);   // (diagnostic)
 // (diagnostic: the halo exchange's bounded wait on a row that never arrives)
 cudaError_t run_halo_wait(int *err, unsigned long long *ns, cudaStream_t st);
 template <typename Real, int NS>

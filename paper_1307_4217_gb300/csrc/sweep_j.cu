@@ -177,9 +177,9 @@ __device__ __forceinline__ double xlane(double a, int) { return a; }
 // three w. With q = w_O, h = t (1 - q) / 2 gives e0 = t (1 - h), w_O + w_C = e0 - w_M (or
 // 2 h - q): below t = 1.5 two polynomials (w_M and w_O over t, minimax in relative error:
 // 5e-9 and 3e-9) yield all five, above it closed forms whose cancellation costs a factor of
-// about 3. e0 is within 1.2e-7 of its value and e + e0 = 1 to rounding, so a constant source
-// function is kept; w_M is within 2e-7, w_O + w_C and w_C, which multiply differences of
-// source functions, within 3e-7 and 8e-7. The polynomials are evaluated for both lanes
+// about 3. Measured over t from 1e-7 to 1e3 (porta_eval_unit): e0 within 7.3e-8 of its value
+// and e + e0 = 1 to rounding, so a constant source function is kept; w_O within 1.6e-7, w_M
+// 5.4e-7 (just above 1.5) and w_C, which multiplies differences of source functions, 5.6e-7. The polynomials are evaluated for both lanes
 // always; the closed forms replace them where some lane needs them. (Three polynomials, an
 // exponential per lane and the sums: 26 instructions more per unit, 3% of the sweep's time.)
 template <typename X> struct XCoef { X e, e0, wm, wo, wc; };
@@ -1284,6 +1284,39 @@ cudaError_t run_halo_wait(int *err, unsigned long long *ns, cudaStream_t st)
     halo_wait_kernel<<<1, 1, 0, st>>>(err, ns);
     return cudaGetLastError();
 }
+
+// diagnostic: the coefficients of a unit and the profile as the sweep evaluates them (a thread
+// takes a pair in FP32): out[6 i] = e, e0, w_M, w_O, w_C at t[i], exp(-x[i]^2)
+template <typename Real>
+__global__ void unit_kernel(int n, const double *t, const double *x, double *out)
+{
+    using X = typename XOf<Real>::X;
+    constexpr int XW = jsweep_lanes<Real>();
+    __shared__ double s_exp[64];
+    profile_table<Real>(s_exp);
+    __syncthreads();
+    const int i0 = XW * (blockIdx.x * blockDim.x + threadIdx.x), i1 = min(i0 + XW - 1, n - 1);
+    if (i0 >= n) return;
+    auto put = [](double a, double b) {
+        if constexpr (XW == 2) return make_float2((float)a, (float)b);
+        else return a;
+    };
+    const XCoef<X> c = xcoef(put(t[i0], t[i1]));
+    const X p = xprofile(put(x[i0], x[i1]), smem_u32(s_exp));
+    for (int w = 0; w <= i1 - i0; ++w) {
+        const X v[6] = {c.e, c.e0, c.wm, c.wo, c.wc, p};
+        for (int k = 0; k < 6; ++k) out[6 * (i0 + w) + k] = (double)xlane(v[k], w);
+    }
+}
+template <typename Real>
+cudaError_t run_unit(int n, const double *t, const double *x, double *out, cudaStream_t st)
+{
+    const int nt = (n + jsweep_lanes<Real>() - 1) / jsweep_lanes<Real>();
+    unit_kernel<Real><<<(nt + 127) / 128, 128, 0, st>>>(n, t, x, out);
+    return cudaGetLastError();
+}
+template cudaError_t run_unit<float>(int, const double *, const double *, double *, cudaStream_t);
+template cudaError_t run_unit<double>(int, const double *, const double *, double *, cudaStream_t);
 
 template <typename Real, int NS>
 cudaError_t launch_jacc_prepare(const SweepArgs<Real> &a, cudaStream_t st)
