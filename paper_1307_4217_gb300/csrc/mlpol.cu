@@ -839,7 +839,7 @@ __global__ void __launch_bounds__(kVoxThreads, MP <= 64 ? 5 : 1) mlpol_see_kerne
             }
         }
         __syncthreads();
-        // the K > 0 block by FP32 factors and FP64 refinement; if that fails, Gaussian
+        // the K > 0 block by an FP32 inverse and FP64 refinement; if that fails, Gaussian
         // elimination in FP64 with partial pivoting on [A | b]: for pivot k the lanes
         // take the columns, the warps the rows of the trailing block
         bool ok = ok1 != 0;

@@ -149,15 +149,16 @@ __host__ __device__ inline int jsweep_threads(int nx, int R, int FX, int tmax)
 template <typename Real, int NS> constexpr int jsweep_max_threads() { return NS == 4 && sizeof(Real) == 8 ? 256 : 512; }
 template <typename Real, int NS>
 int jsweep_smem_bytes(int nodes, int ipts, int tots, int F);
-template <typename Real>
-cudaError_t run_unit(int n, const double *t, const double *x, double *out, cudaStream_t st);   // (diagnostic)
-// (diagnostic: the halo exchange's bounded wait on a row that never arrives)
-cudaError_t run_halo_wait(int *err, unsigned long long *ns, cudaStream_t st);
 template <typename Real, int NS>
 cudaError_t jsweep_max_active_clusters(int cluster, int smem, int threads, int *out);
-// (a.out set: the emergent Stokes profiles of the nitems directions of a.rays, a.geom)
+// (a.out set: the emergent Stokes profiles of the nitems directions of a.rays, a.geom; a.pack
+// null: the inputs are copied word by word from where they are, with the same results)
 template <typename Real, int NS>
 cudaError_t launch_jsweep(const SweepArgs<Real> &a, LaunchCfg &cfg, cudaStream_t st);
+// diagnostics: its coefficients and profile; its bounded wait on a halo row that never arrives
+template <typename Real>
+cudaError_t run_unit(int n, const double *t, const double *x, double *out, cudaStream_t st);
+cudaError_t run_halo_wait(int *err, unsigned long long *ns, cudaStream_t st);
 // the same for planes too wide for sweep_j.cu's shared memory (sweep_jw.cu: three ring slots
 // instead of four, one frequency per unit, no staged inputs). Plane strides are padded to 16
 // (mod 32) 4-byte words, so that the two frequency lanes of a point (adjacent threads) read

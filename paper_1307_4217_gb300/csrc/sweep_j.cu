@@ -36,8 +36,13 @@
 // as the threads hold. Against the kernel of sweep_jw.cu, which this one replaces where it
 // fits (one frequency of one point per thread and step, one cluster barrier per plane), ms
 // per formal solution: 64 x 64 x 64 x 160 rays x 21 frequencies 20.1 -> 17.9, 33 x 27 x 41 x
-// 80 x 21 1.91 -> 1.21, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.1, 64 x 64 x 48 x 160 x 31
-// x 2 lines, unpolarized, 46.4 -> 31.8 (with the rate equations).
+// 80 x 21 1.91 -> 1.20, 24 x 24 x 32 x 48 x 11 in FP64 10.6 -> 6.1, 64 x 64 x 48 x 160 x 31
+// x 4 lines, unpolarized, 46.4 -> 31.4 (with the rate equations).
+//
+// FP32 errors against 64 bits, that kernel's and this one's: J^K_Q of 33 x 27 x 41 9.0e-8 and
+// 3.6e-8, Lambda-bar* 4.1e-8 and 2.3e-8; iterates of 64 x 64 x 64 6.2e-6 and 4.5e-6. What kept them
+// above were roundings that are the same for all rays or planes and do not average out (those
+// of the geometry, of the weights and of the reciprocal in kappa^-1; each is explained at its place).
 //
 // Shared memory per CTA (X: 8 bytes, a frequency unit):
 //   ring[4][nodes]        source vectors, Real
@@ -179,9 +184,10 @@ __device__ __forceinline__ double xlane(double a, int) { return a; }
 // 5e-9 and 3e-9) yield all five, above it closed forms whose cancellation costs a factor of
 // about 3. Measured over t from 1e-7 to 1e3 (porta_eval_unit): e0 within 7.3e-8 of its value
 // and e + e0 = 1 to rounding, so a constant source function is kept; w_O within 1.6e-7, w_M
-// 5.4e-7 (just above 1.5) and w_C, which multiplies differences of source functions, 5.6e-7. The polynomials are evaluated for both lanes
-// always; the closed forms replace them where some lane needs them. (Three polynomials, an
-// exponential per lane and the sums: 26 instructions more per unit, 3% of the sweep's time.)
+// within 5.4e-7 (just above 1.5) and w_C, which multiplies differences of source functions,
+// 5.6e-7. The polynomials are evaluated for both lanes always; the closed forms replace them
+// where some lane needs them. (Three polynomials, an exponential per lane and the sums: 26
+// instructions more per unit, 3% of the sweep's time, and the same errors of J.)
 template <typename X> struct XCoef { X e, e0, wm, wo, wc; };
 __device__ __forceinline__ XCoef<double> xcoef(double t)
 {
@@ -987,15 +993,21 @@ __device__ __forceinline__ void jsweep_item(const SweepArgs<Real> &a, const unsi
                 }
                 if constexpr (NS == 4) {
                     // kappa^-1 = 1 + psi'_O K'_O (Eq. 8) couples I and V only; psi' = w + w_C / 2.
-                    // 1 / (1 - a^2) as 1 + a^2 / (1 - a^2): the approximate reciprocal of a number
-                    // near 1 is 2.5e-8 too large on average, which went into every plane's I
+                    // In FP32 1 / (1 - a^2) as 1 + a^2 / (1 - a^2): the approximate reciprocal of a
+                    // number near 1 is 2.5e-8 too large on average, which went into every plane's I
                     // (64 x 64 x 64: J^0_0 of the deep layers 1.8e-8 too large, now 1e-9; the iterates'
                     // error from 64 bits 6.3e-6 -> 4.5e-6)
                     const X nav = xmul(xfs(Real(0.5), co.wc, co.wo), nkO), a2 = xmul(nav, nav);
-                    const X g = xmul(a2, xrcp(xadd(xset(Real(1)), xneg(a2))));
+                    const X idet = xrcp(xadd(xset(Real(1)), xneg(a2)));
                     const X i = xfma(nav, r[3], r[0]), v = xfma(nav, r[0], r[3]);
-                    r[0] = xfma(i, g, i);
-                    r[3] = xfma(v, g, v);
+                    if constexpr (SZ == 4) {
+                        const X g = xmul(a2, idet);
+                        r[0] = xfma(i, g, i);
+                        r[3] = xfma(v, g, v);
+                    } else {
+                        r[0] = xmul(i, idet);
+                        r[3] = xmul(v, idet);
+                    }
                 }
                 if (active) {
                     if constexpr (NS == 1) {

@@ -107,3 +107,13 @@ def test_emergent_profiles(prec):
     finally:
         assert P.porta_set_device_limit(0) == P.PORTA_OK
     assert np.array_equal(out, ref)
+
+
+def test_wide_planes_take_their_own_kernel():
+    """FP32 planes too wide for the four-slot kernel: fixed-point sums, but no packed inputs (nor
+    the per-ray partials of the general sweep)."""
+    atm = polarized_case(200, 60, 4, seed=5)
+    ctx = make_ctx(atm, 1, 2, 4, 3, F32, rho=initial_rho(atm, 1, seed=6))
+    before = P.porta_device_bytes()
+    ctx.formal_solve()
+    assert P.porta_device_bytes() - before == 200 * 60 * 4 * (7 * 8 + 4)
