@@ -76,6 +76,7 @@ void check_global_sweep(porta_ctx *c);
 
 inline long long wrapll(long long a, long long n)
 {
+    if (a >= 0 && a < n) return a;      // (mostly: a division is the longest part of a plane's geometry)
     long long r = a % n;
     return r < 0 ? r + n : r;
 }
